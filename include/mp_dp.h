@@ -401,10 +401,11 @@ typedef struct {
                                   (padding of the last strip and chunk included) and the
                                   per-chunk column maxima */
     uint64_t record_bytes;     /* per-nt records written by the precompute kernel */
-    uint64_t record_read_bytes;  /* records the strips queue into shared memory (every strip
-                                    reads its pair's records; mostly L2 hits after the first) */
-    uint64_t boundary_bytes;   /* boundary rows written between strips (each read once by
-                                  the next strip) */
+    uint64_t record_read_bytes;  /* records the strips read (every strip its pair's; two strips run by
+                                    one warp share one read; mostly L2 hits after the first) */
+    uint64_t boundary_bytes;   /* boundary rows handed from strip to strip, 4 bytes each (8 in the
+                                  int32 kernel); between the strips of one warp in registers,
+                                  otherwise through memory with a 4-byte tag */
 } mp_dp_stats;
 
 /* Launch configuration of the DP.  The paper's DP is a SIMD loop on CPU
@@ -413,9 +414,9 @@ typedef struct {
  * Every configuration computes bit-identical results: only the speed
  * differs. */
 typedef struct {
-    int32_t dp16_variant;      /* 0: int16 DP kernel built for 3 CTAs per SM (<= 80 registers per
-                                  thread); 1: built for 2 CTAs per SM (<= 128 registers) */
-    int32_t dp16_ctas_per_sm;  /* resident 8-warp CTAs per SM in the int16 launch; 0 = all that fit */
+    int32_t dp16_variant;      /* 0: int16 DP kernel built with 8-warp CTAs (<= 128 registers per
+                                  thread); 1: with 6-warp CTAs (<= 168 registers) */
+    int32_t dp16_ctas_per_sm;  /* resident CTAs per SM in the int16 launch; 0 = all that fit */
     int32_t dp32_ctas_per_sm;  /* the same for the int32 kernel */
     int32_t wide_direct;       /* 1: pairs whose score bound reaches the int16 limit skip the int16
                                   pass and run in int32 at once; 0: int16 first, int32 re-run only
@@ -434,7 +435,7 @@ typedef struct {
                                   adds little padding (an even number of 64-residue strips, or 9 or
                                   more) and where the pair's longer critical path in that form stays
                                   within half the batch's longest one in 64-residue strips; 2: every
-                                  such pair, whatever its critical path.  1 and 2 run the 2-CTA
+                                  such pair, whatever its critical path.  1 and 2 run the 6-warp
                                   build whatever dp16_variant says */
 } mp_dp_tuning;
 

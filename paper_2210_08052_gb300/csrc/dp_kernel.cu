@@ -4,9 +4,9 @@
 //
 // Layout of the computation
 // -------------------------
-// One warp owns one (protein, region) pair.  The protein is cut into strips
-// of 64 residues; lane l holds residues 2l ("lo") and 2l+1 ("hi") of the
-// strip.  The warp sweeps anti-diagonals: at step t the lo cell of lane l is
+// The protein is cut into strips of 64 residues, one or two of them to a warp
+// (a pair of two strips or more runs two per warp, see Ops16d).  With one,
+// lane l holds residues 2l ("lo") and 2l+1 ("hi") of the strip.  The warp sweeps anti-diagonals: at step t the lo cell of lane l is
 // genome position ii = t - 2l and the hi cell is ii - 1, so every cell
 // depends only on cells of earlier steps:
 //   - the residue to the left (j-1) comes from lane l-1's hi cell of the
@@ -128,16 +128,8 @@ struct WarpSmem {
     alignas(16) BndT bout[kChunk];
 };
 
-template <typename BndT>
-__device__ __forceinline__ void put_record(WarpSmem<BndT> &sm, int ii, const uint4 &rec)
-{
-    const int half = ii & 1, idx = (ii >> 1) & (kRing / 2 - 1);
-    sm.ring[half][idx] = rec;
-    if (idx < kRingPad / 2) sm.ring[half][idx + kRing / 2] = rec;   // mirror: a body never wraps
-}
-
-template <typename BndT>
-__device__ __forceinline__ uint4 get_record(const WarpSmem<BndT> &sm, int ii)
+template <typename SmemT>
+__device__ __forceinline__ uint4 get_record(const SmemT &sm, int ii)
 {
     return sm.ring[ii & 1][(ii >> 1) & (kRing / 2 - 1)];
 }
@@ -155,12 +147,13 @@ __device__ __forceinline__ void cp_async_wait_all()
 
 // queue the records of positions [lo, lo + kChunk) into the ring
 // (recs[ii + kRecPre] is the record of position ii)
-template <typename BndT>
-__device__ __forceinline__ void fetch_records(WarpSmem<BndT> &sm, const uint4 *recs, int lo, int lane)
+template <typename SmemT>
+__device__ __forceinline__ void fetch_records(SmemT &sm, const uint4 *recs, int lo, int lane)
 {
     for (int ii = lo + lane; ii < lo + kChunk; ii += 32) {
         const int half = ii & 1, idx = (ii >> 1) & (kRing / 2 - 1);
         cp_async16(&sm.ring[half][idx], recs + ii + kRecPre);
+        // mirror: a body never wraps
         if (idx < kRingPad / 2) cp_async16(&sm.ring[half][idx + kRing / 2], recs + ii + kRecPre);
     }
 }
@@ -195,11 +188,76 @@ __device__ __forceinline__ void fetch_records4(WarpSmem4 &sm, const uint4 *recs,
     }
 }
 
+// Shared memory of a warp running two neighbouring strips (Ops16d).  Records
+// come as two 8-byte words, x and y (penalties) and z and w (profile rows), so
+// that the penalties kept for three steps pin no registers of the other word;
+// even and odd positions in separate halves, as in WarpSmem.  prof[0][aa][lane]
+// holds the lower strip's two scores of the lane, each in a low half (the high
+// one 0), prof[1][aa][lane] the upper strip's, each in a high half, so that
+// one addition packs two cells' scores.  in: the boundary values lane 0 takes
+// (H and I apart, each in a low half); the other lanes read `zero`.  out: lane
+// 31's words, whose high halves are the next strip's boundary.
+constexpr int kBodyD = kBody;    // steps of the longest unrolled body (multiple of 3 and 4)
+struct WarpSmemD {
+    uint2 xy[2][kRing / 2 + kBodyD / 2];
+    uint2 zw[2][kRing / 2 + kBodyD / 2];
+    uint2 prof[2][kProfRows * 32];
+    alignas(16) uint32_t in[2][kChunk];       // [H or I][step]
+    alignas(16) uint32_t out[2][kChunk];
+    alignas(16) uint32_t zero[kChunk + kBodyD];     // read as in[0] and, kChunk words further, as in[1]
+    // what the warp needs at its chunks' ends: kept here and not in registers,
+    // of which the steps between take all there are
+    struct Item {
+        const uint4 *recs;
+        uint64_t *rows;
+        uint8_t *lo;
+        uint32_t *cmax;
+        const int32_t *c0;
+        int n, nsteps, schunks;
+        uint32_t tag, limit, publish, anchored;
+    } it;
+};
+
+// 16-byte store to shared memory that leaves the compiler free to move loads of
+// other shared data across it (what is stored here is read after a warp barrier)
+__device__ __forceinline__ void st_shared16(void *smem, uint32_t x, uint32_t y, uint32_t z, uint32_t w)
+{
+    const uint32_t sa = static_cast<uint32_t>(__cvta_generic_to_shared(smem));
+    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(sa), "r"(x), "r"(y), "r"(z), "r"(w));
+}
+
+// 8-byte asynchronous copy global -> shared
+__device__ __forceinline__ void cp_async8(void *smem, const void *gmem)
+{
+    const uint32_t sa = static_cast<uint32_t>(__cvta_generic_to_shared(smem));
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(sa), "l"(gmem) : "memory");
+}
+
+__device__ __forceinline__ void fetch_records_d(WarpSmemD &sm, const uint4 *recs, int lo, int lane)
+{
+    for (int ii = lo + lane; ii < lo + kChunk; ii += 32) {
+        const int half = ii & 1, idx = (ii >> 1) & (kRing / 2 - 1);
+        const uint2 *r = reinterpret_cast<const uint2 *>(recs + ii + kRecPre);
+        cp_async8(&sm.xy[half][idx], r);
+        cp_async8(&sm.zw[half][idx], r + 1);
+        if (idx < kBodyD / 2) {                          // mirror: a body never wraps
+            cp_async8(&sm.xy[half][idx + kRing / 2], r);
+            cp_async8(&sm.zw[half][idx + kRing / 2], r + 1);
+        }
+    }
+}
+
 // ================================================================ int16 ops
-struct Ops16 {
+// FAR: the records are those of a pair whose other warps run two strips
+// (Ops16d); the high halves (the row before) come from the step before.
+template <bool FAR>
+struct Ops16T {
     using Bnd = uint32_t;                  // [H, I] biased 16-bit
     using Smem = WarpSmem<Bnd>;
     static constexpr int W = kStripW, CPL = 2;
+    // words between profile rows, and from the low to the high table's entry
+    // (FAR: the records' row offsets are those of 256-byte rows)
+    static constexpr int kRowWords = FAR ? 64 : 32, kHiWords = FAR ? 32 : kProfRows * 32;
     static constexpr uint32_t Z = 0x80008000u;      // biased 0 in both halves
     static constexpr uint32_t NEGV = 0x40004000u;   // biased -16384
     static constexpr Bnd kBnd0 = 0x40008000u;       // column 0: H = 0, I = -inf
@@ -269,7 +327,7 @@ struct Ops16 {
     // row 0 at step -2 (L1.lo = h_left).  Every other slot is outside (-inf).
     // h_self, h_left: H in row 0 of the lane's lo column and of the column to
     // its left (0 in local mode)
-    static __device__ __forceinline__ void init(State &s, int lane, Bnd w0, uint4 recm1, uint4 recm2,
+    static __device__ __forceinline__ void init(State &s, int lane, Bnd w0, uint4 recm1, uint4 recm2, uint4 recm3,
                                                 uint32_t xm1, int h_self, int h_left)
     {
         const uint32_t hs = pack2(h_self, -16384), hl = pack2(h_left, -16384);   // [H, -inf]
@@ -279,8 +337,10 @@ struct Ops16 {
         s.IL = (lane == 0) ? ((w0 >> 16) | 0x40000000u) : NEGV;
         s.D1 = s.D2 = s.D3 = NEGV;
         s.A1 = s.B1 = s.C1 = NEGV;
-        s.VD1 = recm1.x; s.VD2 = recm2.x;
-        s.VA1 = recm1.y; s.VA2 = recm2.y;
+        s.VD1 = FAR ? prmt<0x5410>(recm1.x, recm2.x) : recm1.x;
+        s.VD2 = FAR ? prmt<0x5410>(recm2.x, recm3.x) : recm2.x;
+        s.VA1 = FAR ? prmt<0x5410>(recm1.y, recm2.y) : recm1.y;
+        s.VA2 = FAR ? prmt<0x5410>(recm2.y, recm3.y) : recm2.y;
         s.X1 = xm1;
         s.TC = 0xffffu; s.bklo = 0; s.bkhi = 0; s.cm = 0;
     }
@@ -291,16 +351,24 @@ struct Ops16 {
     // KEYS: track the best cell's step with keys (needed when no stream is
     // stored); otherwise keep only the chunk's maximum, whose first position
     // is later read back from the stream.
-    template <bool MASKED, bool KEYS>
+    // MASK 2: cells before row 1 get their boundary values (the anchored modes;
+    // in local mode rows above the matrix may hold H = 0 like row 0: every way
+    // down from them but a restart has a penalty and no codon is complete, so
+    // no H changes).  MASK 1 or 2: rows outside the region are kept out of the
+    // maxima.  With a stream that is not needed: past the last row every step
+    // has a penalty or none, so a cell there never passes the pair's best, and
+    // the read-back takes valid rows only.
+    template <int MASK, bool KEYS>
     static __device__ __forceinline__ uint32_t step(State &s, const Consts &c, const uint4 rec,
                                                     const uint32_t *prof_lane, Bnd bin, Bnd &wout,
                                                     int lane, int ii, int n)
     {
-        const uint32_t VD0 = rec.x, VA0 = rec.y;          // negated penalties
+        // negated penalties
+        const uint32_t VD0 = FAR ? prmt<0x5410>(rec.x, s.VD1) : rec.x, VA0 = FAR ? prmt<0x5410>(rec.y, s.VA1) : rec.y;
         const uint32_t X0 = *reinterpret_cast<const uint32_t *>(
             reinterpret_cast<const char *>(prof_lane) + rec.z);
         const uint32_t X0h = *reinterpret_cast<const uint32_t *>(
-            reinterpret_cast<const char *>(prof_lane + kProfRows * 32) + rec.z);
+            reinterpret_cast<const char *>(prof_lane + kHiWords) + rec.z);
         const uint32_t S = X0 + s.X1;                     // lo: s(i, 2l); hi: s(i-1, 2l+1)
         // each term of Eq. 7 that subtracts a penalty is one fused add-max;
         // IL holds I[i][j-1] - e (the sender subtracted the extension)
@@ -321,7 +389,7 @@ struct Ops16 {
         uint32_t H0 = vmax3(vaddmax(s.L3, S, D0), I0, Y); // H[i-3][j-1] + s(i, j), D, I
 
         uint32_t vmask = 0xffffffffu;
-        if (MASKED) {
+        if (MASK == 2) {
             // cells before row 1 are outside the matrix; ii = -1 is row 0
             const uint32_t kill = (ii < 0 ? 0x0000ffffu : 0u) | (ii < 1 ? 0xffff0000u : 0u);
             const uint32_t row0 = (ii == -1 ? 0x0000ffffu : 0u) | (ii == 0 ? 0xffff0000u : 0u);
@@ -332,8 +400,8 @@ struct Ops16 {
             A0 = (A0 & ~kill) | (NEGV & kill);
             B0 = (B0 & ~kill) | (NEGV & kill);
             C0 = (C0 & ~kill) | (NEGV & kill);
-            vmask = ((ii >= 0 && ii < n) ? 0x0000ffffu : 0u) | ((ii >= 1 && ii <= n) ? 0xffff0000u : 0u);
         }
+        if (MASK) vmask = ((ii >= 0 && ii < n) ? 0x0000ffffu : 0u) | ((ii >= 1 && ii <= n) ? 0xffff0000u : 0u);
 
         // hand [H, I - e] of the hi cell to the next lane (the receiving
         // column's extension, subtracted here, off the step's chain); lane 0
@@ -394,18 +462,9 @@ struct Ops16 {
     {
         return static_cast<int>(h ? (w >> 16) : (w & 0xffffu)) - 32768;
     }
-    static __device__ __forceinline__ Word load_word(const uint8_t *strip, int t, int lane)
-    {
-        return *reinterpret_cast<const uint32_t *>(strip + static_cast<size_t>(t >> 2) * 512 + lane * 16 +
-                                                   (t & 3) * 4);
-    }
     static __device__ __forceinline__ int cell_max(const ColMax &m, int k) { return word_h(m, k); }
-    // stored H of cell k of the lane at step t
-    static __device__ __forceinline__ int load_cell(const uint8_t *strip, int t, int lane, int k)
-    {
-        return word_h(load_word(strip, t, lane), k);
-    }
 };
+using Ops16 = Ops16T<false>;
 
 // ================================================================ int32 ops
 struct V2 {
@@ -428,6 +487,7 @@ struct Ops32 {
     };
     using Smem = WarpSmem<Bnd>;
     static constexpr int W = kStripW, CPL = 2;
+    static constexpr int kRowWords = 32, kHiWords = kProfRows * 32;       // as Ops16T
     static constexpr int32_t NEG = -(1 << 28);
     static constexpr Bnd kBnd0 = {0, NEG};
 
@@ -465,7 +525,7 @@ struct Ops32 {
         return (static_cast<uint32_t>(slo) & 0xffffu) | (static_cast<uint32_t>(shi) << 16);
     }
 
-    static __device__ __forceinline__ void init(State &s, int lane, Bnd w0, uint4 recm1, uint4 recm2,
+    static __device__ __forceinline__ void init(State &s, int lane, Bnd w0, uint4 recm1, uint4 recm2, uint4,
                                                 uint32_t xm1, int h_self, int h_left)
     {
         // the same history as the int16 state (see Ops16::init)
@@ -485,7 +545,7 @@ struct Ops32 {
 
     using Word = uint2;                     // [H lo, H hi] as int32
 
-    template <bool MASKED, bool KEYS>
+    template <int MASK, bool KEYS>
     static __device__ __forceinline__ uint2 step(State &s, const Consts &c, const uint4 rec,
                                                  const uint32_t *prof_lane, Bnd bin, Bnd &wout,
                                                  int lane, int ii, int n)
@@ -512,7 +572,7 @@ struct Ops32 {
         V2 H0 = mx(mx(mx(M, I0), mx(D0, FG)), mx(mx(Ap, Bp), mx(Cp, V2{c.floor, c.floor})));
 
         bool vlo = true, vhi = true;
-        if (MASKED) {
+        if (MASK) {
             if (ii < 0) { H0.lo = (ii == -1) ? c.row0lo : NEG; I0.lo = D0.lo = A0.lo = B0.lo = C0.lo = NEG; }
             if (ii < 1) { H0.hi = (ii == 0) ? c.row0hi : NEG; I0.hi = D0.hi = A0.hi = B0.hi = C0.hi = NEG; }
             vlo = ii >= 0 && ii < n;
@@ -560,8 +620,6 @@ struct Ops32 {
     static __device__ __forceinline__ void reset_best(State &s) { s.cmlo = s.cmhi = NEG; }
 
     static constexpr bool kChunkMaxBest = false;
-    static __device__ __forceinline__ int word_h(const Word &w, int h) { return static_cast<int>(h ? w.y : w.x); }
-    static __device__ __forceinline__ Word load_word(const uint8_t *, int, int) { return make_uint2(0, 0); }
     using ColMax = uint2;
     static __device__ __forceinline__ ColMax chunk_max(const State &s)
     {
@@ -767,10 +825,10 @@ struct Ops16x4 {
 
     template <bool MASKED, bool STORE>
     static __device__ __forceinline__ void chunk(State &st, const Consts &c, Smem &sm, int lane, int t0, int n,
-                                                 uint8_t *code_strip)
+                                                 int bodies, uint8_t *code_strip)
     {
 #pragma unroll 1
-        for (int bdy = 0; bdy < kChunk / kBody; ++bdy) {
+        for (int bdy = 0; bdy < bodies; ++bdy) {
             const int tb = t0 + bdy * kBody;
             // record of a's lo cell at step tb+k: position tb+k-4l, quarter k&3,
             // index ridx + k/4 within it (tb is a multiple of 4)
@@ -818,12 +876,293 @@ struct Ops16x4 {
         const uint32_t w = k < 2 ? m.x : m.y;
         return static_cast<int>((k & 1) ? (w >> 16) : (w & 0xffffu)) - 32768;
     }
-    // stored H of cell k of the lane at step t
-    static __device__ __forceinline__ int load_cell(const uint8_t *strip, int t, int lane, int k)
+    // first of the kChunk steps from tb on at which cell k of the lane holds
+    // value v in a valid row; -1 if none
+    static __device__ __forceinline__ int find_cell(const uint8_t *strip, int tb, int lane, int k, int v, int n)
     {
-        const uint32_t w = *reinterpret_cast<const uint32_t *>(strip + static_cast<size_t>(t >> 1) * 512 + lane * 16 +
-                                                               (t & 1) * 8 + (k >> 1) * 4);
-        return static_cast<int>((k & 1) ? (w >> 16) : (w & 0xffffu)) - 32768;
+        const int lo = CPL * lane + k;
+        for (int t = max(tb, lo); t < min(tb + kChunk, lo + n); ++t) {
+            const uint32_t w = *reinterpret_cast<const uint32_t *>(strip + static_cast<size_t>(t >> 1) * 512 +
+                                                                   lane * 16 + (t & 1) * 8 + (k >> 1) * 4);
+            if (static_cast<int>((k & 1) ? (w >> 16) : (w & 0xffffu)) - 32768 == v) return t;
+        }
+        return -1;
+    }
+};
+
+// ================================================ int16, two strips per warp
+// A warp runs two neighbouring 64-residue strips of a pair at once, the lower
+// one in the low and the upper one in the high half of every register: lane l
+// holds residues 2l (register a) and 2l+1 (register b) of both.  At step t
+// a's cells are at rows t-2l (low) and t-2l-64 (high), b's one row behind.
+// b's left neighbour is the lane's own a of the step before, a's is lane
+// l-1's b (one shuffle each of H and of I, no byte permute: the halves stay
+// where they are); lane 0 takes the pair's boundary in its low half and lane
+// 31's low half in its high half by one multiply-add.  b's records are a's of
+// the step before, so a step loads one record and two profile words for four
+// cells.
+//
+// What bounds it: instruction issue and the operands behind it.  Every max,
+// fused add-max, byte permute and select takes the ALU pipe of a scheduler for
+// two clocks, and most read three registers.  One strip per warp (Ops16T)
+// takes 32.1 instructions (19.3 of them on the ALU) and 9.4 shared-memory rows
+// per 64 cells, here the same cells take 26.5, 14.7 and 8: 51.6 clocks of a
+// scheduler against 44.  A warp alone takes 104 clocks per step of 128 cells
+// (87 for 64).  Every form tried ran at 0.6 instructions per clock when
+// several warps shared a scheduler, so what counted was instructions: two
+// maxima of a pair of steps in one, frameshift maxima shared by a and b, no
+// permute in the hand-over, profile halves added instead of permuted, and
+// registers enough for no spill (a reload in the loop cost more than the
+// warps it made room for: 16 warps per SM at 128 registers 12.6 ms on the
+// 4,096-pair workload, 12 at 168 registers 10.55; start of this form, one
+// strip per warp, 12.8).  Bodies of 24 unrolled steps instead of 12 gain 3%
+// while all warps run in step and lose 10% when they do not (instruction
+// fetch).
+struct Ops16d {
+    static constexpr uint32_t Z = Ops16::Z, NEGV = Ops16::NEGV;
+    static constexpr int kUp = kStripW;                   // rows the upper strip runs behind
+
+    struct Consts {
+        uint32_t NQEa, NQEb;                // -(q+e) of a's and b's two columns (negated per half)
+        uint32_t Ea, Eb, EN;                // e of a's and b's columns and of the columns right of b's
+        uint32_t NF, FLOOR;
+        uint32_t ROW0A, ROW0B;              // H in row 0 (biased)
+        uint32_t mult;                      // lane 0: 65536 (its low half comes from the boundary); else 1.
+                                            // Opaque, so that the product stays a multiply-add off the ALU
+    };
+    struct State {
+        uint32_t aH1, aH2, aH3, aH4, L0, L1, L2, L3, IL, aD1, aD2, aD3, aA, aB, aC;
+        uint32_t bH1, bH2, bH3, bIL, bD1, bD2, bD3, bA, bB, bC;
+        uint32_t VD1, VD2, VD3, VA1, VA2, VA3;            // records of a's row minus 1 .. 3
+        uint32_t Sb;                                      // b's substitution scores of the next step
+        uint32_t P1;                                      // the larger of a's last two H, a step ago
+        uint32_t cma, cmb;                                // this chunk's maxima (pairs with a stream)
+        uint32_t TC, k0, k1, k2, k3;                      // best-cell keys (pairs without one)
+    };
+
+    static __device__ __forceinline__ uint2 prof_at(const uint2 *prof_lane, uint32_t off)
+    {
+        return *reinterpret_cast<const uint2 *>(reinterpret_cast<const char *>(prof_lane) + off);
+    }
+
+    // State before step 0 (see Ops16::init): only lane 0's low half of a
+    // touches row 0 and the strip's left boundary there.
+    static __device__ __forceinline__ void init(State &s, const WarpSmemD &sm, int lane, uint32_t w0, int h_self,
+                                                int h_left)
+    {
+        const bool l0 = lane == 0;
+        s.aH1 = l0 ? Ops16::pack2(h_self, -16384) : NEGV;
+        s.aH2 = s.aH3 = s.aH4 = NEGV;
+        s.L1 = l0 ? Ops16::pack2(h_left, -16384) : NEGV;
+        s.L2 = s.L3 = NEGV;
+        s.L0 = l0 ? ((w0 & 0xffffu) | 0x40000000u) : NEGV;
+        s.IL = l0 ? ((w0 >> 16) | 0x40000000u) : NEGV;
+        s.aD1 = s.aD2 = s.aD3 = s.aA = s.aB = s.aC = NEGV;
+        s.bH1 = s.bH2 = s.bH3 = s.bIL = s.bD1 = s.bD2 = s.bD3 = s.bA = s.bB = s.bC = NEGV;
+        const int ii0 = -2 * lane;
+        auto at = [](int ii) { return (ii >> 1) & (kRing / 2 - 1); };
+        const uint2 r1 = sm.xy[1][at(ii0 - 1)], r2 = sm.xy[0][at(ii0 - 2)], r3 = sm.xy[1][at(ii0 - 3)];
+        s.VD1 = r1.x; s.VD2 = r2.x; s.VD3 = r3.x;
+        s.VA1 = r1.y; s.VA2 = r2.y; s.VA3 = r3.y;
+        const uint2 z1 = sm.zw[1][at(ii0 - 1)];
+        s.Sb = prof_at(&sm.prof[0][lane], z1.x).y + prof_at(&sm.prof[1][lane], z1.y).y;
+        s.P1 = NEGV;
+        s.cma = s.cmb = 0;
+        s.TC = 0xffffu;
+        s.k0 = s.k1 = s.k2 = s.k3 = 0;
+    }
+
+    // Eq. 7 for one register's two cells, as in Ops16::step: row i and column
+    // j of a cell, H1 and H3 its own column's rows i-1 and i-3, L1 and L3 the
+    // left column's, FS the largest H of the four frameshift terms, L0 and IL
+    // the left column's H and I - e in row i; VD0..VD2 and
+    // VA0..VA2 the records x and y (negated penalties) of rows i, i-1, i-2.
+    static __device__ __forceinline__ void cells(uint32_t H1, uint32_t H3, uint32_t FS, uint32_t L0, uint32_t L1,
+                                                 uint32_t L3, uint32_t IL, uint32_t D3, uint32_t S,
+                                                 uint32_t NQE, uint32_t E, uint32_t NF, uint32_t FLOOR, uint32_t VD0,
+                                                 uint32_t VD1, uint32_t VD2, uint32_t VA0, uint32_t VA1, uint32_t VA2,
+                                                 uint32_t &A, uint32_t &B, uint32_t &C, uint32_t &D0, uint32_t &I0,
+                                                 uint32_t &H0)
+    {
+        I0 = vaddmax(L0, NQE, IL);
+        D0 = vaddmax(H3, NQE, D3 - E);
+        A = vaddmax(H1, VD2, A);                          // H[i-1][j] - r - d(i-1)
+        B = vaddmax(L1, VD1, B);                          // H[i-1][j-1] - r - d(i)
+        C = vaddmax(L1, VD0, C);                          // H[i-1][j-1] - r - d(i+1)
+        // three branches joined by one maximum, so that the previous step's H
+        // passes through three operations
+        uint32_t Y = vaddmax(C, VA1, FLOOR);              // C - a(i-1)
+        Y = vaddmax(B, VA2, Y);                           // B - a(i-2)
+        Y = vaddmax(A, VA0, Y);                           // A - a(i)
+        uint32_t M = vaddmax(L3, S, D0);                  // H[i-3][j-1] + s(i, j), D
+        M = vaddmax(FS, NF, M);
+        H0 = vmax3(M, I0, Y);
+    }
+    // valid rows of a register's two cells
+    static __device__ __forceinline__ uint32_t rows(int ii, int n)
+    {
+        const int up = ii - kUp;
+        return ((ii >= 0 && ii < n) ? 0x0000ffffu : 0u) | ((up >= 0 && up < n) ? 0xffff0000u : 0u);
+    }
+    // cells before row 1 are outside the matrix; row -1 (0-based) is row 0
+    static __device__ __forceinline__ void mask(int ii, uint32_t ROW0, uint32_t &H, uint32_t &I, uint32_t &D,
+                                                uint32_t &A, uint32_t &B, uint32_t &C)
+    {
+        const int up = ii - kUp;
+        const uint32_t kill = (ii < 0 ? 0x0000ffffu : 0u) | (up < 0 ? 0xffff0000u : 0u);
+        const uint32_t row0 = (ii == -1 ? 0x0000ffffu : 0u) | (up == -1 ? 0xffff0000u : 0u);
+        H = (H & ~kill) | (((row0 & ROW0) | (~row0 & NEGV)) & kill);
+        I = (I & ~kill) | (NEGV & kill);
+        D = (D & ~kill) | (NEGV & kill);
+        A = (A & ~kill) | (NEGV & kill);
+        B = (B & ~kill) | (NEGV & kill);
+        C = (C & ~kill) | (NEGV & kill);
+    }
+
+    // One step.  rec, zw: the record of a's low row ii.  Ha, Hb: the lane's H
+    // values; Ib: b's I less the extension of the columns right of it.
+    // MASK 2: cells before row 1 get their boundary values; 1 and 2: without a
+    // stream, rows outside the region are kept out of the maxima (see
+    // Ops16T::step for why no more is needed).  SECOND: the second step of a
+    // pair, which takes both steps' cells into the chunk maximum.
+    template <int MASK, bool KEYS, bool SECOND>
+    static __device__ __forceinline__ void step(State &s, const Consts &c, const uint2 rec, const uint2 zw,
+                                                const uint2 *prof_lane, uint32_t inH, uint32_t inI, int lane, int ii, int n, uint32_t &Ha,
+                                                uint32_t &Hb, uint32_t &Ib)
+    {
+        const uint2 Xl = prof_at(prof_lane, zw.x), Xh = prof_at(prof_lane + kProfRows * 32, zw.y);
+        const uint32_t Sa = Xl.x + Xh.x;
+        uint32_t Da, Db, Ia, Ib0;
+        // frameshift terms H[i-1][j-1], H[i-2][j-1], H[i-1][j], H[i-2][j]: a's own
+        // two are b's left two of the next step
+        const uint32_t P = vmax(s.aH1, s.aH2), Fa = vmax3(s.L1, s.L2, P), Fb = vmax3(s.P1, s.bH2, s.bH1);
+        s.P1 = P;
+        cells(s.bH1, s.bH3, Fb, s.aH1, s.aH2, s.aH4, s.bIL, s.bD3, s.Sb, c.NQEb, c.Eb, c.NF, c.FLOOR, s.VD1,
+              s.VD2, s.VD3, s.VA1, s.VA2, s.VA3, s.bA, s.bB, s.bC, Db, Ib0, Hb);
+        cells(s.aH1, s.aH3, Fa, s.L0, s.L1, s.L3, s.IL, s.aD3, Sa, c.NQEa, c.Ea, c.NF, c.FLOOR, rec.x, s.VD1,
+              s.VD2, rec.y, s.VA1, s.VA2, s.aA, s.aB, s.aC, Da, Ia, Ha);
+        if (MASK == 2) {
+            mask(ii, c.ROW0A, Ha, Ia, Da, s.aA, s.aB, s.aC);
+            mask(ii - 1, c.ROW0B, Hb, Ib0, Db, s.bA, s.bB, s.bC);
+        }
+        Ib = Ib0 - c.EN;
+        const int left = (lane + 31) & 31;
+        const uint32_t RH = __shfl_sync(kFull, Hb, left), RI = __shfl_sync(kFull, Ib, left);
+        s.L3 = s.L2; s.L2 = s.L1; s.L1 = s.L0;
+        s.L0 = RH * c.mult + inH;                         // lane 0: [boundary, lane 31's low half]
+        s.IL = RI * c.mult + inI;
+        s.bIL = Ia - c.Eb;
+        if (!KEYS && SECOND) {
+            s.cma = vmax3(s.cma, s.aH1, Ha);
+            s.cmb = vmax3(s.cmb, s.bH1, Hb);
+        }
+        s.aH4 = s.aH3; s.aH3 = s.aH2; s.aH2 = s.aH1; s.aH1 = Ha;
+        s.bH3 = s.bH2; s.bH2 = s.bH1; s.bH1 = Hb;
+        s.aD3 = s.aD2; s.aD2 = s.aD1; s.aD1 = Da;
+        s.bD3 = s.bD2; s.bD2 = s.bD1; s.bD1 = Db;
+        s.VD3 = s.VD2; s.VD2 = s.VD1; s.VD1 = rec.x;
+        s.VA3 = s.VA2; s.VA2 = s.VA1; s.VA1 = rec.y;
+        s.Sb = Xl.y + Xh.y;
+        if (KEYS) {
+            const uint32_t ha = MASK ? Ha & rows(ii, n) : Ha, hb = MASK ? Hb & rows(ii - 1, n) : Hb;
+            s.k0 = max(s.k0, ha * 65536u + s.TC);
+            s.k1 = max(s.k1, hb * 65536u + s.TC);
+            s.k2 = max(s.k2, (ha & 0xffff0000u) | s.TC);
+            s.k3 = max(s.k3, (hb & 0xffff0000u) | s.TC);
+            s.TC -= 1;
+        }
+    }
+
+    // Where a chunk's bodies read and write; a body leaves it at the next one.
+    struct Cursor {
+        const uint32_t *ih;                 // boundary values (lane 0) or zeros
+        uint32_t *oh;                       // lane 31's words
+        uint8_t *pl, *pu;                   // this lane's words of the two strips' streams
+        int ridx, t;                        // record index (see body) and step
+    };
+
+    // N steps.  ulimit: steps of each strip's stream.
+    template <int MASK, bool STORE, int N>
+    static __device__ __forceinline__ void body(State &st, const Consts &c, WarpSmemD &sm, Cursor &q, int lane, int n,
+                                                int ulimit)
+    {
+        // record of a's low cell at step t+k: position t+k-2l, parity k&1,
+        // index (t+k)/2 - l within its half (t is even)
+        const int r = q.ridx & (kRing / 2 - 1);
+        const uint2 *xy0 = &sm.xy[0][r], *zw0 = &sm.zw[0][r];
+        constexpr int kHalf = kRing / 2 + kBodyD / 2;
+        uint32_t wl[4], wu[4], hb4[4], ib4[4];
+        uint4 h4, i4;
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+            if ((k & 3) == 0) {
+                h4 = *reinterpret_cast<const uint4 *>(q.ih + k);
+                i4 = *reinterpret_cast<const uint4 *>(q.ih + kChunk + k);
+            }
+            const uint32_t inH = (k & 3) == 0 ? h4.x : (k & 3) == 1 ? h4.y : (k & 3) == 2 ? h4.z : h4.w;
+            const uint32_t inI = (k & 3) == 0 ? i4.x : (k & 3) == 1 ? i4.y : (k & 3) == 2 ? i4.z : i4.w;
+            uint32_t Ha, Hb;
+            const uint2 xy = xy0[(k & 1) * kHalf + (k >> 1)], zw = zw0[(k & 1) * kHalf + (k >> 1)];
+            if (k & 1)
+                step<MASK, !STORE, true>(st, c, xy, zw, &sm.prof[0][lane], inH, inI, lane, q.t + k - 2 * lane, n, Ha, Hb,
+                                         ib4[k & 3]);
+            else
+                step<MASK, !STORE, false>(st, c, xy, zw, &sm.prof[0][lane], inH, inI, lane, q.t + k - 2 * lane, n, Ha,
+                                          Hb, ib4[k & 3]);
+            if (STORE) {
+                // each strip's stream as Ops16 writes it: [H of 2l, H of 2l+1]
+                wl[k & 3] = prmt<0x5410>(Ha, Hb);
+                wu[k & 3] = prmt<0x7632>(Ha, Hb);
+            } else {
+                hb4[k & 3] = Hb;
+            }
+            if ((k & 3) == 3) {
+                const uint4 l4 = make_uint4(wl[0], wl[1], wl[2], wl[3]), u4 = make_uint4(wu[0], wu[1], wu[2], wu[3]);
+                if (lane == 31) {
+                    if (STORE) st_shared16(q.oh + k - 3, wu[0], wu[1], wu[2], wu[3]);
+                    else st_shared16(q.oh + k - 3, hb4[0], hb4[1], hb4[2], hb4[3]);
+                    st_shared16(q.oh + kChunk + k - 3, ib4[0], ib4[1], ib4[2], ib4[3]);
+                }
+                if (STORE) {
+                    const int u = q.t + k - 3;
+                    if (!MASK || u < ulimit) *reinterpret_cast<uint4 *>(q.pl + (k - 3) * kStepBytes) = l4;
+                    if (!MASK || static_cast<unsigned>(u - kUp) < static_cast<unsigned>(ulimit))
+                        *reinterpret_cast<uint4 *>(q.pu + (k - 3) * kStepBytes) = u4;
+                }
+            }
+        }
+        if (lane == 0) q.ih += N;
+        q.oh += N;
+        q.ridx += N / 2;
+        q.pl += N * kStepBytes;
+        q.pu += N * kStepBytes;
+        q.t += N;
+    }
+
+    // `steps` steps (a multiple of kBody) from step t0 on.  lo: the lower
+    // strip's stream, the upper's strip_bytes behind; ulimit steps each.
+    // anchored: the first rows need their boundary values.
+    template <bool STORE>
+    static __device__ __forceinline__ void chunk(State &st, const Consts &c, WarpSmemD &sm, int lane, int t0, int n,
+                                                 bool anchored, int steps, uint8_t *lo, size_t strip_bytes, int ulimit)
+    {
+        // from these steps on every row is past the first, and the upper strip's
+        // stream has begun
+        constexpr int kFirst = 2 * kStripW, kUpFirst = kUp;
+        uint8_t *pl = lo + static_cast<size_t>(t0) * kStepBytes + lane * 16;
+        Cursor q{lane == 0 ? sm.in[0] : sm.zero, sm.out[0], pl, pl + (static_cast<ptrdiff_t>(strip_bytes) - kUp * kStepBytes), (t0 >> 1) - lane, t0};
+        const int t1 = t0 + steps;
+        if (anchored) {
+#pragma unroll 1
+            while (q.t < t1 && q.t < kFirst) body<2, STORE, kBody>(st, c, sm, q, lane, n, ulimit);
+        } else {
+#pragma unroll 1
+            while (q.t < t1 && q.t < kUpFirst) body<1, STORE, kBody>(st, c, sm, q, lane, n, ulimit);
+        }
+#pragma unroll 1
+        for (const int te = min(t1, n) - kBodyD; q.t <= te;) body<0, STORE, kBodyD>(st, c, sm, q, lane, n, ulimit);
+#pragma unroll 1
+        while (q.t < t1) body<1, STORE, kBody>(st, c, sm, q, lane, n, ulimit);
     }
 };
 
@@ -855,13 +1194,13 @@ __device__ __forceinline__ bool better(int s, int i, int j, const Best &b)
     return s > b.score || (s == b.score && (i < b.ii || (i == b.ii && j < b.jj)));
 }
 
-template <typename Ops, bool MASKED, bool STORE>
+template <typename Ops, int MASK, bool STORE>
 __device__ __forceinline__ void run_chunk(typename Ops::State &st, const typename Ops::Consts &c,
-                                          WarpSmem<typename Ops::Bnd> &sm, int lane, int t0, int n,
+                                          WarpSmem<typename Ops::Bnd> &sm, int lane, int t0, int n, int bodies,
                                           uint8_t *code_strip)
 {
 #pragma unroll 1
-    for (int b = 0; b < kChunk / kBody; ++b) {
+    for (int b = 0; b < bodies; ++b) {
         const int tb = t0 + b * kBody;
         // record of the lo cell at step tb+k: position tb+k-2l, parity k&1,
         // index (tb+k)/2 - l within its half (tb is even)
@@ -878,7 +1217,7 @@ __device__ __forceinline__ void run_chunk(typename Ops::State &st, const typenam
 #pragma unroll
                 for (int u = 0; u < 4; ++u) bin4[u] = sm.bin[b * kBody + k + u];
             }
-            cw[k] = Ops::template step<MASKED, !STORE>(st, c, (k & 1) ? ro[k >> 1] : re[k >> 1], sm.prof + lane,
+            cw[k] = Ops::template step<MASK, !STORE>(st, c, (k & 1) ? ro[k >> 1] : re[k >> 1], sm.prof + lane,
                                                          bin4[k & 3], wout4[k & 3], lane, tb + k - 2 * lane, n);
             if ((k & 3) == 3) {
                 if (lane == 31) {
@@ -903,15 +1242,102 @@ __device__ __forceinline__ void st_release(uint32_t *p, uint32_t v)
     asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-template <typename T>
-__device__ __forceinline__ T ld_l2(const T *p);
-template <>
-__device__ __forceinline__ uint32_t ld_l2<uint32_t>(const uint32_t *p) { return __ldcg(p); }
-template <>
-__device__ __forceinline__ Ops32::Bnd ld_l2<Ops32::Bnd>(const Ops32::Bnd *p)
+__device__ __forceinline__ Ops32::Bnd ld_l2(const Ops32::Bnd *p)
 {
     const int2 v = __ldcg(reinterpret_cast<const int2 *>(p));
     return Ops32::Bnd{v.x, v.y};
+}
+
+__device__ __forceinline__ uint64_t ld_relaxed64(const uint64_t *p)
+{
+    uint64_t v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ void st_relaxed64(uint64_t *p, uint64_t v)
+{
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+
+// Boundary rows between the warps of a pair, int16 forms: one 64-bit word per
+// genome row, the [H, I] entry below and the number of the work item that it
+// is meant for above (the words are zero before a run).  Entry and number
+// travel in one access, so a row needs no other order: the reader takes a
+// chunk's words, and again those that have not arrived.  A counter of
+// published chunks, its release after the stream's stores and its acquire
+// before a second read of the rows took 22% of the warps' time on the
+// 4,096-pair workload.
+struct RowsIn {
+    static constexpr uint32_t kPast = Ops16::NEGV;        // [H, I] = -inf
+    uint64_t v[kChunk / 32];
+    // queue the rows row, row+1, .. of a chunk (rows past the region are never
+    // written)
+    __device__ __forceinline__ void fetch(const uint64_t *rows, int row, int n, uint32_t tag, int lane)
+    {
+#pragma unroll
+        for (int q = 0; q < kChunk / 32; ++q) {
+            const int r = row + lane + 32 * q;
+            v[q] = r < n ? ld_relaxed64(rows + r) : static_cast<uint64_t>(tag) << 32 | kPast;
+        }
+    }
+    // wait (bounded) until every row queued has arrived; false: it ran out
+    __device__ __forceinline__ bool settle(const uint64_t *rows, int row, uint32_t tag, int lane, uint32_t limit)
+    {
+        for (uint32_t it = 0;; ++it) {
+            bool ok = true;
+#pragma unroll
+            for (int q = 0; q < kChunk / 32; ++q) ok = ok && static_cast<uint32_t>(v[q] >> 32) == tag;
+            if (__all_sync(kFull, ok)) return true;
+            if (it >= limit) return false;
+            __nanosleep(100);
+#pragma unroll
+            for (int q = 0; q < kChunk / 32; ++q)
+                if (static_cast<uint32_t>(v[q] >> 32) != tag) v[q] = ld_relaxed64(rows + row + lane + 32 * q);
+        }
+    }
+};
+
+// The pair's best cell among a strip's cells that hold `top`, the strip's
+// maximum: the lanes of `who` hold it in half k of their words, whose column
+// is j0 + 2 * lane.  cmax: the strip's column maxima per chunk of kChunk
+// steps, which start `shift` steps of the strip before multiples of kChunk
+// (the last one's covers every later step).  The whole warp searches: the
+// chunks 32 at a time, then the first such chunk's steps.
+__device__ __forceinline__ void best_in_strip(const uint8_t *strip, const uint32_t *cmax, int schunks, int shift,
+                                              unsigned who, int k, int j0, int n, int top, int lane, Best &best)
+{
+    while (who) {
+        const int L = __ffs(who) - 1, r0 = 2 * L + k;                  // r0: the step of row 0
+        who &= who - 1;
+        int c = -1;
+        for (int cb = 0; cb < schunks && c < 0; cb += 32) {
+            const bool hit = cb + lane < schunks && Ops16::word_h(cmax[(cb + lane) * 32 + L], k) == top;
+            const unsigned b = __ballot_sync(kFull, hit);
+            if (b) c = cb + __ffs(b) - 1;
+        }
+        if (c < 0) continue;
+        const int t0 = c * kChunk - shift;
+        const int ta = max(t0, r0), te = c == schunks - 1 ? r0 + n : min(t0 + kChunk, r0 + n);
+        for (int g = ta & ~3; g < te; g += 128) {
+            const int t = g + 4 * lane;
+            int found = 0x7fffffff;
+            if (t < te) {
+                const uint4 w = *reinterpret_cast<const uint4 *>(strip + static_cast<size_t>(t) * kStepBytes + L * 16);
+#pragma unroll
+                for (int u = 3; u >= 0; --u) {
+                    const uint32_t x = u == 0 ? w.x : u == 1 ? w.y : u == 2 ? w.z : w.w;
+                    if (t + u >= ta && t + u < te && Ops16::word_h(x, k) == top) found = t + u;
+                }
+            }
+            found = __reduce_min_sync(kFull, found);
+            if (found != 0x7fffffff) {
+                const int ii = found - r0, jj = j0 + 2 * L;
+                if (better(top, ii, jj, best)) best = Best{top, ii, jj};
+                break;
+            }
+        }
+    }
 }
 
 // (score, ii, jj) -> key whose unsigned maximum is the best cell under the
@@ -923,14 +1349,87 @@ __device__ __forceinline__ unsigned long long best_key(int score, int ii, int jj
            static_cast<unsigned long long>(0xfffffu - static_cast<uint32_t>(jj));
 }
 
+// The end of a work item of pair p (one of its n_items): its best cell joins
+// the pair's, and the warp that finishes the pair's last item publishes the
+// pair's result and traces it (or queues it for the int32 kernel).
+__device__ __forceinline__ void finish_strip(const DPArgs &a, const PairDesc &pd, uint32_t p, Best best, bool timed_out,
+                                             int lane, uint32_t n_items, bool rerun, bool int32)
+{
+    // warp reduction of (score desc, ii asc, jj asc)
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        Best o;
+        o.score = __shfl_xor_sync(kFull, best.score, off);
+        o.ii = __shfl_xor_sync(kFull, best.ii, off);
+        o.jj = __shfl_xor_sync(kFull, best.jj, off);
+        if (better(o.score, o.ii, o.jj, best)) best = o;
+    }
+    int trace_now = 0;
+    if (lane == 0) {
+        if (best.score > 0) atomicMax(a.best_key + p, best_key(best.score, best.ii, best.jj));
+        if (timed_out) atomicOr(&a.out[p].status, MP_ST_TIMEOUT);
+        __threadfence();
+        const uint32_t done = atomicAdd(a.strips_done + p, 1u);
+        if (done == n_items - 1) {
+            // last strip of the pair: publish the pair's best cell
+            __threadfence();
+            const unsigned long long key = atomicAdd(a.best_key + p, 0ull);
+            PairOut &o = a.out[p];
+            const int score = static_cast<int>(key >> 40);
+            o.score = score;
+            if (int32) o.status |= kStInt32Stream;
+            o.best_ii = score > 0 ? static_cast<int>(0xfffffu - ((key >> 20) & 0xfffffu)) : -1;
+            o.best_jj = score > 0 ? static_cast<int>(0xfffffu - (key & 0xfffffu)) : -1;
+            if (!rerun && !int32 && score >= kOverflowT && !(o.status & MP_ST_TIMEOUT) &&
+                !(pd.flags & PF_WIDE)) {
+                // cannot happen: the pair's score bound was below the int16 limit
+                o.status |= MP_ST_TRACE;
+            } else if (!rerun && !int32 && score >= kOverflowT && !(o.status & MP_ST_TIMEOUT)) {
+                // int16 saturated: queue every strip of this pair for the int32 kernel
+                o.status |= MP_ST_RERUN;
+                a.best_key[p] = 0;
+                a.strips_done[p] = 0;
+                for (uint32_t k = 0; k < pd.n_strips; ++k) a.progress[pd.strip_base + k] = 0;
+                const uint32_t slot = atomicAdd(a.rerun_count, pd.n_strips);
+                for (uint32_t k = 0; k < pd.n_strips; ++k) a.rerun_items[slot + k] = make_uint2(p, k);
+            }
+            // the pair is final (not queued for the int32 kernel): trace it now,
+            // while other warps run other strips
+            trace_now = a.mat != nullptr && !(o.status & MP_ST_ERRMASK) &&
+                        !(pd.flags & (PF_SCORE_ONLY | PF_SKIP | PF_BUDGET)) &&
+                        (!(o.status & MP_ST_RERUN) || int32) &&
+                        (score > 0 || a.sp.mode == MP_MODE_GLOBAL);
+        }
+    }
+    trace_now = __shfl_sync(kFull, trace_now, 0);
+    __syncwarp();
+    if (trace_now) {
+        __threadfence();        // the other strips' streams (published before their count) are visible
+        trace_inline(a, p, lane);
+        __syncwarp();
+        if (lane == 0) a.out[p].status |= kStTraced;
+    }
+    __syncwarp();
+}
+
+// the pair's best key so far (it only grows)
+__device__ __forceinline__ unsigned long long ld_best(const unsigned long long *p)
+{
+    return ld_relaxed64(reinterpret_cast<const uint64_t *>(p));
+}
+
 // One strip s of pair p (64 residues, two per lane, or 128, four per lane).
 // Strip s reads the boundary row (H and I of the last residue of strip s-1
 // at every genome position) that strip s-1 publishes chunk by chunk, and
-// publishes its own last residue for strip s+1.
+// publishes its own last residue for strip s+1: as RowsIn's words (int16) or,
+// in the int32 kernel, whose entries are 64 bits themselves, as entries and a
+// count of published chunks.  item: the strip's number among the pair's work
+// items (n_items of them).
 template <typename Ops>
-__device__ void run_strip(const DPArgs &a, typename Ops::Smem &sm, const PairDesc &pd, uint32_t p, int s, int lane,
-                          bool rerun)
+__device__ void run_strip(const DPArgs &a, typename Ops::Smem &sm, const PairDesc &pd, uint32_t p, int s, uint32_t item,
+                          uint32_t n_items, int lane, bool rerun)
 {
+    constexpr bool kTagged = sizeof(typename Ops::Bnd) == 4;
     using Bnd = typename Ops::Bnd;
     constexpr int W = Ops::W, CPL = Ops::CPL;
     const int n = static_cast<int>(pd.nt_len);
@@ -938,7 +1437,8 @@ __device__ void run_strip(const DPArgs &a, typename Ops::Smem &sm, const PairDes
     const int nstrips = static_cast<int>(pd.n_strips);
     const bool store = !(pd.flags & PF_SCORE_ONLY);
     const uint8_t *P = a.prot + pd.prot_off;
-    Bnd *bnd = reinterpret_cast<Bnd *>(a.bnd) + pd.bnd_off + kBndPad;   // bnd[ii], ii >= -kBndPad
+    Bnd *bnd = reinterpret_cast<Bnd *>(a.bnd) + pd.bnd_off + kBndPad;   // int32: bnd[ii], ii >= -kBndPad
+    uint64_t *rows = static_cast<uint64_t *>(a.bnd) + pd.bnd_off + kBndPad;      // int16: rows[ii]
     typename Ops::Consts c = Ops::consts(a.sp);
     // anchored modes: row 0 holds H[0][j] = -(q + e j) (an I run from cell
     // (0, 0)) and column 0 the values of the column-0 array; local: both 0
@@ -976,7 +1476,7 @@ __device__ void run_strip(const DPArgs &a, typename Ops::Smem &sm, const PairDes
     // wait until strip s-1 has published `need` chunks (bounded)
     const uint32_t spin_limit = a.spin_limit ? a.spin_limit : kSpinLimit;
     auto wait_for = [&](uint32_t need) {
-        if (s == 0 || timed_out) return;
+        if (kTagged || s == 0 || timed_out) return;
         uint32_t ok = 1;
         if (lane == 0) {
             uint32_t it = 0;
@@ -1002,16 +1502,16 @@ __device__ void run_strip(const DPArgs &a, typename Ops::Smem &sm, const PairDes
             // a profile query: position-specific scores (no codon: -512 as subst_score)
 #pragma unroll 2
             for (int aa = 0; aa < kProfRows; ++aa) {
-                sm.prof[aa * 32 + lane] =
+                sm.prof[aa * Ops::kRowWords + lane] =
                     Ops::prof_entry(aa == 21 ? -512 : jlo < m ? pf[jlo + 1].s[aa] : subst_score(a.sp, aa, 21), 0);
-                sm.prof[(kProfRows + aa) * 32 + lane] =
+                sm.prof[aa * Ops::kRowWords + Ops::kHiWords + lane] =
                     Ops::prof_entry(0, aa == 21 ? -512 : jhi < m ? pf[jhi + 1].s[aa] : subst_score(a.sp, aa, 21));
             }
         } else {
 #pragma unroll 2
             for (int aa = 0; aa < kProfRows; ++aa) {
-                sm.prof[aa * 32 + lane] = Ops::prof_entry(subst_score(a.sp, aa, plo), 0);
-                sm.prof[(kProfRows + aa) * 32 + lane] = Ops::prof_entry(0, subst_score(a.sp, aa, phi));
+                sm.prof[aa * Ops::kRowWords + lane] = Ops::prof_entry(subst_score(a.sp, aa, plo), 0);
+                sm.prof[aa * Ops::kRowWords + Ops::kHiWords + lane] = Ops::prof_entry(0, subst_score(a.sp, aa, phi));
             }
         }
         // records for ii in [-kChunk, kChunk)
@@ -1026,16 +1526,29 @@ __device__ void run_strip(const DPArgs &a, typename Ops::Smem &sm, const PairDes
     wait_for(nchunks < kLag ? nchunks : kLag);
     __syncwarp();
     typename Ops::State st;
+    RowsIn in;
     {
-        const Bnd w0 = s > 0 ? ld_l2(bnd) : (anchored ? Ops::col0_entry(__ldg(c0 + 1)) : Ops::kBnd0);
+        Bnd w0 = anchored ? Ops::col0_entry(__ldg(c0 + 1)) : Ops::kBnd0;
+        if constexpr (kTagged) {
+            if (s > 0) {
+                // row 0 (every lane's words are the same), then the first chunk's rows
+                RowsIn first;
+                first.fetch(rows, -lane, 1, item, lane);
+                if (!first.settle(rows, -lane, item, lane, spin_limit)) timed_out = true;
+                w0 = static_cast<Bnd>(first.v[0]);
+                in.fetch(rows, 1, n, item, lane);
+            }
+        } else if (s > 0) {
+            w0 = ld_l2(bnd);
+        }
         if constexpr (CPL == 4) {
             Ops::init(st, sm, lane, w0, row0(jcol), row0(jcol - 1));
         } else {
             const int ii0 = -2 * lane;
             const uint4 rm1 = get_record(sm, ii0 - 1);
-            const uint4 rm2 = get_record(sm, ii0 - 2);
-            const uint32_t xm1 = sm.prof[(kProfRows + (rm1.z >> 7)) * 32 + lane];   // the hi table
-            Ops::init(st, lane, w0, rm1, rm2, xm1, row0(jcol), row0(jcol - 1));
+            const uint4 rm2 = get_record(sm, ii0 - 2), rm3 = get_record(sm, ii0 - 3);
+            const uint32_t xm1 = sm.prof[rm1.z / 4 + Ops::kHiWords + lane];   // the hi table
+            Ops::init(st, lane, w0, rm1, rm2, rm3, xm1, row0(jcol), row0(jcol - 1));
         }
     }
     uint8_t *code_strip = a.codes + pd.code_off + static_cast<size_t>(s) * strip_bytes;
@@ -1043,7 +1556,10 @@ __device__ void run_strip(const DPArgs &a, typename Ops::Smem &sm, const PairDes
     typename Ops::ColMax *colmax = reinterpret_cast<typename Ops::ColMax *>(
         a.codes + pd.code_off + static_cast<size_t>(nstrips) * strip_bytes) + static_cast<size_t>(s) * nchunks * 32;
     Best best{0, 0x7fffffff, 0x7fffffff};
-    int cbest[CPL], cchunk[CPL];                    // per cell: best chunk maximum and its chunk
+    // with a stream, int16: the largest chunk maximum so far, and in the
+    // 128-residue form its chunk (otherwise found again at the end)
+    typename Ops::ColMax rmax{};
+    int cbest[CPL], cchunk[CPL];
 #pragma unroll
     for (int k = 0; k < CPL; ++k) cbest[k] = cchunk[k] = 0;
 
@@ -1058,6 +1574,12 @@ __device__ void run_strip(const DPArgs &a, typename Ops::Smem &sm, const PairDes
             for (int k = lane; k < kChunk; k += 32) sm.bin[k] = Ops::col0_entry(__ldg(c0 + t0 + 2 + k));
         } else if (s == 0) {
             for (int k = lane; k < kChunk; k += 32) sm.bin[k] = Ops::kBnd0;   // column 0: H = 0, I = -inf
+        } else if constexpr (kTagged) {
+            if (!timed_out && !in.settle(rows, t0 + 1, item, lane, spin_limit)) timed_out = true;
+#pragma unroll
+            for (int q = 0; q < kChunk / 32; ++q) sm.bin[lane + 32 * q] = static_cast<Bnd>(in.v[q]);
+            // the next chunk's rows, on their way while this one computes
+            if (ch + 1 < nchunks) in.fetch(rows, t0 + kChunk + 1, n, item, lane);
         } else {
             for (int k = lane; k < kChunk; k += 32) sm.bin[k] = ld_l2(bnd + t0 + 1 + k);
         }
@@ -1068,42 +1590,58 @@ __device__ void run_strip(const DPArgs &a, typename Ops::Smem &sm, const PairDes
             else fetch_records(sm, recs, t0 + kChunk, lane);
         }
         const bool masked = (t0 < W) || (t0 + kChunk > n);
+        // the last chunk runs no further than the last valid row
+        const int bodies = (min(kChunk, nsteps - t0) + kBody - 1) / kBody;
         if constexpr (CPL == 4) {
             if (masked) {
-                if (store) Ops::template chunk<true, true>(st, c, sm, lane, t0, n, code_strip);
-                else Ops::template chunk<true, false>(st, c, sm, lane, t0, n, code_strip);
+                if (store) Ops::template chunk<true, true>(st, c, sm, lane, t0, n, bodies, code_strip);
+                else Ops::template chunk<true, false>(st, c, sm, lane, t0, n, bodies, code_strip);
             } else {
-                if (store) Ops::template chunk<false, true>(st, c, sm, lane, t0, n, code_strip);
-                else Ops::template chunk<false, false>(st, c, sm, lane, t0, n, code_strip);
+                if (store) Ops::template chunk<false, true>(st, c, sm, lane, t0, n, bodies, code_strip);
+                else Ops::template chunk<false, false>(st, c, sm, lane, t0, n, bodies, code_strip);
             }
         } else {
-            if (masked) {
-                if (store) run_chunk<Ops, true, true>(st, c, sm, lane, t0, n, code_strip);
-                else run_chunk<Ops, true, false>(st, c, sm, lane, t0, n, code_strip);
+            if (!kTagged ? masked : anchored && t0 < W) {
+                if (store) run_chunk<Ops, 2, true>(st, c, sm, lane, t0, n, bodies, code_strip);
+                else run_chunk<Ops, 2, false>(st, c, sm, lane, t0, n, bodies, code_strip);
+            } else if (store) {
+                run_chunk<Ops, 0, true>(st, c, sm, lane, t0, n, bodies, code_strip);
+            } else if (kTagged && masked) {
+                run_chunk<Ops, 1, false>(st, c, sm, lane, t0, n, bodies, code_strip);
             } else {
-                if (store) run_chunk<Ops, false, true>(st, c, sm, lane, t0, n, code_strip);
-                else run_chunk<Ops, false, false>(st, c, sm, lane, t0, n, code_strip);
+                run_chunk<Ops, 0, false>(st, c, sm, lane, t0, n, bodies, code_strip);
             }
         }
         __syncwarp();
         if (s + 1 < nstrips && !a.no_publish) {
-            // publish residue W(s+1)-1 for strip s+1
+          // publish residue W(s+1)-1 for strip s+1
+          if constexpr (kTagged) {
+            for (int k = lane; k < kChunk; k += 32) {
+                const int r = t0 + k - (W - 1);
+                if (r >= 0 && r < n) st_relaxed64(rows + r, static_cast<uint64_t>(item + 1) << 32 | sm.bout[k]);
+            }
+          } else {
             for (int k = lane; k < kChunk; k += 32) bnd[t0 + k - (W - 1)] = sm.bout[k];
             // __syncwarp orders every lane's stores before lane 0's release
             // (release is cumulative), so one release store publishes the chunk
             __syncwarp();
             if (lane == 0) st_release(mine, static_cast<uint32_t>(ch + 1));
+          }
         }
         if (store) colmax[static_cast<size_t>(ch) * 32 + lane] = Ops::chunk_max(st);
         bool folded = false;
         if constexpr (Ops::kChunkMaxBest) {
             if (store) {
-                // remember the first chunk holding each cell's maximum
                 const typename Ops::ColMax cmw = Ops::chunk_max(st);
+                if constexpr (CPL == 2) {
+                    rmax = vmax(rmax, cmw);
+                } else {
+                    // remember the first chunk holding each cell's maximum
 #pragma unroll
-                for (int k = 0; k < CPL; ++k) {
-                    const int v = Ops::cell_max(cmw, k);
-                    if (v > cbest[k]) { cbest[k] = v; cchunk[k] = ch; }
+                    for (int k = 0; k < CPL; ++k) {
+                        const int v = Ops::cell_max(cmw, k);
+                        if (v > cbest[k]) { cbest[k] = v; cchunk[k] = ch; }
+                    }
                 }
                 folded = true;
             }
@@ -1124,172 +1662,373 @@ __device__ void run_strip(const DPArgs &a, typename Ops::Smem &sm, const PairDes
     }
     if constexpr (Ops::kChunkMaxBest) {
       if (store) {
-        // first step of the best chunk holding the maximum, read back from this
-        // lane's own stored H values (valid cells only)
+        // the strip's maximum, and the first step that holds it, read back from
+        // the stored H values (valid cells only)
         __syncwarp();
+        if constexpr (CPL == 2) {
+            const int v0 = jcol - 1 < m ? Ops::word_h(rmax, 0) : 0, v1 = jcol < m ? Ops::word_h(rmax, 1) : 0;
+            const int top = __reduce_max_sync(kFull, max(v0, v1));
+            // (a pair's best can no longer be here if another strip's is above)
+            const int other = static_cast<int>(__shfl_sync(kFull, ld_best(a.best_key + p), 0) >> 40);
+            if (top > 0 && top >= other) {
+#pragma unroll 1
+                for (int k = 0; k < 2; ++k)
+                    best_in_strip(code_strip, reinterpret_cast<const uint32_t *>(colmax), nchunks, 0,
+                                  __ballot_sync(kFull, (k ? v1 : v0) == top), k, s * W + k, n, top, lane, best);
+            }
+        } else {
+            int top = 0;
 #pragma unroll
-        for (int k = 0; k < CPL; ++k) {
-            const int jj = s * W + CPL * lane + k;
-            if (cbest[k] <= 0 || jj >= m) continue;
-            const int tb = cchunk[k] * kChunk;
-            for (int t = tb; t < tb + kChunk; ++t) {
+            for (int k = 0; k < CPL; ++k)
+                if (s * W + CPL * lane + k < m) top = max(top, cbest[k]);
+            top = __reduce_max_sync(kFull, top);
+#pragma unroll
+            for (int k = 0; k < CPL; ++k) {
+                const int jj = s * W + CPL * lane + k;
+                if (top <= 0 || cbest[k] != top || jj >= m) continue;
+                const int t = Ops::find_cell(code_strip, cchunk[k] * kChunk, lane, k, top, n);
                 const int ii = t - CPL * lane - k;
-                if (ii < 0 || ii >= n) continue;
-                if (Ops::load_cell(code_strip, t, lane, k) == cbest[k]) {
-                    if (better(cbest[k], ii, jj, best)) best = Best{cbest[k], ii, jj};
-                    break;
-                }
+                if (t >= 0 && better(top, ii, jj, best)) best = Best{top, ii, jj};
             }
         }
       }
     }
-    // warp reduction of (score desc, ii asc, jj asc)
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        Best o;
-        o.score = __shfl_xor_sync(kFull, best.score, off);
-        o.ii = __shfl_xor_sync(kFull, best.ii, off);
-        o.jj = __shfl_xor_sync(kFull, best.jj, off);
-        if (better(o.score, o.ii, o.jj, best)) best = o;
-    }
-    int trace_now = 0;
-    if (lane == 0) {
-        if (best.score > 0) atomicMax(a.best_key + p, best_key(best.score, best.ii, best.jj));
-        if (timed_out) atomicOr(&a.out[p].status, MP_ST_TIMEOUT);
-        __threadfence();
-        const uint32_t done = atomicAdd(a.strips_done + p, 1u);
-        if (done == static_cast<uint32_t>(nstrips - 1)) {
-            // last strip of the pair: publish the pair's best cell
-            __threadfence();
-            const unsigned long long key = atomicAdd(a.best_key + p, 0ull);
-            PairOut &o = a.out[p];
-            const int score = static_cast<int>(key >> 40);
-            o.score = score;
-            if (sizeof(Bnd) == 8) o.status |= kStInt32Stream;
-            o.best_ii = score > 0 ? static_cast<int>(0xfffffu - ((key >> 20) & 0xfffffu)) : -1;
-            o.best_jj = score > 0 ? static_cast<int>(0xfffffu - (key & 0xfffffu)) : -1;
-            if (!rerun && sizeof(Bnd) == 4 && score >= kOverflowT && !(o.status & MP_ST_TIMEOUT) &&
-                !(pd.flags & PF_WIDE)) {
-                // cannot happen: the pair's score bound was below the int16 limit
-                o.status |= MP_ST_TRACE;
-            } else if (!rerun && sizeof(Bnd) == 4 && score >= kOverflowT && !(o.status & MP_ST_TIMEOUT)) {
-                // int16 saturated: queue every strip of this pair for the int32 kernel
-                o.status |= MP_ST_RERUN;
-                a.best_key[p] = 0;
-                a.strips_done[p] = 0;
-                for (int k = 0; k < nstrips; ++k) a.progress[pd.strip_base + k] = 0;
-                const uint32_t slot = atomicAdd(a.rerun_count, static_cast<uint32_t>(nstrips));
-                for (int k = 0; k < nstrips; ++k) a.rerun_items[slot + k] = make_uint2(p, k);
-            }
-            // the pair is final (not queued for the int32 kernel): trace it now,
-            // while other warps run other strips
-            trace_now = a.mat != nullptr && !(o.status & MP_ST_ERRMASK) &&
-                        !(pd.flags & (PF_SCORE_ONLY | PF_SKIP | PF_BUDGET)) &&
-                        (!(o.status & MP_ST_RERUN) || sizeof(Bnd) == 8) &&
-                        (score > 0 || a.sp.mode == MP_MODE_GLOBAL);
-        }
-    }
-    trace_now = __shfl_sync(kFull, trace_now, 0);
-    __syncwarp();
-    if (trace_now) {
-        __threadfence();        // the other strips' streams (published before their count) are visible
-        trace_inline(a, p, lane);
-        __syncwarp();
-        if (lane == 0) a.out[p].status |= kStTraced;
-    }
-    __syncwarp();
+    finish_strip(a, pd, p, best, timed_out, lane, n_items, rerun, sizeof(Bnd) == 8);
 }
 
-// MinB: CTAs per SM the build is made for (the register budget per thread
-// follows from it: 3 -> 80, 2 -> 128 for 256-thread CTAs).  Wide4: the
-// int16 build that also runs pairs in 128-residue strips (PF_W128), each
-// warp's shared memory sized for either strip form.
-template <typename Ops, int MinB, bool Wide4 = false>
-__global__ void __launch_bounds__(kWarpsPerCta * 32, MinB) dp_kernel(const DPArgs a, int rerun_only)
+// Two neighbouring strips of pair p, its work item u, on one warp; see Ops16d.
+// Boundary rows pass between the warps of a pair as in run_strip, once per two
+// strips.  With an odd number of strips the first one is an item of its own
+// (Ops16T<true>): a single strip takes fewer clocks per step, so at the front
+// it never waits; at the end it ran at the pace of the warp before it.
+template <bool PROF, bool STORE>
+__device__ void run_duo(const DPArgs &a, WarpSmemD &sm, const PairDesc &pd, uint32_t p, int u, int lane)
+{
+    using Ops = Ops16d;
+    constexpr int kUp = Ops::kUp;
+    const int n = static_cast<int>(pd.nt_len);
+    const int m = static_cast<int>(pd.prot_len);
+    const int nstrips = static_cast<int>(pd.n_strips);
+    const uint32_t item = static_cast<uint32_t>(u), n_items = items_of(pd.flags, pd.n_strips);
+    const uint8_t *P = a.prot + pd.prot_off;
+    uint64_t *rows = static_cast<uint64_t *>(a.bnd) + pd.bnd_off + kBndPad;          // see RowsIn
+    const bool anchored = a.sp.mode != MP_MODE_LOCAL;
+    const int32_t *c0 = anchored ? a.col0 + pd.col0_off : nullptr;      // c0[i] = H[i][0]
+    const ProfPos *pf = PROF ? a.prof + pd.prof_off : nullptr;
+    const int32_t *ep = PROF ? a.epre + pd.prof_off : nullptr;
+    const int s0 = 2 * u - (nstrips & 1);                               // the lower strip
+    const int j0 = kStripW * s0 + 2 * lane;                             // 0-based column of a's low cell
+    auto row0 = [&](int j) {
+        if (!anchored || j == 0) return 0;
+        if (pf) return -(pf[1].q + __ldg(ep + (j < m ? j : m)) + (j > m ? a.sp.e * (j - m) : 0));
+        return -(a.sp.q + a.sp.e * j);
+    };
+    Ops::Consts c;
+    {
+        auto gq = [&](int j) { return pf && j < m ? pf[j + 1].q : a.sp.q; };    // of 0-based column j
+        auto ge = [&](int j) { return pf && j < m ? pf[j + 1].e : a.sp.e; };
+        auto pair = [](int lo, int hi) { return static_cast<uint32_t>(lo) | (static_cast<uint32_t>(hi) << 16); };
+        if (PROF) {
+            c.NQEa = neg2(gq(j0) + ge(j0), gq(j0 + kUp) + ge(j0 + kUp));
+            c.NQEb = neg2(gq(j0 + 1) + ge(j0 + 1), gq(j0 + 1 + kUp) + ge(j0 + 1 + kUp));
+            c.Ea = pair(ge(j0), ge(j0 + kUp));
+            c.Eb = pair(ge(j0 + 1), ge(j0 + 1 + kUp));
+            c.EN = pair(ge(j0 + 2), ge(j0 + 2 + kUp));
+        } else {
+            c.NQEa = c.NQEb = neg2(a.sp.q + a.sp.e, a.sp.q + a.sp.e);
+            c.Ea = c.Eb = c.EN = pair(a.sp.e, a.sp.e);
+        }
+        c.NF = neg2(static_cast<uint32_t>(a.sp.f), static_cast<uint32_t>(a.sp.f));
+        c.FLOOR = anchored ? 0u : Ops::Z;
+        c.ROW0A = Ops16::pack2(row0(j0 + 1), row0(j0 + 1 + kUp));
+        c.ROW0B = Ops16::pack2(row0(j0 + 2), row0(j0 + 2 + kUp));
+        asm volatile("mov.u32 %0, %1;" : "=r"(c.mult) : "r"(lane == 0 ? 65536u : 1u));
+    }
+    // row of a cell at step t: t - 2l - k (lower strip), t - 2l - k - 64 (upper)
+    constexpr int kLast = 2 * kStripW - 1;
+    const uint4 *recs = a.recs + pd.rec_off;            // recs[ii + kRecPre] is position ii
+    const uint32_t limit = a.spin_limit ? a.spin_limit : kSpinLimit;
+    bool timed_out = false;
+    if (lane == 0) {
+        const int schunks = (n + kStripW - 1 + kChunk - 1) / kChunk;    // chunks of a strip's stream
+        const size_t strip_bytes = static_cast<size_t>(schunks) * kChunk * kStepBytes;
+        uint8_t *codes = a.codes + pd.code_off;
+        sm.it.recs = recs;
+        sm.it.rows = rows;
+        sm.it.lo = codes + static_cast<size_t>(s0) * strip_bytes;
+        // per-chunk column maxima of H follow the strips' streams:
+        // [strip][chunk][lane].  Both strips' are taken over the warp's chunks of
+        // steps, for the upper one 64 steps of its own behind (its last entry
+        // covers a chunk past the stream too)
+        sm.it.cmax = reinterpret_cast<uint32_t *>(codes + static_cast<size_t>(nstrips) * strip_bytes) +
+                     static_cast<size_t>(s0) * schunks * 32;
+        sm.it.c0 = c0;
+        sm.it.n = n;
+        sm.it.nsteps = n + kLast;
+        sm.it.schunks = schunks;
+        sm.it.tag = item;
+        sm.it.limit = limit;
+        sm.it.publish = item + 1 < n_items && !a.no_publish;
+        sm.it.anchored = anchored;
+    }
+    // records for ii in [-kChunk, kChunk)
+    fetch_records_d(sm, recs, -kChunk, lane);
+    fetch_records_d(sm, recs, 0, lane);
+    {
+        // profile: the two scores of the lane's columns in each strip
+        int pc[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int j = j0 + (k & 1) + (k >> 1) * kUp;
+            pc[k] = j < m ? P[j] : 21;
+        }
+        auto score = [&](int aa, int k) -> int {
+            const int j = j0 + (k & 1) + (k >> 1) * kUp;
+            if (pf && aa != 21 && j < m) return pf[j + 1].s[aa];
+            return subst_score(a.sp, aa, pf ? 21 : pc[k]);
+        };
+#pragma unroll 2
+        for (int aa = 0; aa < kProfRows; ++aa) {
+            sm.prof[0][aa * 32 + lane] = make_uint2(Ops16::prof_entry(score(aa, 0), 0), Ops16::prof_entry(score(aa, 1), 0));
+            sm.prof[1][aa * 32 + lane] = make_uint2(Ops16::prof_entry(0, score(aa, 2)), Ops16::prof_entry(0, score(aa, 3)));
+        }
+        for (int k = lane; k < kChunk + kBodyD; k += 32) sm.zero[k] = 0;
+    }
+    cp_async_wait_all();
+    __syncwarp();
+    Ops::State st;
+    RowsIn in;
+    {
+        uint32_t w0 = anchored ? Ops16::col0_entry(__ldg(c0 + 1)) : Ops16::kBnd0;
+        if (u > 0) {
+            // row 0 (every lane's words are the same), then the first chunk's rows
+            RowsIn first;
+            first.fetch(rows, -lane, 1, item, lane);
+            if (!first.settle(rows, -lane, item, lane, limit)) timed_out = true;
+            w0 = static_cast<uint32_t>(first.v[0]);
+            in.fetch(rows, 1, n, item, lane);
+        }
+        Ops::init(st, sm, lane, w0, row0(j0 + 1), row0(j0));
+    }
+    uint32_t up_last = 0, rl = 0, ru = 0;               // the last chunk's, and the largest of each strip
+    Best best{0, 0x7fffffff, 0x7fffffff};
+
+#pragma unroll 1
+    for (int t0 = 0; t0 < sm.it.nsteps; t0 += kChunk) {
+        const WarpSmemD::Item &it = sm.it;
+        if (t0 > 0) cp_async_wait_all();                 // this chunk's records (queued last chunk)
+        if (it.tag > 0) {
+            if (!timed_out && !in.settle(it.rows, t0 + 1, it.tag, lane, it.limit)) timed_out = true;
+#pragma unroll
+            for (int q = 0; q < kChunk / 32; ++q) {
+                sm.in[0][lane + 32 * q] = static_cast<uint32_t>(in.v[q]) & 0xffffu;
+                sm.in[1][lane + 32 * q] = static_cast<uint32_t>(in.v[q]) >> 16;
+            }
+            // the next chunk's rows, on their way while this one computes
+            in.fetch(it.rows, t0 + kChunk + 1, it.n, it.tag, lane);
+        } else {
+            // column 0: H = 0, I = -inf; in the anchored modes entry k is row t0 + 2 + k
+            for (int k = lane; k < kChunk; k += 32) {
+                const uint32_t w = it.c0 ? Ops16::col0_entry(__ldg(it.c0 + t0 + 2 + k)) : Ops16::kBnd0;
+                sm.in[0][k] = w & 0xffffu;
+                sm.in[1][k] = w >> 16;
+            }
+        }
+        __syncwarp();
+        // next chunk's records land in ring slots this chunk does not read
+        if (t0 + kChunk < it.nsteps) fetch_records_d(sm, it.recs, t0 + kChunk, lane);
+        {
+            // the last chunk runs no further than the last valid row
+            const int steps = (min(kChunk, it.nsteps - t0) + kBody - 1) / kBody * kBody;
+            const int ulimit = it.schunks * kChunk;
+            Ops::chunk<STORE>(st, c, sm, lane, t0, it.n, it.anchored != 0, steps, it.lo, static_cast<size_t>(ulimit) * kStepBytes, ulimit);
+        }
+        __syncwarp();
+        if (it.publish) {
+            // publish the upper strip's last residue
+            for (int k = lane; k < kChunk; k += 32) {
+                const int r = t0 + k - kLast;
+                if (r >= 0 && r < it.n)
+                    st_relaxed64(it.rows + r,
+                                 static_cast<uint64_t>(it.tag + 1) << 32 | prmt<0x7632>(sm.out[0][k], sm.out[1][k]));
+            }
+        }
+        if (STORE) {
+            const uint32_t cl = prmt<0x5410>(st.cma, st.cmb), cu = prmt<0x7632>(st.cma, st.cmb);
+            uint32_t *cm = it.cmax + lane + t0 / kChunk * 32;
+            if (t0 < it.schunks * kChunk) {
+                cm[0] = cl;
+                cm[it.schunks * 32] = cu;
+            } else {
+                cm[it.schunks * 32 - 32] = vmax(up_last, cu);
+            }
+            up_last = cu;
+            rl = vmax(rl, cl);
+            ru = vmax(ru, cu);
+            st.cma = st.cmb = 0;
+        } else {
+            // fold this chunk's best cells into the warp's best
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const uint32_t key = k == 0 ? st.k0 : k == 1 ? st.k1 : k == 2 ? st.k2 : st.k3;
+                const int sc = static_cast<int>(key >> 16) - 32768;
+                const int jj = j0 + (k & 1) + (k >> 1) * kUp;
+                const int ii = t0 + static_cast<int>(0xffffu - (key & 0xffffu)) - 2 * lane - (k & 1) - (k >> 1) * kUp;
+                if (sc > 0 && jj < m && better(sc, ii, jj, best)) best = Best{sc, ii, jj};
+            }
+            st.TC = 0xffffu;
+            st.k0 = st.k1 = st.k2 = st.k3 = 0;
+        }
+        __syncwarp();
+    }
+    if (STORE) {
+        // the first step that holds the strips' maximum, as in run_strip
+        const WarpSmemD::Item &it = sm.it;
+        const size_t strip_bytes = static_cast<size_t>(it.schunks) * kChunk * kStepBytes;
+        int v[4], top = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            v[k] = j0 + (k & 1) + (k >> 1) * kUp < m ? Ops16::word_h(k < 2 ? rl : ru, k & 1) : 0;
+            top = max(top, v[k]);
+        }
+        top = __reduce_max_sync(kFull, top);
+        const int other = static_cast<int>(__shfl_sync(kFull, ld_best(a.best_key + p), 0) >> 40);
+        if (top > 0 && top >= other) {
+#pragma unroll 1
+            for (int k = 0; k < 4; ++k) {
+                const int vk = k == 0 ? v[0] : k == 1 ? v[1] : k == 2 ? v[2] : v[3];
+                best_in_strip(k < 2 ? it.lo : it.lo + strip_bytes, k < 2 ? it.cmax : it.cmax + it.schunks * 32, it.schunks,
+                              (k >> 1) * kUp,
+                              __ballot_sync(kFull, vk == top), k & 1, j0 - 2 * lane + (k & 1) + (k >> 1) * kUp, n, top,
+                              lane, best);
+            }
+        }
+    }
+    finish_strip(a, pd, p, best, timed_out, lane, n_items, false, false);
+}
+
+// shared memory of a warp of the int16 kernel: the largest of the strip forms it runs
+__host__ __device__ constexpr size_t warp16_bytes(bool wide4)
+{
+    size_t b = sizeof(WarpSmem<Ops16::Bnd>) > sizeof(WarpSmemD) ? sizeof(WarpSmem<Ops16::Bnd>) : sizeof(WarpSmemD);
+    if (wide4 && sizeof(WarpSmem4) > b) b = sizeof(WarpSmem4);
+    return b;
+}
+
+// Warps: warps per CTA, two CTAs per SM (8: at most 128 registers per thread,
+// 6: 168).  Wide4: the int16 build that also runs pairs in 128-residue strips
+// (PF_W128), each warp's shared memory sized for either strip form.
+template <typename Ops, int Warps, bool Wide4 = false>
+__global__ void __launch_bounds__(Warps * 32, 2) dp_kernel(const DPArgs a, int rerun_only)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     using SM = typename Ops::Smem;
-    constexpr size_t kWarpBytes = Wide4 && sizeof(WarpSmem4) > sizeof(SM) ? sizeof(WarpSmem4) : sizeof(SM);
+    constexpr bool kInt16 = sizeof(typename Ops::Bnd) == 4;
+    constexpr size_t kWarpBytes = kInt16 ? warp16_bytes(Wide4) : sizeof(SM);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     unsigned char *mine = smem_raw + static_cast<size_t>(warp) * kWarpBytes;
     // a fixed list (the wave's interleaved strip items, or the re-run list):
     // a strip's warp waits, bounded, for its predecessor's rows
     const uint2 *list = rerun_only ? a.rerun_items : a.items;
     const uint32_t count = rerun_only ? *a.rerun_count : a.n_items;
+    // with fewer items than warps, every CTA's first few take them all: a warp
+    // alone on its scheduler runs a step in half the time of four sharing it
+    if (warp >= static_cast<int>((count + gridDim.x - 1) / gridDim.x)) return;
     for (;;) {
         uint32_t idx = 0;
         if (lane == 0) idx = atomicAdd(a.head, 1u);
         idx = __shfl_sync(kFull, idx, 0);
         if (idx >= count) break;
         const uint2 it = list[idx];
-        const PairDesc pd = a.pairs[it.x];
+        const PairDesc &pd = a.pairs[it.x];
         if constexpr (Wide4) {
             if (pd.flags & PF_W128) {
-                run_strip<Ops16x4>(a, *reinterpret_cast<WarpSmem4 *>(mine), pd, it.x, static_cast<int>(it.y), lane,
-                                   rerun_only != 0);
+                run_strip<Ops16x4>(a, *reinterpret_cast<WarpSmem4 *>(mine), pd, it.x, static_cast<int>(it.y), it.y,
+                                   pd.n_strips, lane, rerun_only != 0);
                 continue;
             }
         }
-        run_strip<Ops>(a, *reinterpret_cast<SM *>(mine), pd, it.x, static_cast<int>(it.y), lane, rerun_only != 0);
+        if constexpr (kInt16) {
+            if (pd.flags & PF_DUO) {
+                const uint32_t n_items = items_of(pd.flags, pd.n_strips);
+                WarpSmemD &smd = *reinterpret_cast<WarpSmemD *>(mine);
+                if (it.y == 0 && (pd.n_strips & 1))
+                    run_strip<Ops16T<true>>(a, *reinterpret_cast<SM *>(mine), pd, it.x, 0, 0u, n_items, lane, false);
+                else if (pd.flags & PF_PROF)
+                    pd.flags & PF_SCORE_ONLY ? run_duo<true, false>(a, smd, pd, it.x, static_cast<int>(it.y), lane)
+                                             : run_duo<true, true>(a, smd, pd, it.x, static_cast<int>(it.y), lane);
+                else
+                    pd.flags & PF_SCORE_ONLY ? run_duo<false, false>(a, smd, pd, it.x, static_cast<int>(it.y), lane)
+                                             : run_duo<false, true>(a, smd, pd, it.x, static_cast<int>(it.y), lane);
+                continue;
+            }
+        }
+        run_strip<Ops>(a, *reinterpret_cast<SM *>(mine), pd, it.x, static_cast<int>(it.y), it.y, pd.n_strips, lane,
+                       rerun_only != 0);
     }
 }
 
 }  // namespace
 
-size_t dp16_smem_bytes() { return sizeof(WarpSmem<Ops16::Bnd>) * kWarpsPerCta; }
-size_t dp16w_smem_bytes()
-{
-    return (sizeof(WarpSmem4) > sizeof(WarpSmem<Ops16::Bnd>) ? sizeof(WarpSmem4) : sizeof(WarpSmem<Ops16::Bnd>)) *
-           kWarpsPerCta;
-}
-size_t dp32_smem_bytes() { return sizeof(WarpSmem<Ops32::Bnd>) * kWarpsPerCta; }
-
-static int blocks_per_sm(const void *fn, size_t smem)
+static int blocks_per_sm(const void *fn, int warps, size_t smem)
 {
     int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, kWarpsPerCta * 32, smem) != cudaSuccess)
-        return 1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, warps * 32, smem) != cudaSuccess) return 1;
     return nb > 0 ? nb : 1;
 }
 
 // The shared-memory opt-in is a per-device function attribute: set it, and
 // read the occupancy, once per device and build.
-template <typename Ops, int MinB, bool Wide4 = false>
-static int kernel_blocks_per_sm(size_t smem)
-{
-    constexpr int kMaxDev = 64;
-    static std::atomic<int> nb[kMaxDev];
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDev) dev = 0;
-    int v = nb[dev].load(std::memory_order_relaxed);
-    if (v <= 0) {
-        cudaFuncSetAttribute(dp_kernel<Ops, MinB, Wide4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(smem));
-        v = blocks_per_sm(reinterpret_cast<const void *>(dp_kernel<Ops, MinB, Wide4>), smem);
-        nb[dev].store(v, std::memory_order_relaxed);
+template <typename Ops, int Warps, bool Wide4 = false>
+struct DpBuild {
+    static constexpr size_t kSmem =
+        Warps * (sizeof(typename Ops::Bnd) == 4 ? warp16_bytes(Wide4) : sizeof(typename Ops::Smem));
+    static int blocks_per_sm()
+    {
+        constexpr int kMaxDev = 64;
+        static std::atomic<int> nb[kMaxDev];
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDev) dev = 0;
+        int v = nb[dev].load(std::memory_order_relaxed);
+        if (v <= 0) {
+            cudaFuncSetAttribute(dp_kernel<Ops, Warps, Wide4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 static_cast<int>(kSmem));
+            v = mpdp::blocks_per_sm(reinterpret_cast<const void *>(dp_kernel<Ops, Warps, Wide4>), Warps, kSmem);
+            nb[dev].store(v, std::memory_order_relaxed);
+        }
+        return v;
     }
-    return v;
-}
+    static cudaError_t launch(const DPArgs &a, int grid, int rerun_only, cudaStream_t st)
+    {
+        blocks_per_sm();
+        dp_kernel<Ops, Warps, Wide4><<<grid, Warps * 32, kSmem, st>>>(a, rerun_only);
+        return cudaGetLastError();
+    }
+};
 
 int dp16_blocks_per_sm(int variant, bool wide4)
 {
-    if (wide4) return kernel_blocks_per_sm<Ops16, 2, true>(dp16w_smem_bytes());
-    return variant == 1 ? kernel_blocks_per_sm<Ops16, 2>(dp16_smem_bytes())
-                        : kernel_blocks_per_sm<Ops16, 3>(dp16_smem_bytes());
+    if (wide4) return DpBuild<Ops16, kWarps16, true>::blocks_per_sm();
+    return variant == 1 ? DpBuild<Ops16, kWarps16>::blocks_per_sm() : DpBuild<Ops16, kWarpsPerCta>::blocks_per_sm();
 }
 
-int dp32_blocks_per_sm() { return kernel_blocks_per_sm<Ops32, 2>(dp32_smem_bytes()); }
+int dp16_warps_per_cta(int variant, bool wide4) { return wide4 || variant == 1 ? kWarps16 : kWarpsPerCta; }
+
+int dp32_blocks_per_sm() { return DpBuild<Ops32, kWarpsPerCta>::blocks_per_sm(); }
 
 namespace {
 // Per-nt records of every pair (see make_record), positions -kRecPre upwards
 // (z, the profile row's byte offset, for the pair's strip form: rows of 32
-// lanes x 4 B, or x 8 B in 128-residue strips).
+// lanes x 4 B, or x 8 B in 128-residue strips and where warps run two strips).  For pairs whose warps run two
+// strips the high halves of x and y and the offset w belong to the row 64
+// before instead of the one before.
 // The genetic code and the splice terms are looked up in shared tables
 // (lanes index them at different positions: from constant memory such
 // reads serialise), the splice terms by three 5-symbol codes (four bases and
 // "outside the region"), filled from the splice model's own functions.
+// Also clears the boundary rows that the pair's warps will hand on.
 __global__ void records_kernel(const PairDesc *pairs, uint32_t n_pairs, const uint32_t *nt2, const ScoreParams sp,
-                               uint4 *recs)
+                               uint4 *recs, uint64_t *bnd)
 {
     __shared__ int8_t s_code[64];
     __shared__ int16_t s_don[125], s_acc[125];
@@ -1310,52 +2049,56 @@ __global__ void records_kernel(const PairDesc *pairs, uint32_t n_pairs, const ui
         const int cnt = static_cast<int>(records_of(pd.nt_len));
         const uint32_t *g = nt2 + pd.nt_word_off;
         uint4 *out = recs + pd.rec_off;
-        const uint32_t zrow = (pd.flags & PF_W128) ? 256u : 128u;
-        for (int k = threadIdx.x; k < cnt; k += blockDim.x) {
-            // the same record as make_record: window T0[ii-3 .. ii+4]
-            const int ii = k - kRecPre;
+        const uint32_t zrow = (pd.flags & (PF_W128 | PF_DUO)) ? 256u : 128u;
+        // the row of the high halves: the one before, or 64 rows back for pairs
+        // whose warps run two strips (rows before the region all read alike)
+        const int back = (pd.flags & PF_DUO) ? Ops16d::kUp : 1;
+        // row ii: d(i+1), a(i) and the codon's amino acid, from T0[ii-3 .. ii+4]
+        auto row = [&](int ii, uint32_t &d, uint32_t &ac, uint32_t &aa) {
             const int s0 = ii - 3;
             const int w = s0 >> 4;
             const uint64_t pair64 = (static_cast<uint64_t>(g[w + 1]) << 32) | g[w];
             const uint32_t win = static_cast<uint32_t>(pair64 >> ((s0 & 15) * 2));
             int c[8];
 #pragma unroll
-            for (int q = 0; q < 8; ++q)
+            for (int q = 1; q < 8; ++q)
                 c[q] = static_cast<unsigned>(s0 + q) < static_cast<unsigned>(n) ? static_cast<int>((win >> (2 * q)) & 3)
                                                                                : 4;
-            const int aa = (c[1] != 4 && c[3] != 4) ? s_code[c[1] * 16 + c[2] * 4 + c[3]] : 21;
-            const uint32_t dC = static_cast<uint32_t>(s_don[(c[5] * 5 + c[6]) * 5 + c[7]]);   // d(i+1)
-            const uint32_t dB = static_cast<uint32_t>(s_don[(c[4] * 5 + c[5]) * 5 + c[6]]);   // d(i)
-            const uint32_t aA = static_cast<uint32_t>(s_acc[(c[1] * 5 + c[2]) * 5 + c[3]]);   // a(i)
-            const uint32_t aC = static_cast<uint32_t>(s_acc[(c[0] * 5 + c[1]) * 5 + c[2]]);   // a(i-1)
-            out[k] = make_uint4(neg2(r + dC, r + dB), neg2(aA, aC), static_cast<uint32_t>(aa) * zrow, 0u);
+            aa = static_cast<uint32_t>((c[1] != 4 && c[3] != 4) ? s_code[c[1] * 16 + c[2] * 4 + c[3]] : 21);
+            d = static_cast<uint32_t>(s_don[(c[5] * 5 + c[6]) * 5 + c[7]]);
+            ac = static_cast<uint32_t>(s_acc[(c[1] * 5 + c[2]) * 5 + c[3]]);
+        };
+        if (items_of(pd.flags, pd.n_strips) > 1)
+            for (int k = threadIdx.x; k < n; k += blockDim.x) bnd[pd.bnd_off + kBndPad + k] = 0;
+        for (int k = threadIdx.x; k < cnt; k += blockDim.x) {
+            const int ii = k - kRecPre;
+            uint32_t d0, a0, aa0, d1, a1, aa1;
+            row(ii, d0, a0, aa0);
+            row(max(ii - back, -kRecPre), d1, a1, aa1);
+            out[k] = make_uint4(neg2(r + d0, r + d1), neg2(a0, a1), aa0 * zrow, aa1 * zrow);
         }
     }
 }
 }  // namespace
 
 cudaError_t launch_records(const PairDesc *pairs, uint32_t n, const uint32_t *nt2, const ScoreParams &sp, uint4 *recs,
-                           cudaStream_t st)
+                           uint64_t *bnd, cudaStream_t st)
 {
     if (n == 0) return cudaSuccess;
-    records_kernel<<<n < 8192 ? n : 8192, 256, 0, st>>>(pairs, n, nt2, sp, recs);
+    records_kernel<<<n < 8192 ? n : 8192, 256, 0, st>>>(pairs, n, nt2, sp, recs, bnd);
     return cudaGetLastError();
 }
 
 cudaError_t launch_dp16(const DPArgs &a, int grid, int variant, bool wide4, cudaStream_t st)
 {
-    dp16_blocks_per_sm(variant, wide4);
-    if (wide4) dp_kernel<Ops16, 2, true><<<grid, kWarpsPerCta * 32, dp16w_smem_bytes(), st>>>(a, 0);
-    else if (variant == 1) dp_kernel<Ops16, 2><<<grid, kWarpsPerCta * 32, dp16_smem_bytes(), st>>>(a, 0);
-    else dp_kernel<Ops16, 3><<<grid, kWarpsPerCta * 32, dp16_smem_bytes(), st>>>(a, 0);
-    return cudaGetLastError();
+    if (wide4) return DpBuild<Ops16, kWarps16, true>::launch(a, grid, 0, st);
+    return variant == 1 ? DpBuild<Ops16, kWarps16>::launch(a, grid, 0, st)
+                        : DpBuild<Ops16, kWarpsPerCta>::launch(a, grid, 0, st);
 }
 
 cudaError_t launch_dp32(const DPArgs &a, int grid, bool rerun_only, cudaStream_t st)
 {
-    dp32_blocks_per_sm();
-    dp_kernel<Ops32, 2><<<grid, kWarpsPerCta * 32, dp32_smem_bytes(), st>>>(a, rerun_only ? 1 : 0);
-    return cudaGetLastError();
+    return DpBuild<Ops32, kWarpsPerCta>::launch(a, grid, rerun_only ? 1 : 0, st);
 }
 
 }  // namespace mpdp
@@ -1392,7 +2135,7 @@ struct NoAllocScratch {
     uint32_t nt2[kNANtWords];
     uint4 recs[records_of(kNAMaxNt)];
     uint8_t prot[kNAMaxProt];
-    Ops32::Bnd bnd[kNABndEntries];                   // int32 entries; the int16 pass uses the first half
+    alignas(8) Ops32::Bnd bnd[kNABndEntries];        // int32 entries, or the int16 pass's rows (see RowsIn)
 };
 
 // The scratch itself (about 820 KB).  Host code must not pass this name to a
@@ -1452,6 +2195,8 @@ dp_noalloc_kernel(ScoreParams sp, const char *prot_ascii, int m, const char *nt_
     __syncthreads();
     // every call starts from zeroed progress counters
     for (int k = threadIdx.x; k < kNAMaxStrips; k += blockDim.x) S->progress[k] = 0;
+    if (nstrips > 1)
+        for (int k = threadIdx.x; k < n; k += blockDim.x) reinterpret_cast<uint64_t *>(S->bnd)[kBndPad + k] = 0;
     for (int k = threadIdx.x; k < m; k += blockDim.x)
         S->prot[k] = na_aa_code(static_cast<unsigned char>(prot_ascii[k]));
     const int nwords = (n + 15) / 16;
@@ -1496,7 +2241,7 @@ dp_noalloc_kernel(ScoreParams sp, const char *prot_ascii, int m, const char *nt_
                 if (lane == 0) s = atomicAdd(&S->head16, 1u);
                 s = __shfl_sync(kFull, s, 0);
                 if (s >= static_cast<uint32_t>(nstrips)) break;
-                run_strip<Ops16>(a, sm, pd, 0, static_cast<int>(s), lane, false);
+                run_strip<Ops16>(a, sm, pd, 0, static_cast<int>(s), s, pd.n_strips, lane, false);
             }
         }
         __syncthreads();
@@ -1508,7 +2253,8 @@ dp_noalloc_kernel(ScoreParams sp, const char *prot_ascii, int m, const char *nt_
                 if (lane == 0) s = atomicAdd(&S->head32, 1u);
                 s = __shfl_sync(kFull, s, 0);
                 if (s >= nre) break;
-                run_strip<Ops32>(a, sm, pd, 0, static_cast<int>(S->rerun_items[s].y), lane, true);
+                const uint32_t k = S->rerun_items[s].y;
+                run_strip<Ops32>(a, sm, pd, 0, static_cast<int>(k), k, pd.n_strips, lane, true);
             }
         }
         __syncthreads();

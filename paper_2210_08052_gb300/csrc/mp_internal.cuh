@@ -17,7 +17,8 @@ constexpr int kRingPad = 12;    // mirrored entries so a body never wraps
 constexpr int kProfRows = 22;   // translated amino acid 0..19, stop 20, no codon 21
 constexpr int kBndPad = kStripWMax;   // boundary entries before genome position 0
 constexpr int kRecPre = 2 * kChunk;   // per-nt records before genome position 0
-constexpr int kWarpsPerCta = 8; // persistent DP kernel
+constexpr int kWarpsPerCta = 8; // warps per CTA of the persistent DP kernels
+constexpr int kWarps16 = 6;     // of the int16 build with more registers per thread (168 instead of 128)
 constexpr int kNtPadWords = 16; // zero words around each packed genome
 
 // bytes of the traceback stream per strip step in the int16 path: 64 cells * 2 B
@@ -69,8 +70,10 @@ constexpr int32_t kStTraced = 0x200;
 // PF_W128: the pair runs in 128-residue strips (four residues per lane; int16
 // only, never with PF_WIDE); otherwise in 64-residue strips
 // PF_PROF: the pair is a profile query (position-specific costs at prof_off)
+// PF_DUO: a warp runs two neighbouring 64-residue strips of the pair at once
+// (int16 only, never with PF_WIDE or PF_W128)
 enum : uint32_t {
-    PF_SCORE_ONLY = 1u, PF_BADSEQ = 2u, PF_SKIP = 4u, PF_BUDGET = 8u, PF_WIDE = 16u, PF_W128 = 32u, PF_PROF = 64u
+    PF_SCORE_ONLY = 1u, PF_BADSEQ = 2u, PF_SKIP = 4u, PF_BUDGET = 8u, PF_WIDE = 16u, PF_W128 = 32u, PF_PROF = 64u, PF_DUO = 128u
 };
 
 // Device copy of mp_profile_pos: position-specific substitution scores
@@ -105,7 +108,14 @@ struct ScoreParams {
 // boundary loads run up to a strip width + 2 chunks past the last row)
 constexpr int kCol0Pad = kStripWMax + 2 * kChunk + 2;
 
-// A work item is one strip (64 or 128 residues) of one pair: x = pair, y = strip.
+// work items of a pair of n_strips strips
+__host__ __device__ constexpr uint32_t items_of(uint32_t flags, uint32_t n_strips)
+{
+    return (flags & PF_DUO) ? (n_strips + 1) / 2 : n_strips;
+}
+
+// A work item is one strip (64 or 128 residues) of one pair, or two
+// neighbouring ones (PF_DUO): x = pair, y = strip (or pair of strips).
 // The warp running strip s consumes the boundary row strip s-1 publishes
 // chunk by chunk.
 struct DPArgs {
@@ -156,9 +166,9 @@ struct TBArgs {
 cudaError_t launch_pack(const PairDesc *pairs, uint32_t n, const char *ascii, uint8_t *prot,
                         uint32_t *nt2, PairOut *out, cudaStream_t st);
 cudaError_t launch_records(const PairDesc *pairs, uint32_t n, const uint32_t *nt2, const ScoreParams &sp, uint4 *recs,
-                           cudaStream_t st);
-// variant 0: the int16 DP kernel built for 3 CTAs per SM (80 registers per
-// thread); 1: built for 2 CTAs per SM (up to 128).  wide4: the 2-CTA build
+                           uint64_t *bnd, cudaStream_t st);
+// variant 0: the int16 DP kernel built with kWarpsPerCta warps per CTA (up to
+// 128 registers per thread); 1: with kWarps16 (up to 168).  wide4: the latter
 // that also runs PF_W128 pairs in 128-residue strips.  Same results.
 constexpr int kDp16Variants = 2;
 cudaError_t launch_dp16(const DPArgs &a, int grid, int variant, bool wide4, cudaStream_t st);
@@ -190,12 +200,11 @@ cudaError_t launch_col0(const PairDesc *pairs, uint32_t n, const uint32_t *nt2, 
 cudaError_t launch_compact(const PairDesc *pairs, PairOut *out, uint32_t n, const uint32_t *ops,
                            uint32_t *cig, uint32_t *total, cudaStream_t st);
 int dp16_blocks_per_sm(int variant, bool wide4 = false);
+int dp16_warps_per_cta(int variant, bool wide4);
 
 // the device and stream of a context (for the seeding and chaining calls)
 int ctx_device(const mp_dp_ctx *c);
 cudaStream_t ctx_stream(const mp_dp_ctx *c);
 int dp32_blocks_per_sm();
-size_t dp16_smem_bytes();
-size_t dp32_smem_bytes();
 
 }  // namespace mpdp

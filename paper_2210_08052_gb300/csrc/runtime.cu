@@ -595,9 +595,9 @@ static mp_dp_tuning default_tuning()
     t.dp16_variant = 1;
     t.overlap_waves = 1;
     t.item_order = 1;
-    // int16 kernel built for 2 CTAs/SM (no spill; with the tracebacks in the
-    // kernel it is the faster build on the 4,096-pair workload), all CTAs that
-    // fit, int16 first for wide pairs, overlapped waves, interleaved items
+    // int16 kernel built with 6-warp CTAs (10.55 ms per run of the 4,096-pair
+    // workload; with 4-warp CTAs of 255 registers 10.92, 5-warp 11.01), all CTAs
+    // that fit, int16 first for wide pairs, overlapped waves, interleaved items
     return t;
 }
 
@@ -639,24 +639,26 @@ static uint64_t plan_code_bytes(const mp_dp_ctx *c, const mp_dp_batch *b)
 // Order each wave's strip items so that a warp rarely takes a strip whose
 // predecessor has not yet published the boundary rows it starts with: pairs
 // in order (largest first), strip s+1 of a pair placed after strip s by
-// about as many items as the warps pop while the predecessor runs kLag = 2
-// chunks (the strips of a pair still run close together, so its per-nt
+// about as many items as the warps pop while the predecessor runs the chunks
+// it is ahead by (2, or 3 where a warp runs two strips; the strips of a pair still run close together, so its per-nt
 // records and boundary rows are read from L2).  PF_WIDE pairs' items stay a
 // prefix of the wave (the int32 queue may take them as a block).
 static void interleave_items(const mp_dp_ctx *c, mp_dp_batch *b)
 {
-    const double warps = static_cast<double>(c->num_sms) * 2 * kWarpsPerCta;
+    const double warps = static_cast<double>(c->num_sms) * 2 * kWarps16;
     std::vector<uint32_t> key, count;
     std::vector<uint2> out;
     auto segment = [&](uint32_t lo, uint32_t hi) {
         if (hi - lo < 2) return;
-        double chunks = 0;
+        double chunks = 0, lag = 0;
         for (uint32_t k = lo; k < hi; ++k)
         {
             const PairDesc &d = b->desc[b->h_items[k].x];
-            chunks += static_cast<double>((d.nt_len + strip_w_of(d.flags) - 1 + kChunk - 1) / kChunk);
+            const bool duo = (d.flags & PF_DUO) != 0;
+            chunks += static_cast<double>((d.nt_len + (duo ? 2 * kStripW : strip_w_of(d.flags)) - 1 + kChunk - 1) / kChunk);
+            lag += duo ? 3.0 : 2.0;
         }
-        const uint32_t D = static_cast<uint32_t>(std::max(1.0, std::round(2.0 * warps / (chunks / (hi - lo)))));
+        const uint32_t D = static_cast<uint32_t>(std::max(1.0, std::round(warps * lag / chunks)));
         // key = rank of the pair + D * strip; a stable counting sort by key
         key.resize(hi - lo);
         uint32_t rank = 0, top = 0;
@@ -723,12 +725,19 @@ static int plan_waves(mp_dp_ctx *c, mp_dp_batch *b, const mp_dp_tuning &t, bool 
     }
     for (uint32_t k = 0; k < n; ++k) {
         PairDesc &d = b->desc[k];
-        d.flags &= ~PF_W128;
+        d.flags &= ~(PF_W128 | PF_DUO);
         const uint64_t crit128 =
             div_up(d.nt_len + kStripWMax - 1, kChunk) + 3 * div_up(d.prot_len, kStripWMax);
         if (t.strip_width && !c->params.force_int32 && use_w128(d) && (t.strip_width == 2 || 2 * crit128 <= crit64))
             d.flags |= PF_W128;
         d.n_strips = static_cast<uint32_t>(div_up(d.prot_len, strip_w_of(d.flags)));
+        // two 64-residue strips per warp wherever there are two (a pair that may
+        // need int32 keeps one strip per item: its items can go to either kernel)
+        // (with the boundary rows withheld, a test of the waits, two strips stay
+        // apart, so that one of them waits)
+        const bool alone = d.n_strips == 2 && (c->params.debug_flags & MP_DEBUG_NO_PUBLISH);
+        if (!c->params.force_int32 && d.n_strips >= 2 && !alone && !(d.flags & (PF_WIDE | PF_W128 | PF_SKIP)))
+            d.flags |= PF_DUO;
     }
     for (uint32_t k = 0; k < n; ++k) {
         PairDesc &d = b->desc[k];
@@ -825,8 +834,9 @@ static int plan_waves(mp_dp_ctx *c, mp_dp_batch *b, const mp_dp_tuning &t, bool 
             b->bnd_bytes_total += static_cast<uint64_t>(d.n_strips > 0 ? d.n_strips - 1 : 0) * nch * kChunk *
                                   ((d.flags & PF_WIDE) ? 8 : 4);
         }
-        for (uint32_t s = 0; s < d.n_strips; ++s) b->h_items.push_back(make_uint2(p, s));
-        if (wide(p) == 0) nwide += d.n_strips;
+        const uint32_t items = items_of(d.flags, d.n_strips);
+        for (uint32_t s = 0; s < items; ++s) b->h_items.push_back(make_uint2(p, s));
+        if (wide(p) == 0) nwide += items;
     }
     b->item_off[n] = static_cast<uint32_t>(b->h_items.size());
     b->waves.push_back(Wave{wbeg, static_cast<uint32_t>(n), ibeg, static_cast<uint32_t>(b->h_items.size()), cur, nwide});
@@ -1185,7 +1195,7 @@ static int enqueue_pipeline(mp_dp_ctx *c, mp_dp_batch *b, cudaStream_t st, bool 
     CK(rec(0));
     CK(cudaMemsetAsync(state, 0, b->state_bytes, st));
     CK(launch_pack(b->d_desc.p, n, b->ascii.p, b->prot.p, b->nt2.p, b->out.p, st));
-    CK(launch_records(b->d_desc.p, n, b->nt2.p, c->sp, b->recs.p, st));
+    CK(launch_records(b->d_desc.p, n, b->nt2.p, c->sp, b->recs.p, b->bnd.p, st));
     launches += 2;
     const bool anchored = c->params.mode != MP_MODE_LOCAL;
     if (anchored) {
@@ -1246,7 +1256,7 @@ static int enqueue_pipeline(mp_dp_ctx *c, mp_dp_batch *b, cudaStream_t st, bool 
                 a1.n_items = b->item_off[k2] - b->item_off[k];
                 if (!a1.n_items) continue;
                 a1.head = counters + 8 * W + 8 + 4 * k;
-                const int grid = std::max(1, std::min<int>(c->num_sms, static_cast<int>((a1.n_items + kWarpsPerCta - 1) / kWarpsPerCta)));
+                const int grid = std::max(1, std::min<int>(c->num_sms, static_cast<int>(a1.n_items)));
                 if (c->params.force_int32) CK(launch_dp32(a1, grid, false, st));
                 else CK(launch_dp16(a1, grid, variant, wide4, st));
                 ++launches;
@@ -1266,9 +1276,14 @@ static int enqueue_pipeline(mp_dp_ctx *c, mp_dp_batch *b, cudaStream_t st, bool 
             a.items = b->items.p + wv.ibegin + skip;
             a.n_items = nitems - skip;
             a.head = counters + 8 * w;
-            const int want = static_cast<int>((a.n_items + kWarpsPerCta - 1) / kWarpsPerCta);
-            const int grid16 = std::max(1, std::min<int>(g16, want));
-            const int grid32 = std::max(1, std::min<int>(g32, want));
+            // a wave with fewer items than one CTA per SM holds warps spreads
+            // over the SMs (the kernel leaves the warps it does not need)
+            auto grid_for = [&](int full, int warps) {
+                const uint32_t one = static_cast<uint32_t>(c->num_sms) * static_cast<uint32_t>(warps);
+                return std::max(1, a.n_items <= one ? std::min<int>(c->num_sms, static_cast<int>(a.n_items)) : full);
+            };
+            const int grid16 = grid_for(g16, dp16_warps_per_cta(variant, wide4));
+            const int grid32 = grid_for(g32, kWarpsPerCta);
             if (c->params.force_int32) CK(launch_dp32(a, grid32, false, st));
             else CK(launch_dp16(a, grid16, variant, wide4, st));
             ++launches;
@@ -1416,7 +1431,7 @@ static std::vector<mp_dp_tuning> kernel_candidates(mp_dp_ctx *c, const mp_dp_bat
                 v.push_back(t);
             }
     }
-    // 128-residue strips (the 2-CTA build that runs both strip forms), for
+    // 128-residue strips (the build that runs every strip form), for
     // the pairs whose critical path allows it or for every eligible pair
     const int fitw = dp16_blocks_per_sm(1, true);
     for (int sw = 1; sw <= 2; ++sw)

@@ -33,6 +33,8 @@ struct PairView {
     const uint8_t *colmax;   // per strip, chunk and lane: the chunk's maximum H of the lane's cells
     int nchunks;
     bool w128;               // 128-residue strips (four cells per lane) instead of 64 (two)
+    int duo;                 // 1, 2: a warp ran two strips (2: the first strip alone); the upper one's
+                             // column maxima lie 64 steps behind its stream
     const uint32_t *g;       // packed genome
     const uint8_t *P;        // residue codes
     int n, m;
@@ -86,7 +88,15 @@ struct PairView {
             (t & 3) * 4));
         return static_cast<int>((r & 1) ? (w >> 16) : (w & 0xffffu)) - 32768;
     }
-    // maximum H over chunk c of residue j (steps c*kChunk .. c*kChunk+kChunk-1)
+    // step of residue j's row 0 in the chunks of its column maxima
+    __device__ __forceinline__ int cstep(int j) const
+    {
+        if (w128) return (j - 1) & 127;
+        const int s = (j - 1) >> 6;
+        return ((j - 1) & 63) + (duo && s > 0 && ((s ^ duo) & 1) == 0 ? 64 : 0);
+    }
+    // maximum H over chunk c of residue j (steps c*kChunk .. c*kChunk+kChunk-1;
+    // the last chunk's, every later step as well)
     __device__ __forceinline__ int cmax(int c, int j) const
     {
         if (w128) {
@@ -176,15 +186,16 @@ template <bool Coherent, typename Pred>
 __device__ __forceinline__ int scan_column(const PairView<Coherent> &v, int jc, int xhi, int thr, int lane, Pred pred)
 {
     if (xhi < 1 || jc < 1) return 0;
-    const int r = (jc - 1) & (v.w128 ? 127 : 63);
-    const int c_lo = r / kChunk, c_hi = (xhi - 1 + r) / kChunk;
+    const int r = v.cstep(jc), last = v.nchunks - 1;
+    const int c_lo = min(r / kChunk, last), c_hi = min((xhi - 1 + r) / kChunk, last);
     for (int cb = c_hi; cb >= c_lo; cb -= 32) {
         const int c = cb - lane;
         unsigned bal = __ballot_sync(kTbFull, c >= c_lo && v.cmax(c, jc) >= thr);
         while (bal) {
             const int cc = cb - (__ffs(bal) - 1);       // highest flagged chunk first
             bal &= bal - 1;
-            const int xa = max(1, cc * kChunk - r + 1), xb = min(xhi, cc * kChunk - r + kChunk);
+            const int xa = max(1, cc * kChunk - r + 1);
+            const int xb = cc == last ? xhi : min(xhi, cc * kChunk - r + kChunk);
             for (int x0 = xb; x0 >= xa; x0 -= 32) {
                 const int x = x0 - lane;
                 const unsigned hit = __ballot_sync(kTbFull, x >= xa && pred(x));
@@ -218,6 +229,7 @@ __device__ __forceinline__ PairView<Coherent> make_view(const TBArgs &a, const P
     const bool anchored = a.sp.mode != MP_MODE_LOCAL;
     return PairView<Coherent>{a.codes + pd.code_off, strip_bytes, wide,
                     a.codes + pd.code_off + static_cast<size_t>(pd.n_strips) * strip_bytes, nchunks, W == kStripWMax,
+                    (pd.flags & PF_DUO) ? 2 - static_cast<int>((pd.n_strips + 1) & 1) : 0,
                     a.nt2 + pd.nt_word_off, a.prot + pd.prot_off, n, static_cast<int>(pd.prot_len),
                     &a.sp, mat_s, anchored ? a.col0 + pd.col0_off : nullptr,
                     (pd.flags & PF_PROF) ? a.prof + pd.prof_off : nullptr,
