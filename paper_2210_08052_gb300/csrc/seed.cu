@@ -21,8 +21,8 @@
 // (strand, x = bin, y = residue), sorted; the recurrence of Eq. 2 with the
 // gap of Eq. 1 and the penalty of Eq. 3 (G = 200,000, beta = 0.75) in fixed
 // point with 16 fractional bits (the log term from a table of every |g| < G),
-// predecessors evaluated 32 at a time; then the chains in order of
-// decreasing score of their last anchor.
+// 32 anchors at a time, one per lane (see chain_dp); then the chains in order
+// of decreasing score of their last anchor.
 //
 // Second round, per (protein, region) pair: every 5-mer of the protein
 // (reduced alphabet, sorted in shared memory) against the 5-mer starting at
@@ -30,6 +30,8 @@
 // pair, contiguous base ranges per thread, so the anchors come out in (x, y)
 // order), counted then written; chained by one warp per pair with
 // g' = 3 dy - dx and Eq. 3.
+#include <algorithm>
+#include <climits>
 #include <cstdint>
 #include <cstring>
 #include <vector>
@@ -430,11 +432,13 @@ struct ChainArgs {
     uint64_t *anc;                // anchors
     int64_t *f;                   // chaining score per anchor
     int32_t *pred;                // predecessor per anchor (-1: none)
-    uint8_t *used;
+    uint8_t *mark;                // kNoStart, kTaken
+    int64_t *tmax;                // per 32 anchors of a protein: the largest f of one that may start a chain
     int top;
     mp_chain *chains;             // n_prot * top
     uint32_t *n_chains;
     const int32_t *log_tab;       // log terms of Eq. 3 for |g| < G
+    const uint32_t *order;        // proteins, those with most anchors first
 };
 
 __global__ void anchor_count_kernel(ChainArgs a, uint64_t *count)
@@ -525,115 +529,378 @@ __global__ void __launch_bounds__(kSortThreads) anchor_sort_kernel(ChainArgs a, 
     }
 }
 
+// an anchor that starts no chain (no predecessor, or one of no smaller f); one
+// that a chain has taken
+constexpr uint8_t kNoStart = 1, kTaken = 2;
+
 __device__ __forceinline__ int anc_strand(uint64_t v) { return static_cast<int>(v >> 63); }
 __device__ __forceinline__ int64_t anc_x(uint64_t v) { return static_cast<int64_t>((v >> 20) & 0x7fffffffffull); }
 __device__ __forceinline__ int64_t anc_y(uint64_t v) { return static_cast<int64_t>(v & 0xfffffu); }
 
-// One warp per protein: Eq. 2 over its sorted anchors, then its chains.
-__global__ void chain_kernel(ChainArgs a)
+// Eq. 2 over sorted anchors, 32 anchors at a time (a tile), one per lane.  A
+// lane keeps its anchor's best predecessor; every predecessor is read once per
+// tile and tried by all lanes (in ascending order, a later one only if
+// strictly better, so that the first of equal best ones stays).  Most tries
+// end at a bound that takes the penalty's log2(|g| + 1) down to its integer
+// part and so needs no table; only a link that may win looks its log term up.
+// Inside a tile the anchors depend on one another: the same bound with the
+// scores found so far shows which anchors of the tile any other can follow, a
+// few of the 32; only these are tried one by one.
+//
+// What bounds it: the tries' integer instructions (about 20 a try, some 50
+// tries per anchor on the 50 Mb workload) and, for the longest protein, the
+// tiles' chain of dependent loads.  With the predecessors spread over the
+// lanes and a 64-bit warp maximum per anchor (five rounds of four shuffles, in
+// series) 4,000 proteins took 80 ms.
+//
+// T: int32_t for proteins up to kMax32 residues (f is at most (m + 6) * 2^16;
+// links whose linear term alone passes every f are left out by the clamp of
+// |g|), else int64_t.
+constexpr int64_t kMax32 = 32000;
+constexpr int32_t kClamp32 = 98000;          // kClamp32 * 21845 is just below 2^31, above every 32-bit f
+constexpr int32_t kBits = 3 * static_cast<int32_t>(kScale) / 4;      // beta in units of 2^-16: one bit of |g| + 1
+
+struct TileAnchor {
+    uint32_t x;
+    int32_t y;
+};
+
+// First round: x a bin, the strand in bit 30; the gap of Eq. 1.  reach: from
+// this many bins on |g| >= G (dx is clamped to it; the other strand's anchors
+// are further).
+struct BinGeo {
+    static constexpr int K = kK;
+    uint32_t reach;
+    __device__ __forceinline__ explicit BinGeo(int64_t m) : reach(static_cast<uint32_t>((kG + 3 * m) / kBin + 2)) {}
+    static __device__ __forceinline__ TileAnchor anchor(uint64_t v)
+    {
+        return TileAnchor{static_cast<uint32_t>((v >> 20) & 0x3fffffffu) | static_cast<uint32_t>(v >> 63) << 30,
+                          static_cast<int32_t>(v & 0xfffffu)};
+    }
+    __device__ __forceinline__ int32_t gap(uint32_t dx, int32_t dy) const
+    {
+        const int32_t d = static_cast<int32_t>(dx < reach ? dx : reach) * kBin, py = 3 * dy;
+        return py - min(max(py, d - kBin), d + kBin);
+    }
+};
+
+// Second round: x a base of the region; g' = 3 dy - dx.
+struct BaseGeo {
+    static constexpr int K = 5;
+    uint32_t reach;
+    __device__ __forceinline__ explicit BaseGeo(int64_t m) : reach(static_cast<uint32_t>(kG + 3 * m)) {}
+    static __device__ __forceinline__ TileAnchor anchor(uint64_t v)
+    {
+        return TileAnchor{static_cast<uint32_t>(v >> 20), static_cast<int32_t>(v & 0xfffffu)};
+    }
+    __device__ __forceinline__ int32_t gap(uint32_t dx, int32_t dy) const
+    {
+        return 3 * dy - static_cast<int32_t>(dx < reach ? dx : reach);
+    }
+};
+
+// the largest value of the lanes
+__device__ __forceinline__ int32_t warp_max(int32_t v) { return __reduce_max_sync(0xffffffffu, v); }
+__device__ __forceinline__ int64_t warp_max(int64_t v)
 {
-    const int lane = threadIdx.x & 31;
-    const int64_t S = kScale;
-    for (uint32_t p = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; p < a.n_prot; p += (gridDim.x * blockDim.x) >> 5) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const int64_t ov = __shfl_xor_sync(0xffffffffu, v, o);
+        v = ov > v ? ov : v;
+    }
+    return v;
+}
+
+// the largest value of the lanes, the first index among equals
+__device__ __forceinline__ void warp_first_max(int64_t &v, int64_t &i)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const int64_t ov = __shfl_xor_sync(0xffffffffu, v, o);
+        const int64_t oi = __shfl_xor_sync(0xffffffffu, i, o);
+        if (ov > v || (ov == v && oi < i)) {
+            v = ov;
+            i = oi;
+        }
+    }
+}
+
+// One lane's anchor and its best predecessor so far.
+template <typename T, typename Geo>
+struct Seeker {
+    Geo geo;
+    TileAnchor t;
+    T best;
+    int32_t arg = -1;
+    bool gains = false;                      // best is above the predecessor's f
+    static constexpr T kFirst = static_cast<T>(Geo::K) * static_cast<T>(kScale);
+
+    __device__ __forceinline__ Seeker(const Geo &g, const TileAnchor &a) : geo(g), t(a), best(kFirst) {}
+
+    // Whether an anchor at (x, y) with score f may be a better predecessor.
+    // A link is worth at most K less the penalty, and the penalty at least
+    // one kBits per bit of |g| + 1 above the first (less only for |g| <= 6, by
+    // the linear term, which always passes here).
+    __device__ __forceinline__ bool may(uint32_t x, int32_t y, T f, int32_t &g, int32_t &dy) const
+    {
+        dy = t.y - y;
+        g = geo.gap(t.x - x, dy);
+        const T slack = f + kFirst - best, top = static_cast<T>(INT_MAX);
+        const uint32_t s = static_cast<uint32_t>(max(min(slack, top), static_cast<T>(0)));
+        const uint32_t bits = max(__umulhi(s, 87382u) + 1u, 3u);             // floor(s / kBits) + 1, or one more
+        return dy > 0 && __funnelshift_rc(static_cast<uint32_t>(abs(g)) + 1u, 0u, bits) == 0;
+    }
+    // The same with the linear term: the link's worth is at most `up`
+    __device__ __forceinline__ bool may_win(T f, int32_t g, int32_t dy) const
+    {
+        const int32_t a = abs(g);
+        const int32_t l2 = (31 - __clz(a + 1)) * kBits;
+        const T lin = static_cast<T>(sizeof(T) == 4 ? min(a, kClamp32) : a) * 21845;        // 65536 = 3 * 21845 + 1
+        const T low = g < 0 ? (lin < static_cast<T>(l2) ? lin : static_cast<T>(l2)) : lin + static_cast<T>(l2);
+        // (32 bits: f is positive and the rest above -2^31)
+        return a < static_cast<int32_t>(kG) && f + (static_cast<T>(min(dy, Geo::K)) * static_cast<T>(kScale) - low) > best;
+    }
+    __device__ __forceinline__ void try_link(uint32_t x, int32_t y, T f, int32_t i, const int32_t *lt)
+    {
+        int32_t g, dy;
+        if (may(x, y, f, g, dy) && may_win(f, g, dy)) {
+            const int64_t c = static_cast<int64_t>(f) + static_cast<int64_t>(min(dy, Geo::K)) * kScale - penalty_eq3(g, lt);
+            if (c > static_cast<int64_t>(best)) {
+                best = static_cast<T>(c);
+                arg = i;
+                gains = c > static_cast<int64_t>(f);
+            }
+        }
+    }
+};
+
+// Shared memory of chain_dp: the predecessors at hand, per warp, and what the
+// other warps found for the tile's anchors.
+template <int NW>
+struct ChainSmem {
+    int4 stage[NW][32];
+    int64_t best[NW][32];
+    int32_t arg[NW][32];                     // predecessor, its bit 31 flipped if best is above its f
+    unsigned from[NW][32];
+};
+
+// The anchors [0, n) of A by NW warps of a block (0 .. NW-1, which meet at
+// barrier `bar`; with one, nothing but that warp takes part), which share out
+// a tile's tries.  done(j0, j, have, seeker): called by warp 0 for every tile.
+template <typename T, typename Geo, int NW, typename Done>
+__device__ void chain_dp(const uint64_t *A, int64_t n, const Geo &geo, const int32_t *lt, int64_t *F, int32_t *Pr,
+                         ChainSmem<NW> &sm, int bar, int warp, int lane, Done done)
+{
+    auto meet = [&] {
+        if (NW == 1) __syncwarp();
+        else asm volatile("bar.sync %0, %1;" ::"r"(bar), "n"(NW * 32) : "memory");
+    };
+    int4 *stage = sm.stage[warp];
+    auto put = [&](const TileAnchor &u, int64_t f) {
+        stage[lane] = make_int4(static_cast<int>(u.x), u.y, static_cast<int>(f), static_cast<int>(f >> 32));
+    };
+    auto f_of = [](const int4 &u) {
+        return sizeof(T) == 4 ? static_cast<T>(u.z)
+                              : static_cast<T>(static_cast<int64_t>(u.w) << 32 | static_cast<uint32_t>(u.z));
+    };
+    int64_t lo = 0;
+    uint64_t next = A[lane < n ? lane : n - 1];
+    for (int64_t j0 = 0; j0 < n; j0 += 32) {
+        const int64_t j = j0 + lane;
+        const bool have = j < n;
+        Seeker<T, Geo> me(geo, Geo::anchor(next));
+        next = A[j + 32 < n ? j + 32 : n - 1];         // the next tile's, on its way
+        // the window of the tile's first anchor holds every lane's
+        const uint32_t x0 = __shfl_sync(0xffffffffu, me.t.x, 0);
+        for (;;) {
+            const int64_t i = lo + lane;
+            const bool far = i < j0 && x0 - Geo::anchor(A[i]).x > geo.reach;
+            const unsigned near = __ballot_sync(0xffffffffu, !far);
+            lo += near ? __ffs(near) - 1 : 32;
+            if (near) break;
+        }
+        for (int64_t i0 = lo + 32 * warp; i0 < j0; i0 += 32 * NW) {
+            const int cnt = static_cast<int>(j0 - i0 < 32 ? j0 - i0 : 32);
+            __syncwarp();
+            if (lane < cnt) put(Geo::anchor(A[i0 + lane]), F[i0 + lane]);
+            __syncwarp();
+#pragma unroll 4
+            for (int k = 0; k < cnt; ++k) {
+                const int4 u = stage[k];
+                me.try_link(static_cast<uint32_t>(u.x), u.y, f_of(u), static_cast<int32_t>(i0) + k, lt);
+            }
+        }
+        if (NW > 1) {
+            // the largest of the warps, the first predecessor among equals
+            sm.best[warp][lane] = static_cast<int64_t>(me.best);
+            sm.arg[warp][lane] = me.gains ? me.arg ^ INT_MIN : me.arg;
+            meet();
+#pragma unroll
+            for (int w = 0; w < NW; ++w) {
+                const T b = static_cast<T>(sm.best[w][lane]);
+                const int32_t r = sm.arg[w][lane];
+                const bool gains = r < -1;
+                const int32_t i = gains ? r ^ INT_MIN : r;
+                if (b > me.best || (b == me.best && i >= 0 && me.arg >= 0 && i < me.arg)) {
+                    me.best = b;
+                    me.arg = i;
+                    me.gains = gains;
+                }
+            }
+        }
+        // inside the tile: which anchors can any other follow?
+        __syncwarp();
+        put(me.t, static_cast<int64_t>(me.best));
+        __syncwarp();
+        const int cnt = static_cast<int>(n - j0 < 32 ? n - j0 : 32);
+        unsigned from = 0;                                 // anchors this lane's may follow
+#pragma unroll 4
+        for (int k = warp; k < cnt - 1; k += NW) {
+            const int4 u = stage[k];
+            int32_t g, dy;
+            if (me.may(static_cast<uint32_t>(u.x), u.y, f_of(u), g, dy) && k < lane && me.may_win(f_of(u), g, dy))
+                from |= 1u << k;
+        }
+        if (NW > 1) {
+            sm.from[warp][lane] = from;
+            meet();
+        }
+        if (warp == 0) {
+#pragma unroll
+            for (int w = 1; w < NW; ++w) from |= sm.from[w][lane];
+            // the anchors that any other may follow, in ascending order; one that
+            // gains joins them (a test that failed with a lower score and an
+            // unchanged one of the other anchor keeps failing)
+            unsigned todo = __reduce_or_sync(0xffffffffu, have ? from : 0u);
+            while (todo) {
+                const int k = __ffs(todo) - 1;
+                todo &= todo - 1;
+                const uint32_t xi = __shfl_sync(0xffffffffu, me.t.x, k);
+                const int32_t yi = __shfl_sync(0xffffffffu, me.t.y, k);
+                const T fi = __shfl_sync(0xffffffffu, me.best, k);
+                const T was = me.best;
+                if (lane > k) me.try_link(xi, yi, fi, static_cast<int32_t>(j0) + k, lt);
+                todo |= __ballot_sync(0xffffffffu, have && me.best != was);
+            }
+            if (have) {
+                F[j] = static_cast<int64_t>(me.best);
+                Pr[j] = me.arg;
+            }
+            done(j0, j, have, me);
+        }
+        meet();                                            // F is read by the next tiles
+    }
+}
+
+// One block per protein, the ones with most anchors first: Eq. 2 over its
+// sorted anchors, kStrandWarps warps per strand (chains stay on one; the
+// longest protein's tiles are a chain of their own), then its chains.
+//
+// Chains are taken in order of decreasing f of the last anchor (ties: the
+// earlier anchor), each cut at an anchor already taken, and single anchors
+// are dropped, which takes them too.  An anchor whose predecessor has no
+// smaller f comes after it in that order and so is always alone; the walk of a
+// chain from b stops at an anchor of an earlier chain or one that precedes b
+// in the order.  So only anchors above their predecessor's f are looked at,
+// and no single one is ever taken by itself: near a long chain thousands
+// follow it at a loss, and with a look at every anchor before each of them one
+// protein of 4,000 took 20 ms.  The best is found from the largest f of each
+// tile; a tile whose largest is out of date is seen when it is looked at.
+__device__ __forceinline__ uint64_t tile_base(uint64_t b0, uint32_t p) { return b0 / 32 + 2ull * p; }    // in ChainArgs::tmax
+
+constexpr int kStrandWarps = 4;
+__global__ void __launch_bounds__(kStrandWarps * 64) chain_kernel(ChainArgs a)
+{
+    __shared__ ChainSmem<kStrandWarps> sm[2];
+    const int lane = threadIdx.x & 31, strand = threadIdx.x / (kStrandWarps * 32);
+    const int warp = (threadIdx.x >> 5) % kStrandWarps;
+    for (uint32_t k = blockIdx.x; k < a.n_prot; k += gridDim.x) {
+        const uint32_t p = a.order[k];
         const uint64_t b0 = a.anc_off[p];
         const int64_t n = static_cast<int64_t>(a.anc_off[p + 1] - b0);
         const uint64_t *A = a.anc + b0;
         int64_t *F = a.f + b0;
         int32_t *Pr = a.pred + b0;
-        uint8_t *U = a.used + b0;
+        uint8_t *U = a.mark + b0;
         const int64_t m = a.prot_len[p];
-        // predecessors further than this many bins have |g| >= G
-        const int64_t wbins = (kG + 3 * m) / kBin + 2;
-        int64_t lo = 0;
-        for (int64_t j = 0; j < n; ++j) {
-            const uint64_t vj = A[j];
-            const int sj = anc_strand(vj);
-            const int64_t xj = anc_x(vj), yj = anc_y(vj);
-            while (lo < j && (anc_strand(A[lo]) != sj || anc_x(A[lo]) < xj - wbins)) ++lo;
-            int64_t best = static_cast<int64_t>(kK) * S;
-            int64_t arg = -1;
-            for (int64_t i0 = lo; i0 < j; i0 += 32) {
-                const int64_t i = i0 + lane;
-                int64_t cand = INT64_MIN;
-                if (i < j) {
-                    const uint64_t vi = A[i];
-                    const int64_t dy = yj - anc_y(vi);
-                    if (anc_strand(vi) == sj && anc_x(vi) <= xj && dy > 0) {
-                        const int64_t pen = penalty_eq3(gap_eq1(xj - anc_x(vi), dy), a.log_tab);
-                        if (pen >= 0) cand = F[i] + (dy < kK ? dy : kK) * S - pen;
-                    }
-                }
-                // the largest candidate, the first index among equals
-                int64_t c = cand, ci = i;
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    const int64_t oc = __shfl_xor_sync(0xffffffffu, c, o);
-                    const int64_t oi = __shfl_xor_sync(0xffffffffu, ci, o);
-                    if (oc > c || (oc == c && oi < ci)) {
-                        c = oc;
-                        ci = oi;
-                    }
-                }
-                if (c > best) {
-                    best = c;
-                    arg = ci;
-                }
-            }
-            if (lane == 0) {
-                F[j] = best;
-                Pr[j] = static_cast<int32_t>(arg);
-                U[j] = 0;
-            }
-            __syncwarp();
+        int64_t *tmax = a.tmax + tile_base(b0, p);
+        // the first anchor of strand 1: 31 probes at a time
+        int64_t s0 = 0, s1 = n;                            // strand 0 below s0, strand 1 from s1 on
+        while (s0 < s1) {
+            const int64_t step = (s1 - s0 + 31) / 32, at = s0 + step * lane;
+            const unsigned zero = __ballot_sync(0xffffffffu, at < s1 && anc_strand(A[at]) == 0);
+            const int c = __popc(zero);                    // probes on strand 0, the first ones
+            if (c < 32 && s0 + step * c < s1) s1 = s0 + step * c;
+            if (c) s0 = s0 + step * (c - 1) + 1;
         }
-        // chains in order of decreasing f of the last anchor (ties: the earlier
-        // anchor), each cut at an anchor already used; single anchors dropped;
-        // once the best unused anchor starts no chain (f = k), none follows
+        const int64_t split = s0, nt0 = (split + 31) / 32, nt = nt0 + (n - split + 31) / 32;
+        {
+            const int64_t from = strand ? split : 0, cnt = strand ? n - split : split;
+            int64_t *tm = tmax + (strand ? nt0 : 0);
+            uint8_t *Us = U + from;
+            // (predecessors are numbered from the strand's first anchor)
+            auto run = [&](auto zero) {
+                using T = decltype(zero);
+                chain_dp<T, BinGeo, kStrandWarps>(
+                    A + from, cnt, BinGeo(m), a.log_tab, F + from, Pr + from, sm[strand], 1 + strand, warp, lane,
+                    [&](int64_t j0, int64_t j, bool have, const Seeker<T, BinGeo> &me) {
+                        if (have) Us[j] = me.gains ? 0 : kNoStart;
+                        const T top = warp_max(have && me.gains ? me.best : static_cast<T>(0));
+                        if (lane == 0) tm[j0 >> 5] = static_cast<int64_t>(top);
+                    });
+            };
+            if (cnt > 0) {
+                if (m <= kMax32) run(static_cast<int32_t>(0));
+                else run(static_cast<int64_t>(0));
+            }
+        }
+        __syncthreads();
+        if (strand || warp) continue;
         int nc = 0;
         while (nc < a.top) {
-            int64_t bf = INT64_MIN, bi = -1;
-            for (int64_t i0 = 0; i0 < n; i0 += 32) {
-                const int64_t i = i0 + lane;
-                int64_t v = INT64_MIN, vi = i;
-                if (i < n && !U[i]) v = F[i];
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    const int64_t ov = __shfl_xor_sync(0xffffffffu, v, o);
-                    const int64_t oi = __shfl_xor_sync(0xffffffffu, vi, o);
-                    if (ov > v || (ov == v && oi < vi)) {
-                        v = ov;
-                        vi = oi;
-                    }
-                }
-                if (v > bf || (v == bf && vi < bi)) {
-                    bf = v;
-                    bi = vi;
+            // each lane the first best of its own tiles, then the warp's
+            int64_t bf = INT64_MIN, bt = INT64_MAX;
+#pragma unroll 4
+            for (int64_t t = lane; t < nt; t += 32) {
+                const int64_t f = tmax[t];
+                if (f > bf) {
+                    bf = f;
+                    bt = t;
                 }
             }
-            if (bi < 0 || bf <= static_cast<int64_t>(kK) * S) break;
-            if (lane == 0) {
-                int64_t cnt = 0, cur = bi, first = bi, stop = -1;
-                while (cur >= 0 && !U[cur]) {
-                    U[cur] = 1;
-                    first = cur;
-                    ++cnt;
-                    cur = Pr[cur];
-                }
-                if (cur >= 0) stop = cur;
-                if (cnt >= 2) {
-                    mp_chain &c = a.chains[static_cast<uint64_t>(p) * a.top + nc];
-                    c.strand = anc_strand(A[bi]);
-                    c.n_anchors = static_cast<int32_t>(cnt);
-                    c.score = F[bi] - (stop >= 0 ? F[stop] : 0);
-                    c.x_first = anc_x(A[first]);
-                    c.x_last = anc_x(A[bi]);
-                    c.y_first = anc_y(A[first]);
-                    c.y_last = anc_y(A[bi]);
-                }
-                nc += cnt >= 2 ? 1 : 0;
+            warp_first_max(bf, bt);
+            if (bf <= static_cast<int64_t>(kK) * kScale) break;
+            const int64_t base = bt < nt0 ? 0 : split;     // of the strand
+            const int64_t at = bt < nt0 ? bt * 32 + lane : split + (bt - nt0) * 32 + lane;
+            int64_t f = 0;
+            if (at < (bt < nt0 ? split : n) && U[at] == 0 && !(U[base + Pr[at]] & kTaken)) f = F[at];
+            const int64_t best = warp_max(f);
+            if (best < bf) {
+                // some of the tile's were taken, or their predecessors were
+                if (lane == 0) tmax[bt] = best;
+                __syncwarp();
+                continue;
             }
-            nc = __shfl_sync(0xffffffffu, nc, 0);
+            const int64_t bi = at - lane + __ffs(__ballot_sync(0xffffffffu, f == bf)) - 1;
+            int64_t cnt = 0, cur = bi, first = bi;
+            do {
+                if (lane == 0) U[cur] |= kTaken;
+                first = cur;
+                ++cnt;
+                cur = Pr[cur] < 0 ? -1 : base + Pr[cur];
+            } while (cur >= 0 && !(U[cur] & kTaken) && F[cur] < bf);
             __syncwarp();
+            if (lane == 0) {
+                mp_chain &c = a.chains[static_cast<uint64_t>(p) * a.top + nc];
+                c.strand = anc_strand(A[bi]);
+                c.n_anchors = static_cast<int32_t>(cnt);
+                c.score = bf - (cur >= 0 ? F[cur] : 0);
+                c.x_first = anc_x(A[first]);
+                c.x_last = anc_x(A[bi]);
+                c.y_first = anc_y(A[first]);
+                c.y_last = anc_y(A[bi]);
+            }
+            ++nc;
         }
         if (lane == 0) a.n_chains[p] = static_cast<uint32_t>(nc);
     }
@@ -773,86 +1040,6 @@ __global__ void __launch_bounds__(kRefineThreads) refine_anchor_kernel(RefineArg
     }
 }
 
-// One warp per pair: f of every anchor with g' = 3 dy - dx, then the best chain.
-__global__ void refine_chain_kernel(RefineArgs a)
-{
-    const int lane = threadIdx.x & 31;
-    const int64_t S = kScale;
-    for (uint32_t p = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; p < a.n; p += (gridDim.x * blockDim.x) >> 5) {
-        const uint64_t b0 = a.anc_off[p];
-        const int64_t n = static_cast<int64_t>(a.anc_off[p + 1] - b0);
-        if (n > kRefineBig) continue;               // refine_chain_block_kernel's
-        const uint64_t *A = a.anc + b0;
-        int64_t *F = a.f + b0;
-        int32_t *Pr = a.pred + b0;
-        // predecessors more than G + 3m bases back have g' <= -G
-        const int64_t wx = kG + 3 * static_cast<int64_t>(a.prot_len[p]);
-        int64_t lo = 0, bf = INT64_MIN, bi = -1;
-        for (int64_t j = 0; j < n; ++j) {
-            const int64_t xj = static_cast<int64_t>(A[j] >> 20), yj = static_cast<int64_t>(A[j] & 0xfffffu);
-            while (lo < j && static_cast<int64_t>(A[lo] >> 20) < xj - wx) ++lo;
-            int64_t best = static_cast<int64_t>(kK2) * S;
-            int64_t arg = -1;
-            for (int64_t i0 = lo; i0 < j; i0 += 32) {
-                const int64_t i = i0 + lane;
-                int64_t cand = INT64_MIN;
-                if (i < j) {
-                    const uint64_t vi = A[i];
-                    const int64_t dx = xj - static_cast<int64_t>(vi >> 20);
-                    const int64_t dy = yj - static_cast<int64_t>(vi & 0xfffffu);
-                    if (dx >= 0 && dy > 0) {
-                        const int64_t pen = penalty_eq3(3 * dy - dx, a.log_tab);
-                        if (pen >= 0) cand = F[i] + (dy < kK2 ? dy : kK2) * S - pen;
-                    }
-                }
-                // the largest candidate, the first index among equals
-                int64_t cv = cand, ci = i;
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    const int64_t oc = __shfl_xor_sync(0xffffffffu, cv, o);
-                    const int64_t oi = __shfl_xor_sync(0xffffffffu, ci, o);
-                    if (oc > cv || (oc == cv && oi < ci)) {
-                        cv = oc;
-                        ci = oi;
-                    }
-                }
-                if (cv > best) {
-                    best = cv;
-                    arg = ci;
-                }
-            }
-            if (lane == 0) {
-                F[j] = best;
-                Pr[j] = static_cast<int32_t>(arg);
-            }
-            if (best > bf) {                    // the first anchor with the largest f
-                bf = best;
-                bi = j;
-            }
-            __syncwarp();
-        }
-        if (lane == 0) {
-            mp_chain2 c{};
-            if (bi >= 0 && Pr[bi] >= 0) {
-                int64_t cnt = 0, cur = bi, first = bi;
-                while (cur >= 0) {
-                    first = cur;
-                    ++cnt;
-                    cur = Pr[cur];
-                }
-                c.n_anchors = static_cast<int32_t>(cnt);
-                c.score = F[bi];
-                c.x_first = static_cast<int64_t>(A[first] >> 20);
-                c.x_last = static_cast<int64_t>(A[bi] >> 20);
-                c.y_first = static_cast<int64_t>(A[first] & 0xfffffu);
-                c.y_last = static_cast<int64_t>(A[bi] & 0xfffffu);
-            }
-            a.out[p] = c;
-        }
-        __syncwarp();
-    }
-}
-
 // The pair's best chain from f and the predecessors (one thread).
 __device__ __forceinline__ mp_chain2 best_chain(const uint64_t *A, const int64_t *F, const int32_t *Pr, int64_t bi)
 {
@@ -874,77 +1061,54 @@ __device__ __forceinline__ mp_chain2 best_chain(const uint64_t *A, const int64_t
     return c;
 }
 
-// The same recurrence for the pairs with more than kRefineBig anchors, one
-// block per pair: each anchor's predecessors split over the block's
-// threads, the best (largest, then first) found by a block reduction.
+// f of every anchor of pair p with g' = 3 dy - dx by NW warps, then the best
+// chain (the first anchor with the largest f and its predecessors).
+template <int NW>
+__device__ __forceinline__ void refine_pair(const RefineArgs &a, uint32_t p, ChainSmem<NW> &sm, int warp, int lane)
+{
+    const uint64_t b0 = a.anc_off[p];
+    const int64_t n = static_cast<int64_t>(a.anc_off[p + 1] - b0);
+    const uint64_t *A = a.anc + b0;
+    int64_t *F = a.f + b0;
+    int32_t *Pr = a.pred + b0;
+    int64_t bf = INT64_MIN, bi = INT64_MAX;             // this lane's first best anchor
+    // (proteins have at most kRefineMaxProt residues: 32-bit scores)
+    if (n > 0)
+        chain_dp<int32_t, BaseGeo, NW>(A, n, BaseGeo(a.prot_len[p]), a.log_tab, F, Pr, sm, 0, warp, lane,
+                                       [&](int64_t, int64_t j, bool have, const Seeker<int32_t, BaseGeo> &me) {
+                                           if (have && me.best > bf) {
+                                               bf = me.best;
+                                               bi = j;
+                                           }
+                                       });
+    if (warp == 0) {
+        warp_first_max(bf, bi);
+        if (lane == 0) a.out[p] = best_chain(A, F, Pr, n > 0 ? bi : -1);
+    }
+}
+
+// One warp per pair.
+constexpr int kRefineWarps = 4;
+__global__ void __launch_bounds__(kRefineWarps * 32) refine_chain_kernel(RefineArgs a)
+{
+    __shared__ ChainSmem<1> sm[kRefineWarps];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (uint32_t p = blockIdx.x * kRefineWarps + warp; p < a.n; p += gridDim.x * kRefineWarps)
+        if (static_cast<int64_t>(a.anc_off[p + 1] - a.anc_off[p]) <= kRefineBig) refine_pair<1>(a, p, sm[warp], 0, lane);
+}
+
+// One block per pair with more than kRefineBig anchors: every earlier anchor
+// of a region is within reach, so the tries grow with the square of their
+// number, and the warps share each tile's out.
 __global__ void __launch_bounds__(kRefineThreads) refine_chain_block_kernel(RefineArgs a)
 {
-    __shared__ int64_t rv[kRefineThreads / 32];
-    __shared__ int64_t ri[kRefineThreads / 32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t S = kScale;
-    for (uint32_t p = blockIdx.x; p < a.n; p += gridDim.x) {
-        const uint64_t b0 = a.anc_off[p];
-        const int64_t n = static_cast<int64_t>(a.anc_off[p + 1] - b0);
-        if (n <= kRefineBig) continue;              // uniform across the block
-        const uint64_t *A = a.anc + b0;
-        int64_t *F = a.f + b0;
-        int32_t *Pr = a.pred + b0;
-        const int64_t wx = kG + 3 * static_cast<int64_t>(a.prot_len[p]);
-        int64_t lo = 0, bf = INT64_MIN, bi = -1;
-        for (int64_t j = 0; j < n; ++j) {
-            const int64_t xj = static_cast<int64_t>(A[j] >> 20), yj = static_cast<int64_t>(A[j] & 0xfffffu);
-            while (lo < j && static_cast<int64_t>(A[lo] >> 20) < xj - wx) ++lo;
-            int64_t cv = INT64_MIN, ci = INT64_MAX;
-            for (int64_t i = lo + threadIdx.x; i < j; i += blockDim.x) {
-                const uint64_t vi = A[i];
-                const int64_t dx = xj - static_cast<int64_t>(vi >> 20);
-                const int64_t dy = yj - static_cast<int64_t>(vi & 0xfffffu);
-                if (dx >= 0 && dy > 0) {
-                    const int64_t pen = penalty_eq3(3 * dy - dx, a.log_tab);
-                    if (pen >= 0) {
-                        const int64_t cand = F[i] + (dy < kK2 ? dy : kK2) * S - pen;
-                        if (cand > cv) {            // i ascends: the first of equals stays
-                            cv = cand;
-                            ci = i;
-                        }
-                    }
-                }
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const int64_t oc = __shfl_xor_sync(0xffffffffu, cv, o);
-                const int64_t oi = __shfl_xor_sync(0xffffffffu, ci, o);
-                if (oc > cv || (oc == cv && oi < ci)) {
-                    cv = oc;
-                    ci = oi;
-                }
-            }
-            if (lane == 0) {
-                rv[warp] = cv;
-                ri[warp] = ci;
-            }
+    constexpr int NW = kRefineThreads / 32;
+    __shared__ ChainSmem<NW> sm;
+    for (uint32_t p = blockIdx.x; p < a.n; p += gridDim.x)
+        if (static_cast<int64_t>(a.anc_off[p + 1] - a.anc_off[p]) > kRefineBig) {       // uniform across the block
+            refine_pair<NW>(a, p, sm, threadIdx.x >> 5, threadIdx.x & 31);
             __syncthreads();
-            if (threadIdx.x == 0) {
-                int64_t best = static_cast<int64_t>(kK2) * S, arg = -1;
-                for (int w = 0; w < static_cast<int>(blockDim.x >> 5); ++w) {
-                    if (rv[w] > best || (rv[w] == best && arg >= 0 && ri[w] < arg)) {
-                        best = rv[w];
-                        arg = ri[w];
-                    }
-                }
-                F[j] = best;
-                Pr[j] = static_cast<int32_t>(arg);
-                if (best > bf) {
-                    bf = best;
-                    bi = j;
-                }
-            }
-            __syncthreads();                        // F[j] is read by the next anchors
         }
-        if (threadIdx.x == 0) a.out[p] = best_chain(A, F, Pr, bi);
-        __syncthreads();
-    }
 }
 
 }  // namespace
@@ -1160,6 +1324,10 @@ extern "C" int mp_index_chain(mp_dp_ctx *ctx, const mp_index *idx, const char *p
         while (p1 < n_prot && (p1 == p0 || tot + cnt[p1] <= kMaxAnchors)) tot += cnt[p1++];
         const uint32_t np = p1 - p0;
         std::vector<uint64_t> aoff(np + 1ull, 0), soff(np, 0);
+        std::vector<uint32_t> order(np);
+        for (uint32_t k = 0; k < np; ++k) order[k] = k;
+        std::stable_sort(order.begin(), order.end(),
+                         [&](uint32_t x, uint32_t y) { return cnt[p0 + x] > cnt[p0 + y]; });
         uint64_t scratch = 0;
         for (uint32_t k = 0; k < np; ++k) {
             aoff[k + 1] = aoff[k] + cnt[p0 + k];
@@ -1171,11 +1339,16 @@ extern "C" int mp_index_chain(mp_dp_ctx *ctx, const mp_index *idx, const char *p
         Tmp<uint64_t> anc, sc, d_soff;
         Tmp<int64_t> f;
         Tmp<int32_t> pred;
-        Tmp<uint8_t> used;
+        Tmp<uint8_t> mark;
+        Tmp<int64_t> tmax;
+        Tmp<uint32_t> d_order;
+        SCK(d_order.alloc(np));
+        SCK(cudaMemcpyAsync(d_order.p, order.data(), np * sizeof(uint32_t), cudaMemcpyHostToDevice, st));
+        SCK(tmax.alloc(tot / 32 + 2ull * np + 2));
         SCK(anc.alloc(tot));
         SCK(f.alloc(tot));
         SCK(pred.alloc(tot));
-        SCK(used.alloc(tot));
+        SCK(mark.alloc(tot));
         SCK(sc.alloc(scratch));
         SCK(d_soff.alloc(np));
         SCK(cudaMemcpyAsync(d_anc_off.p, aoff.data(), (np + 1ull) * sizeof(uint64_t), cudaMemcpyHostToDevice, st));
@@ -1188,13 +1361,15 @@ extern "C" int mp_index_chain(mp_dp_ctx *ctx, const mp_index *idx, const char *p
         b.anc = anc.p;
         b.f = f.p;
         b.pred = pred.p;
-        b.used = used.p;
+        b.mark = mark.p;
+        b.tmax = tmax.p;
+        b.order = d_order.p;
         b.chains = d_ch.p + static_cast<uint64_t>(p0) * top;
         b.n_chains = d_nch.p + p0;
         anchor_fill_kernel<<<grid_for(np * 32ull, 256), 256, 0, st>>>(b);
         anchor_sort_kernel<<<np < 65535u * 4 ? np : 65535u * 4, kSortThreads, kSortMax * sizeof(uint64_t), st>>>(
             b, sc.p, d_soff.p);
-        chain_kernel<<<grid_for(np * 32ull, 128), 128, 0, st>>>(b);
+        chain_kernel<<<np < 65535u * 16 ? np : 65535u * 16, kStrandWarps * 64, 0, st>>>(b);
         SCK(cudaGetLastError());
         SCK(cudaStreamSynchronize(st));
         p0 = p1;
@@ -1317,7 +1492,7 @@ extern "C" int mp_chain_refine(mp_dp_ctx *ctx, const mp_pair *pairs, size_t n, m
         const uint32_t gb = np < 65535u * 8 ? np : 65535u * 8;
         refine_anchor_kernel<true><<<gb, kRefineThreads, kRefineSmem, st>>>(b, d_tcnt.p + p0 * kRefineThreads,
                                                                              nullptr);
-        refine_chain_kernel<<<grid_for(np * 32ull, 128), 128, 0, st>>>(b);
+        refine_chain_kernel<<<grid_for(np * 32ull, kRefineWarps * 32), kRefineWarps * 32, 0, st>>>(b);
         refine_chain_block_kernel<<<gb, kRefineThreads, 0, st>>>(b);
         SCK(cudaGetLastError());
         SCK(cudaStreamSynchronize(st));

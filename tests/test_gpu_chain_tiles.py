@@ -1,0 +1,96 @@
+"""Chaining in tiles of 32 anchors: chains equal the oracle's (whole numbers)
+where the tiling and the 32-bit scores could go wrong: anchor counts around
+multiples of 32, dense repeats (many equal scores, thousands of anchors that
+follow one chain at a loss), every anchor on one strand, proteins past 32,000
+residues (64-bit scores), and regions with anchor counts around the limit
+between one warp and eight."""
+import numpy as np
+import pytest
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+FIELDS = ("strand", "n_anchors", "score", "x_first", "x_last", "y_first", "y_last")
+REFINE_FIELDS = ("n_anchors", "score", "x_first", "x_last", "y_first", "y_last")
+
+
+@pytest.fixture(scope="module")
+def mp():
+    from paper_2210_08052_gb300 import build
+    build.build()
+    import paper_2210_08052_gb300 as m
+    m.lib()
+    return m
+
+
+def _genome(rng, prots, strand):
+    parts = []
+    for p in prots:
+        gene = synth.reverse_translate(rng, p)
+        parts += [synth.random_dna(rng, int(rng.integers(200, 3000)), 0.4), gene if strand(rng) else synth.revcomp(gene)]
+    return "".join(parts) + synth.random_dna(rng, 2000, 0.4)
+
+
+@pytest.mark.parametrize("case", ["mixed", "one strand", "repeats", "long protein"])
+def test_chains_equal_the_oracles(mp, orc, case):
+    rng = np.random.default_rng(300 + len(case))
+    base = [synth.random_protein(rng, int(m)) for m in rng.integers(40, 400, 30)]
+    strand = (lambda r: True) if case == "one strand" else (lambda r: r.random() < 0.5)
+    queries = [p[:k] for p in base[:6] for k in (6, 7, 37, 38, 39, 40, len(p))] + base
+    planted = base * 2
+    if case == "repeats":
+        unit = synth.random_protein(rng, 12)
+        planted = [unit * 20, base[0], unit * 33, base[0], unit * 8] + base
+        queries += [unit * n for n in (2, 3, 5, 8, 30, 60)]
+    if case == "long protein":
+        queries = ["".join(base) * 6, "".join(reversed(base)) * 7]
+        queries = [(q * 4)[:m] for q, m in zip(queries, (32_000, 33_000))] + base[:3]
+        assert len(queries[1]) == 33_000
+    genome = _genome(rng, planted, strand)
+    off = np.concatenate([[0], np.cumsum([len(q) for q in queries])])
+    ctx = mp.mp_dp_init(None, 0)
+    try:
+        idx = mp.mp_index_build(ctx, genome)
+        got = {top: mp.mp_index_chain(ctx, idx, "".join(queries), off[:-1], np.diff(off), top) for top in (1, 200)}
+        mp.mp_index_free(idx)
+    finally:
+        mp.mp_dp_destroy(ctx)
+    woff, wpos = orc.build_index(genome)
+    most = 0
+    for k, q in enumerate(queries):
+        anc = orc.anchors(woff, wpos, q)
+        most = max(most, len(anc))
+        for top, (ch, n) in got.items():
+            want, _ = orc.chain(anc, top)
+            have = [{f: int(ch[k, t][f]) for f in FIELDS} for t in range(int(n[k]))]
+            assert have == want, (k, len(q), len(anc), top)
+    assert most > 300
+
+
+def test_second_round_around_the_block_limit(mp, orc):
+    """Regions with 1 to about 2,000 anchors, dense ones among them."""
+    rng = np.random.default_rng(320)
+    pairs, counts = [], []
+    for copies in (0, 1, 2, 3, 4, 5, 6, 8, 12):
+        for m in (5, 6, 36, 37, 100, 170, 400):
+            prot = synth.random_protein(rng, m)
+            nt = synth.random_dna(rng, 400, 0.4) + "".join(
+                synth.reverse_translate(rng, prot) + synth.random_dna(rng, int(rng.integers(0, 300)), 0.4)
+                for _ in range(copies))
+            strand = 1 if rng.random() < 0.5 else -1
+            pairs.append(synth.Pair(prot, nt if strand > 0 else synth.revcomp(nt), strand))
+    unit = synth.random_protein(rng, 9)
+    for n in (3, 6, 9, 12):
+        pairs.append(synth.Pair(unit * n, synth.reverse_translate(rng, unit * n), 1))
+    ctx = mp.mp_dp_init(None, 0)
+    try:
+        got = mp.mp_chain_refine(ctx, pairs)
+    finally:
+        mp.mp_dp_destroy(ctx)
+    for k, p in enumerate(pairs):
+        anc = orc.refine_anchors(p.prot, p.nt, p.strand)
+        counts.append(len(anc))
+        want, _ = orc.refine_chain(anc)
+        assert {f: int(got[k][f]) for f in REFINE_FIELDS} == want, (k, len(anc))
+    assert any(c > 512 for c in counts) and any(0 < c <= 512 for c in counts) and any(c == 0 for c in counts)
