@@ -77,13 +77,19 @@ __host__ __device__ __forceinline__ uint32_t neg2(uint32_t lo, uint32_t hi)
     return ((0x10000u - lo) & 0xffffu) | (((0x10000u - hi) & 0xffffu) << 16);
 }
 
-// Per-genome-position record for the lo cell at 0-based position ii
-// (1-based i = ii + 1), the penalties negated per 16-bit half (modulo 2^16,
-// so that one fused add-max subtracts them):
-//   x = [-(r + d(i+1)), -(r + d(i))]   (16-bit halves, lo first)
-//   y = [-a(i), -a(i-1)]
-//   z = byte offset of the profile row of the codon ending at i
-__device__ __forceinline__ uint4 make_record(const uint32_t *g, int n, int ii, const ScoreParams &sp)
+// Per-genome-position record of 0-based position ii (1-based i = ii + 1), the
+// low halves for row ii and the high halves for a row before, the penalties
+// negated per 16-bit half (modulo 2^16, so that one fused add-max subtracts
+// them):
+//   x = -(r + d(i+1))
+//   y = -a(i)
+//   z, w = byte offsets of the profile rows of the codons ending at the low
+//   and the high halves' row
+// The row before is kBackOne rows back where a warp runs one strip (this
+// function), 64 where it runs two, and the one before in 128-residue strips
+// (records_kernel).
+constexpr int kBackOne = kStripW / 2;
+__device__ __forceinline__ void row_terms(const uint32_t *g, int n, int ii, const ScoreParams &sp, int &d, int &ac, int &aa)
 {
     const int s = ii - 3;                  // window T0[ii-3 .. ii+4]
     const int w = s >> 4;                  // floor division (s may be negative)
@@ -93,22 +99,22 @@ __device__ __forceinline__ uint4 make_record(const uint32_t *g, int n, int ii, c
     int b[8];
     bool v[8];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
+    for (int k = 1; k < 8; ++k) {
         b[k] = (win >> (2 * k)) & 3;
         v[k] = static_cast<unsigned>(s + k) < static_cast<unsigned>(n);
     }
-    const int aa = (v[1] && v[3]) ? c_code.v[b[1] * 16 + b[2] * 4 + b[3]] : 21;
-    const int r = sp.r;
-    const int dC = splice_donor(sp, b[5], b[6], b[7], v[5], v[6], v[7]);     // d(i+1)
-    const int dB = splice_donor(sp, b[4], b[5], b[6], v[4], v[5], v[6]);     // d(i)
-    const int aA = splice_acceptor(sp, b[1], b[2], b[3], v[1], v[2], v[3]);  // a(i)
-    const int aC = splice_acceptor(sp, b[0], b[1], b[2], v[0], v[1], v[2]);  // a(i-1)
-    uint4 rec;
-    rec.x = neg2(static_cast<uint32_t>(r + dC), static_cast<uint32_t>(r + dB));
-    rec.y = neg2(static_cast<uint32_t>(aA), static_cast<uint32_t>(aC));
-    rec.z = static_cast<uint32_t>(aa) * 128u;
-    rec.w = 0;
-    return rec;
+    aa = (v[1] && v[3]) ? c_code.v[b[1] * 16 + b[2] * 4 + b[3]] : 21;
+    d = splice_donor(sp, b[5], b[6], b[7], v[5], v[6], v[7]);          // d(i+1)
+    ac = splice_acceptor(sp, b[1], b[2], b[3], v[1], v[2], v[3]);      // a(i)
+}
+__device__ __forceinline__ uint4 make_record(const uint32_t *g, int n, int ii, const ScoreParams &sp)
+{
+    int d0, a0, aa0, d1, a1, aa1;
+    row_terms(g, n, ii, sp, d0, a0, aa0);
+    row_terms(g, n, max(ii - kBackOne, -kRecPre), sp, d1, a1, aa1);
+    return make_uint4(neg2(static_cast<uint32_t>(sp.r + d0), static_cast<uint32_t>(sp.r + d1)),
+                      neg2(static_cast<uint32_t>(a0), static_cast<uint32_t>(a1)), static_cast<uint32_t>(aa0) * 128u,
+                      static_cast<uint32_t>(aa1) * 128u);
 }
 
 // --------------------------------------------------------------- smem
@@ -218,12 +224,32 @@ struct WarpSmemD {
     } it;
 };
 
+// Shared memory of a warp running one strip (Ops16s): as WarpSmemD, the ring
+// in one piece and a word per profile entry.
+struct WarpSmemS {
+    uint2 xy[kRing + kRingPad];
+    uint2 zw[kRing + kRingPad];
+    uint32_t prof[2][kProfRows * 32];
+    alignas(16) uint32_t in[2][kChunk];
+    alignas(16) uint32_t out[2][kChunk];
+    alignas(16) uint32_t zero[kChunk + kBody];
+    WarpSmemD::Item it;
+};
+
 // 16-byte store to shared memory that leaves the compiler free to move loads of
 // other shared data across it (what is stored here is read after a warp barrier)
 __device__ __forceinline__ void st_shared16(void *smem, uint32_t x, uint32_t y, uint32_t z, uint32_t w)
 {
     const uint32_t sa = static_cast<uint32_t>(__cvta_generic_to_shared(smem));
     asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(sa), "r"(x), "r"(y), "r"(z), "r"(w));
+}
+
+// the same to the stream in global memory (a pointer kept in shared memory is
+// not known to be global: as a generic store it would order every shared load
+// behind it)
+__device__ __forceinline__ void st_stream16(uint8_t *p, uint32_t x, uint32_t y, uint32_t z, uint32_t w)
+{
+    asm volatile("st.global.v4.u32 [%0], {%1, %2, %3, %4};" ::"l"(p), "r"(x), "r"(y), "r"(z), "r"(w));
 }
 
 // 8-byte asynchronous copy global -> shared
@@ -247,17 +273,32 @@ __device__ __forceinline__ void fetch_records_d(WarpSmemD &sm, const uint4 *recs
     }
 }
 
+__device__ __forceinline__ void fetch_records_s(WarpSmemS &sm, const uint4 *recs, int lo, int lane)
+{
+    for (int ii = lo + lane; ii < lo + kChunk; ii += 32) {
+        const int idx = ii & (kRing - 1);
+        const uint2 *r = reinterpret_cast<const uint2 *>(recs + ii + kRecPre);
+        cp_async8(&sm.xy[idx], r);
+        cp_async8(&sm.zw[idx], r + 1);
+        if (idx < kRingPad) {
+            cp_async8(&sm.xy[idx + kRing], r);
+            cp_async8(&sm.zw[idx + kRing], r + 1);
+        }
+    }
+}
+
 // ================================================================ int16 ops
-// FAR: the records are those of a pair whose other warps run two strips
-// (Ops16d); the high halves (the row before) come from the step before.
-template <bool FAR>
-struct Ops16T {
+// One strip, two neighbouring residues per lane: the first strip of a pair
+// with an odd number of strips whose other warps run two (Ops16d).  Its
+// records are theirs; the high halves (here of the row before) come from the
+// step before.
+struct Ops16 {
     using Bnd = uint32_t;                  // [H, I] biased 16-bit
     using Smem = WarpSmem<Bnd>;
     static constexpr int W = kStripW, CPL = 2;
-    // words between profile rows, and from the low to the high table's entry
-    // (FAR: the records' row offsets are those of 256-byte rows)
-    static constexpr int kRowWords = FAR ? 64 : 32, kHiWords = FAR ? 32 : kProfRows * 32;
+    // words between profile rows (the records' offsets are those of 256-byte
+    // rows), and from the low to the high table's entry
+    static constexpr int kRowWords = 64, kHiWords = 32;
     static constexpr uint32_t Z = 0x80008000u;      // biased 0 in both halves
     static constexpr uint32_t NEGV = 0x40004000u;   // biased -16384
     static constexpr Bnd kBnd0 = 0x40008000u;       // column 0: H = 0, I = -inf
@@ -337,10 +378,10 @@ struct Ops16T {
         s.IL = (lane == 0) ? ((w0 >> 16) | 0x40000000u) : NEGV;
         s.D1 = s.D2 = s.D3 = NEGV;
         s.A1 = s.B1 = s.C1 = NEGV;
-        s.VD1 = FAR ? prmt<0x5410>(recm1.x, recm2.x) : recm1.x;
-        s.VD2 = FAR ? prmt<0x5410>(recm2.x, recm3.x) : recm2.x;
-        s.VA1 = FAR ? prmt<0x5410>(recm1.y, recm2.y) : recm1.y;
-        s.VA2 = FAR ? prmt<0x5410>(recm2.y, recm3.y) : recm2.y;
+        s.VD1 = prmt<0x5410>(recm1.x, recm2.x);
+        s.VD2 = prmt<0x5410>(recm2.x, recm3.x);
+        s.VA1 = prmt<0x5410>(recm1.y, recm2.y);
+        s.VA2 = prmt<0x5410>(recm2.y, recm3.y);
         s.X1 = xm1;
         s.TC = 0xffffu; s.bklo = 0; s.bkhi = 0; s.cm = 0;
     }
@@ -364,7 +405,7 @@ struct Ops16T {
                                                     int lane, int ii, int n)
     {
         // negated penalties
-        const uint32_t VD0 = FAR ? prmt<0x5410>(rec.x, s.VD1) : rec.x, VA0 = FAR ? prmt<0x5410>(rec.y, s.VA1) : rec.y;
+        const uint32_t VD0 = prmt<0x5410>(rec.x, s.VD1), VA0 = prmt<0x5410>(rec.y, s.VA1);
         const uint32_t X0 = *reinterpret_cast<const uint32_t *>(
             reinterpret_cast<const char *>(prof_lane) + rec.z);
         const uint32_t X0h = *reinterpret_cast<const uint32_t *>(
@@ -462,9 +503,7 @@ struct Ops16T {
     {
         return static_cast<int>(h ? (w >> 16) : (w & 0xffffu)) - 32768;
     }
-    static __device__ __forceinline__ int cell_max(const ColMax &m, int k) { return word_h(m, k); }
 };
-using Ops16 = Ops16T<false>;
 
 // ================================================================ int32 ops
 struct V2 {
@@ -475,11 +514,8 @@ __device__ __forceinline__ V2 mx(V2 a, V2 b) { return V2{max(a.lo, b.lo), max(a.
 __device__ __forceinline__ V2 sub(V2 a, V2 b) { return V2{a.lo - b.lo, a.hi - b.hi}; }
 __device__ __forceinline__ V2 subc(V2 a, int32_t b) { return V2{a.lo - b, a.hi - b}; }
 __device__ __forceinline__ V2 add(V2 a, V2 b) { return V2{a.lo + b.lo, a.hi + b.hi}; }
-// the two negated penalties of a record word, sign-extended
-__device__ __forceinline__ V2 unpack_neg16(uint32_t w)
-{
-    return V2{static_cast<int32_t>(w << 16) >> 16, static_cast<int32_t>(w) >> 16};
-}
+// the negated penalty in the low half of a record word, sign-extended
+__device__ __forceinline__ int32_t low_neg16(uint32_t w) { return static_cast<int32_t>(w << 16) >> 16; }
 
 struct Ops32 {
     struct Bnd {
@@ -487,7 +523,7 @@ struct Ops32 {
     };
     using Smem = WarpSmem<Bnd>;
     static constexpr int W = kStripW, CPL = 2;
-    static constexpr int kRowWords = 32, kHiWords = kProfRows * 32;       // as Ops16T
+    static constexpr int kRowWords = 32, kHiWords = kProfRows * 32;       // as Ops16
     static constexpr int32_t NEG = -(1 << 28);
     static constexpr Bnd kBnd0 = {0, NEG};
 
@@ -525,7 +561,7 @@ struct Ops32 {
         return (static_cast<uint32_t>(slo) & 0xffffu) | (static_cast<uint32_t>(shi) << 16);
     }
 
-    static __device__ __forceinline__ void init(State &s, int lane, Bnd w0, uint4 recm1, uint4 recm2, uint4,
+    static __device__ __forceinline__ void init(State &s, int lane, Bnd w0, uint4 recm1, uint4 recm2, uint4 recm3,
                                                 uint32_t xm1, int h_self, int h_left)
     {
         // the same history as the int16 state (see Ops16::init)
@@ -536,8 +572,8 @@ struct Ops32 {
         s.IL = (lane == 0) ? V2{w0.i, NEG} : ng;
         s.D1 = s.D2 = s.D3 = ng;
         s.A1 = s.B1 = s.C1 = ng;
-        s.VD1 = unpack_neg16(recm1.x); s.VD2 = unpack_neg16(recm2.x);
-        s.VA1 = unpack_neg16(recm1.y); s.VA2 = unpack_neg16(recm2.y);
+        s.VD1 = V2{low_neg16(recm1.x), low_neg16(recm2.x)}; s.VD2 = V2{s.VD1.hi, low_neg16(recm3.x)};
+        s.VA1 = V2{low_neg16(recm1.y), low_neg16(recm2.y)}; s.VA2 = V2{s.VA1.hi, low_neg16(recm3.y)};
         s.X1 = xm1;
         s.bslo = s.bshi = 0; s.btlo = s.bthi = 0; s.t = 0;
         s.cmlo = s.cmhi = NEG;
@@ -550,7 +586,8 @@ struct Ops32 {
                                                  const uint32_t *prof_lane, Bnd bin, Bnd &wout,
                                                  int lane, int ii, int n)
     {
-        const V2 VD0 = unpack_neg16(rec.x), VA0 = unpack_neg16(rec.y);   // negated penalties
+        // negated penalties (the hi cell's row is the lo cell's of the step before)
+        const V2 VD0{low_neg16(rec.x), s.VD1.lo}, VA0{low_neg16(rec.y), s.VA1.lo};
         const uint32_t X0 = *reinterpret_cast<const uint32_t *>(
             reinterpret_cast<const char *>(prof_lane) + rec.z);
         const uint32_t X0h = *reinterpret_cast<const uint32_t *>(
@@ -904,11 +941,11 @@ struct Ops16x4 {
 //
 // What bounds it: instruction issue and the operands behind it.  Every max,
 // fused add-max, byte permute and select takes the ALU pipe of a scheduler for
-// two clocks, and most read three registers.  One strip per warp (Ops16T)
+// two clocks, and most read three registers.  One strip per warp (Ops16)
 // takes 32.1 instructions (19.3 of them on the ALU) and 9.4 shared-memory rows
 // per 64 cells, here the same cells take 26.5, 14.7 and 8: 51.6 clocks of a
-// scheduler against 44.  A warp alone takes 104 clocks per step of 128 cells
-// (87 for 64).  Every form tried ran at 0.6 instructions per clock when
+// scheduler against 44.  A warp alone takes 98 clocks per step of 128 cells
+// (one strip per warp without the loads ahead of their step: 87 for 64).  Every form tried ran at 0.6 instructions per clock when
 // several warps shared a scheduler, so what counted was instructions: two
 // maxima of a pair of steps in one, frameshift maxima shared by a and b, no
 // permute in the hand-over, profile halves added instead of permuted, and
@@ -999,16 +1036,18 @@ struct Ops16d {
         H0 = vmax3(M, I0, Y);
     }
     // valid rows of a register's two cells
+    template <int UP>
     static __device__ __forceinline__ uint32_t rows(int ii, int n)
     {
-        const int up = ii - kUp;
+        const int up = ii - UP;
         return ((ii >= 0 && ii < n) ? 0x0000ffffu : 0u) | ((up >= 0 && up < n) ? 0xffff0000u : 0u);
     }
     // cells before row 1 are outside the matrix; row -1 (0-based) is row 0
+    template <int UP>
     static __device__ __forceinline__ void mask(int ii, uint32_t ROW0, uint32_t &H, uint32_t &I, uint32_t &D,
                                                 uint32_t &A, uint32_t &B, uint32_t &C)
     {
-        const int up = ii - kUp;
+        const int up = ii - UP;
         const uint32_t kill = (ii < 0 ? 0x0000ffffu : 0u) | (up < 0 ? 0xffff0000u : 0u);
         const uint32_t row0 = (ii == -1 ? 0x0000ffffu : 0u) | (up == -1 ? 0xffff0000u : 0u);
         H = (H & ~kill) | (((row0 & ROW0) | (~row0 & NEGV)) & kill);
@@ -1023,14 +1062,13 @@ struct Ops16d {
     // values; Ib: b's I less the extension of the columns right of it.
     // MASK 2: cells before row 1 get their boundary values; 1 and 2: without a
     // stream, rows outside the region are kept out of the maxima (see
-    // Ops16T::step for why no more is needed).  SECOND: the second step of a
+    // Ops16::step for why no more is needed).  SECOND: the second step of a
     // pair, which takes both steps' cells into the chunk maximum.
     template <int MASK, bool KEYS, bool SECOND>
-    static __device__ __forceinline__ void step(State &s, const Consts &c, const uint2 rec, const uint2 zw,
-                                                const uint2 *prof_lane, uint32_t inH, uint32_t inI, int lane, int ii, int n, uint32_t &Ha,
+    static __device__ __forceinline__ void step(State &s, const Consts &c, const uint2 rec, const uint2 Xl,
+                                                const uint2 Xh, uint32_t inH, uint32_t inI, int lane, int ii, int n, uint32_t &Ha,
                                                 uint32_t &Hb, uint32_t &Ib)
     {
-        const uint2 Xl = prof_at(prof_lane, zw.x), Xh = prof_at(prof_lane + kProfRows * 32, zw.y);
         const uint32_t Sa = Xl.x + Xh.x;
         uint32_t Da, Db, Ia, Ib0;
         // frameshift terms H[i-1][j-1], H[i-2][j-1], H[i-1][j], H[i-2][j]: a's own
@@ -1042,8 +1080,8 @@ struct Ops16d {
         cells(s.aH1, s.aH3, Fa, s.L0, s.L1, s.L3, s.IL, s.aD3, Sa, c.NQEa, c.Ea, c.NF, c.FLOOR, rec.x, s.VD1,
               s.VD2, rec.y, s.VA1, s.VA2, s.aA, s.aB, s.aC, Da, Ia, Ha);
         if (MASK == 2) {
-            mask(ii, c.ROW0A, Ha, Ia, Da, s.aA, s.aB, s.aC);
-            mask(ii - 1, c.ROW0B, Hb, Ib0, Db, s.bA, s.bB, s.bC);
+            mask<kUp>(ii, c.ROW0A, Ha, Ia, Da, s.aA, s.aB, s.aC);
+            mask<kUp>(ii - 1, c.ROW0B, Hb, Ib0, Db, s.bA, s.bB, s.bC);
         }
         Ib = Ib0 - c.EN;
         const int left = (lane + 31) & 31;
@@ -1064,7 +1102,7 @@ struct Ops16d {
         s.VA3 = s.VA2; s.VA2 = s.VA1; s.VA1 = rec.y;
         s.Sb = Xl.y + Xh.y;
         if (KEYS) {
-            const uint32_t ha = MASK ? Ha & rows(ii, n) : Ha, hb = MASK ? Hb & rows(ii - 1, n) : Hb;
+            const uint32_t ha = MASK ? Ha & rows<kUp>(ii, n) : Ha, hb = MASK ? Hb & rows<kUp>(ii - 1, n) : Hb;
             s.k0 = max(s.k0, ha * 65536u + s.TC);
             s.k1 = max(s.k1, hb * 65536u + s.TC);
             s.k2 = max(s.k2, (ha & 0xffff0000u) | s.TC);
@@ -1093,8 +1131,22 @@ struct Ops16d {
         constexpr int kHalf = kRing / 2 + kBodyD / 2;
         uint32_t wl[4], wu[4], hb4[4], ib4[4];
         uint4 h4, i4;
+        // a step's record and profile words are loaded a step ahead, its profile
+        // rows two
+        auto xy_at = [&](int k) { return xy0[(k & 1) * kHalf + (k >> 1)]; };
+        auto zw_at = [&](int k) { return zw0[(k & 1) * kHalf + (k >> 1)]; };
+        const uint2 *pr = &sm.prof[0][lane];
+        uint2 xy = xy_at(0), zw = zw_at(0), zn = zw_at(1);
+        uint2 Xl = prof_at(pr, zw.x), Xh = prof_at(pr + kProfRows * 32, zw.y);
 #pragma unroll
         for (int k = 0; k < N; ++k) {
+            const uint2 xyc = xy, Xlc = Xl, Xhc = Xh;
+            if (k + 1 < N) {
+                xy = xy_at(k + 1);
+                Xl = prof_at(pr, zn.x);
+                Xh = prof_at(pr + kProfRows * 32, zn.y);
+                if (k + 2 < N) zn = zw_at(k + 2);
+            }
             if ((k & 3) == 0) {
                 h4 = *reinterpret_cast<const uint4 *>(q.ih + k);
                 i4 = *reinterpret_cast<const uint4 *>(q.ih + kChunk + k);
@@ -1102,13 +1154,12 @@ struct Ops16d {
             const uint32_t inH = (k & 3) == 0 ? h4.x : (k & 3) == 1 ? h4.y : (k & 3) == 2 ? h4.z : h4.w;
             const uint32_t inI = (k & 3) == 0 ? i4.x : (k & 3) == 1 ? i4.y : (k & 3) == 2 ? i4.z : i4.w;
             uint32_t Ha, Hb;
-            const uint2 xy = xy0[(k & 1) * kHalf + (k >> 1)], zw = zw0[(k & 1) * kHalf + (k >> 1)];
             if (k & 1)
-                step<MASK, !STORE, true>(st, c, xy, zw, &sm.prof[0][lane], inH, inI, lane, q.t + k - 2 * lane, n, Ha, Hb,
+                step<MASK, !STORE, true>(st, c, xyc, Xlc, Xhc, inH, inI, lane, q.t + k - 2 * lane, n, Ha, Hb,
                                          ib4[k & 3]);
             else
-                step<MASK, !STORE, false>(st, c, xy, zw, &sm.prof[0][lane], inH, inI, lane, q.t + k - 2 * lane, n, Ha,
-                                          Hb, ib4[k & 3]);
+                step<MASK, !STORE, false>(st, c, xyc, Xlc, Xhc, inH, inI, lane, q.t + k - 2 * lane, n, Ha, Hb,
+                                          ib4[k & 3]);
             if (STORE) {
                 // each strip's stream as Ops16 writes it: [H of 2l, H of 2l+1]
                 wl[k & 3] = prmt<0x5410>(Ha, Hb);
@@ -1117,7 +1168,6 @@ struct Ops16d {
                 hb4[k & 3] = Hb;
             }
             if ((k & 3) == 3) {
-                const uint4 l4 = make_uint4(wl[0], wl[1], wl[2], wl[3]), u4 = make_uint4(wu[0], wu[1], wu[2], wu[3]);
                 if (lane == 31) {
                     if (STORE) st_shared16(q.oh + k - 3, wu[0], wu[1], wu[2], wu[3]);
                     else st_shared16(q.oh + k - 3, hb4[0], hb4[1], hb4[2], hb4[3]);
@@ -1125,9 +1175,9 @@ struct Ops16d {
                 }
                 if (STORE) {
                     const int u = q.t + k - 3;
-                    if (!MASK || u < ulimit) *reinterpret_cast<uint4 *>(q.pl + (k - 3) * kStepBytes) = l4;
+                    if (!MASK || u < ulimit) st_stream16(q.pl + (k - 3) * kStepBytes, wl[0], wl[1], wl[2], wl[3]);
                     if (!MASK || static_cast<unsigned>(u - kUp) < static_cast<unsigned>(ulimit))
-                        *reinterpret_cast<uint4 *>(q.pu + (k - 3) * kStepBytes) = u4;
+                        st_stream16(q.pu + (k - 3) * kStepBytes, wu[0], wu[1], wu[2], wu[3]);
                 }
             }
         }
@@ -1163,6 +1213,160 @@ struct Ops16d {
         for (const int te = min(t1, n) - kBodyD; q.t <= te;) body<0, STORE, kBodyD>(st, c, sm, q, lane, n, ulimit);
 #pragma unroll 1
         while (q.t < t1) body<1, STORE, kBody>(st, c, sm, q, lane, n, ulimit);
+    }
+};
+
+// ================================================ int16, one strip per warp
+// Lane l holds residues l (low half) and l + 32 (high half) of the strip, at
+// rows t - l and t - l - 32: the one-strip counterpart of Ops16d, with its
+// hand-over (lane l-1's whole register, lane 31's low half for lane 0's high
+// half) and no byte permute at all; the stream holds the registers as they
+// are.  For pairs of one strip, pairs that may need int32, and pairs whose own
+// chain of steps would outlast the rest of the batch (see plan_waves): a lone
+// warp takes 81 clocks per step of 64 cells, 98 per Ops16d's of 128.  A step's
+// record and profile words are loaded a step ahead (94 clocks without: the
+// loads and the shuffle, each waited for where it is used, came on top of the
+// arithmetic).  64 genes at once 1.98 -> 1.74 ms.
+struct Ops16s {
+    static constexpr uint32_t Z = Ops16::Z, NEGV = Ops16::NEGV;
+    static constexpr int kUp = kBackOne;                  // rows the high half runs behind
+
+    struct Consts {
+        uint32_t NQE, E, EN, NF, FLOOR, ROW0, mult;       // as Ops16d
+    };
+    struct State {
+        uint32_t H1, H2, H3, L0, L1, L2, L3, IL, D1, D2, D3, A, B, C;
+        uint32_t VD1, VD2, VA1, VA2;
+        uint32_t cm;                                      // this chunk's maxima (pairs with a stream)
+        uint32_t TC, k0, k1;                              // best-cell keys (pairs without one)
+    };
+
+    // State before step 0: lane 0's low half holds row 0, and lane 1 sees it as
+    // its left neighbour (h_left: H of row 0 of the column to the left).
+    static __device__ __forceinline__ void init(State &s, const WarpSmemS &sm, int lane, uint32_t w0, int h_self,
+                                                int h_left)
+    {
+        const uint32_t hl = Ops16::pack2(h_left, -16384);
+        s.H1 = lane == 0 ? Ops16::pack2(h_self, -16384) : NEGV;
+        s.H2 = s.H3 = NEGV;
+        s.L0 = lane == 0 ? ((w0 & 0xffffu) | 0x40000000u) : lane == 1 ? hl : NEGV;
+        s.L1 = lane == 0 ? hl : NEGV;
+        s.L2 = s.L3 = NEGV;
+        s.IL = lane == 0 ? ((w0 >> 16) | 0x40000000u) : NEGV;
+        s.D1 = s.D2 = s.D3 = s.A = s.B = s.C = NEGV;
+        const uint2 r1 = sm.xy[(-lane - 1) & (kRing - 1)], r2 = sm.xy[(-lane - 2) & (kRing - 1)];
+        s.VD1 = r1.x; s.VD2 = r2.x;
+        s.VA1 = r1.y; s.VA2 = r2.y;
+        s.cm = 0;
+        s.TC = 0xffffu;
+        s.k0 = s.k1 = 0;
+    }
+
+    // One step (MASK and SECOND as in Ops16d).  H: the lane's H values; I: its
+    // I less the extension of the columns to the right.
+    template <int MASK, bool KEYS, bool SECOND>
+    static __device__ __forceinline__ void step(State &s, const Consts &c, const uint2 rec, const uint32_t S,
+                                                uint32_t inH, uint32_t inI, int lane, int ii,
+                                                int n, uint32_t &H, uint32_t &I)
+    {
+        uint32_t I0, D0;
+        const uint32_t FS = vmax(vmax3(s.L1, s.L2, s.H2), s.H1);
+        Ops16d::cells(s.H1, s.H3, FS, s.L0, s.L1, s.L3, s.IL, s.D3, S, c.NQE, c.E, c.NF, c.FLOOR, rec.x, s.VD1, s.VD2,
+                      rec.y, s.VA1, s.VA2, s.A, s.B, s.C, D0, I0, H);
+        if (MASK == 2) Ops16d::mask<kUp>(ii, c.ROW0, H, I0, D0, s.A, s.B, s.C);
+        I = I0 - c.EN;
+        const int left = (lane + 31) & 31;
+        const uint32_t RH = __shfl_sync(kFull, H, left), RI = __shfl_sync(kFull, I, left);
+        s.L3 = s.L2; s.L2 = s.L1; s.L1 = s.L0;
+        s.L0 = RH * c.mult + inH;
+        s.IL = RI * c.mult + inI;
+        if (!KEYS && SECOND) s.cm = vmax3(s.cm, s.H1, H);
+        s.H3 = s.H2; s.H2 = s.H1; s.H1 = H;
+        s.D3 = s.D2; s.D2 = s.D1; s.D1 = D0;
+        s.VD2 = s.VD1; s.VD1 = rec.x;
+        s.VA2 = s.VA1; s.VA1 = rec.y;
+        if (KEYS) {
+            const uint32_t h = MASK ? H & Ops16d::rows<kUp>(ii, n) : H;
+            s.k0 = max(s.k0, h * 65536u + s.TC);
+            s.k1 = max(s.k1, (h & 0xffff0000u) | s.TC);
+            s.TC -= 1;
+        }
+    }
+
+    struct Cursor {
+        const uint32_t *ih;
+        uint32_t *oh;
+        uint8_t *pl;
+        int ridx, t;
+    };
+    template <int MASK, bool STORE>
+    static __device__ __forceinline__ void body(State &st, const Consts &c, WarpSmemS &sm, Cursor &q, int lane, int n)
+    {
+        // record of the low cell at step t + k: position t + k - l
+        const int r = q.ridx & (kRing - 1);
+        const uint2 *xy0 = &sm.xy[r], *zw0 = &sm.zw[r];
+        uint32_t h4[4], i4[4];
+        uint4 bh, bi;
+        const char *pr = reinterpret_cast<const char *>(&sm.prof[0][lane]);
+        // (records and profile words ahead of their step, as in Ops16d)
+        auto prof_at = [&](uint2 z) {
+            return make_uint2(*reinterpret_cast<const uint32_t *>(pr + z.x),
+                              *reinterpret_cast<const uint32_t *>(pr + kProfRows * 128 + z.y));
+        };
+        uint2 xy = xy0[0], zn = zw0[1], X = prof_at(zw0[0]);
+#pragma unroll
+        for (int k = 0; k < kBody; ++k) {
+            const uint2 xyc = xy;
+            const uint32_t Sc = X.x + X.y;
+            if (k + 1 < kBody) {
+                xy = xy0[k + 1];
+                X = prof_at(zn);
+                if (k + 2 < kBody) zn = zw0[k + 2];
+            }
+            if ((k & 3) == 0) {
+                bh = *reinterpret_cast<const uint4 *>(q.ih + k);
+                bi = *reinterpret_cast<const uint4 *>(q.ih + kChunk + k);
+            }
+            const uint32_t inH = (k & 3) == 0 ? bh.x : (k & 3) == 1 ? bh.y : (k & 3) == 2 ? bh.z : bh.w;
+            const uint32_t inI = (k & 3) == 0 ? bi.x : (k & 3) == 1 ? bi.y : (k & 3) == 2 ? bi.z : bi.w;
+            if (k & 1)
+                step<MASK, !STORE, true>(st, c, xyc, Sc, inH, inI, lane, q.t + k - lane, n, h4[k & 3], i4[k & 3]);
+            else
+                step<MASK, !STORE, false>(st, c, xyc, Sc, inH, inI, lane, q.t + k - lane, n, h4[k & 3], i4[k & 3]);
+            if ((k & 3) == 3) {
+                if (lane == 31) {
+                    st_shared16(q.oh + k - 3, h4[0], h4[1], h4[2], h4[3]);
+                    st_shared16(q.oh + kChunk + k - 3, i4[0], i4[1], i4[2], i4[3]);
+                }
+                if (STORE) st_stream16(q.pl + (k - 3) * kStepBytes, h4[0], h4[1], h4[2], h4[3]);
+            }
+        }
+        if (lane == 0) q.ih += kBody;
+        q.oh += kBody;
+        q.ridx += kBody;
+        q.pl += kBody * kStepBytes;
+        q.t += kBody;
+    }
+    template <bool STORE>
+    static __device__ __forceinline__ void chunk(State &st, const Consts &c, WarpSmemS &sm, int lane, int t0, int n,
+                                                 bool anchored, int steps, uint8_t *stream)
+    {
+        Cursor q{lane == 0 ? sm.in[0] : sm.zero, sm.out[0], stream + static_cast<size_t>(t0) * kStepBytes + lane * 16,
+                 t0 - lane, t0};
+        const int t1 = t0 + steps;
+        if (anchored) {
+#pragma unroll 1
+            while (q.t < t1 && q.t < kStripW) body<2, STORE>(st, c, sm, q, lane, n);
+        }
+        if (STORE) {
+#pragma unroll 1
+            while (q.t < t1) body<0, STORE>(st, c, sm, q, lane, n);
+        } else {
+#pragma unroll 1
+            while (q.t + kBody <= min(t1, n)) body<0, STORE>(st, c, sm, q, lane, n);
+#pragma unroll 1
+            while (q.t < t1) body<1, STORE>(st, c, sm, q, lane, n);
+        }
     }
 };
 
@@ -1300,15 +1504,16 @@ struct RowsIn {
 
 // The pair's best cell among a strip's cells that hold `top`, the strip's
 // maximum: the lanes of `who` hold it in half k of their words, whose column
-// is j0 + 2 * lane.  cmax: the strip's column maxima per chunk of kChunk
+// is j0 + mul * lane and which are at row 0 in step r + mul * lane.  cmax: the strip's column maxima per chunk of kChunk
 // steps, which start `shift` steps of the strip before multiples of kChunk
 // (the last one's covers every later step).  The whole warp searches: the
 // chunks 32 at a time, then the first such chunk's steps.
 __device__ __forceinline__ void best_in_strip(const uint8_t *strip, const uint32_t *cmax, int schunks, int shift,
-                                              unsigned who, int k, int j0, int n, int top, int lane, Best &best)
+                                              unsigned who, int k, int mul, int r, int j0, int n, int top, int lane,
+                                              Best &best)
 {
     while (who) {
-        const int L = __ffs(who) - 1, r0 = 2 * L + k;                  // r0: the step of row 0
+        const int L = __ffs(who) - 1, r0 = mul * L + r;
         who &= who - 1;
         int c = -1;
         for (int cb = 0; cb < schunks && c < 0; cb += 32) {
@@ -1332,7 +1537,7 @@ __device__ __forceinline__ void best_in_strip(const uint8_t *strip, const uint32
             }
             found = __reduce_min_sync(kFull, found);
             if (found != 0x7fffffff) {
-                const int ii = found - r0, jj = j0 + 2 * L;
+                const int ii = found - r0, jj = j0 + mul * L;
                 if (better(top, ii, jj, best)) best = Best{top, ii, jj};
                 break;
             }
@@ -1674,7 +1879,7 @@ __device__ void run_strip(const DPArgs &a, typename Ops::Smem &sm, const PairDes
 #pragma unroll 1
                 for (int k = 0; k < 2; ++k)
                     best_in_strip(code_strip, reinterpret_cast<const uint32_t *>(colmax), nchunks, 0,
-                                  __ballot_sync(kFull, (k ? v1 : v0) == top), k, s * W + k, n, top, lane, best);
+                                  __ballot_sync(kFull, (k ? v1 : v0) == top), k, 2, k, s * W + k, n, top, lane, best);
             }
         } else {
             int top = 0;
@@ -1699,7 +1904,7 @@ __device__ void run_strip(const DPArgs &a, typename Ops::Smem &sm, const PairDes
 // Two neighbouring strips of pair p, its work item u, on one warp; see Ops16d.
 // Boundary rows pass between the warps of a pair as in run_strip, once per two
 // strips.  With an odd number of strips the first one is an item of its own
-// (Ops16T<true>): a single strip takes fewer clocks per step, so at the front
+// (Ops16): a single strip takes fewer clocks per step, so at the front
 // it never waits; at the end it ran at the pace of the warp before it.
 template <bool PROF, bool STORE>
 __device__ void run_duo(const DPArgs &a, WarpSmemD &sm, const PairDesc &pd, uint32_t p, int u, int lane)
@@ -1899,18 +2104,183 @@ __device__ void run_duo(const DPArgs &a, WarpSmemD &sm, const PairDesc &pd, uint
                 const int vk = k == 0 ? v[0] : k == 1 ? v[1] : k == 2 ? v[2] : v[3];
                 best_in_strip(k < 2 ? it.lo : it.lo + strip_bytes, k < 2 ? it.cmax : it.cmax + it.schunks * 32, it.schunks,
                               (k >> 1) * kUp,
-                              __ballot_sync(kFull, vk == top), k & 1, j0 - 2 * lane + (k & 1) + (k >> 1) * kUp, n, top,
-                              lane, best);
+                              __ballot_sync(kFull, vk == top), k & 1, 2, k & 1,
+                              j0 - 2 * lane + (k & 1) + (k >> 1) * kUp, n, top, lane, best);
             }
         }
     }
     finish_strip(a, pd, p, best, timed_out, lane, n_items, false, false);
 }
 
+// Strip s of pair p on one warp; see Ops16s.
+template <bool STORE>
+__device__ void run_solo(const DPArgs &a, WarpSmemS &sm, const PairDesc &pd, uint32_t p, int s, int lane, bool rerun)
+{
+    using Ops = Ops16s;
+    constexpr int kUp = Ops::kUp, kLast = kStripW - 1;
+    const int n = static_cast<int>(pd.nt_len);
+    const int m = static_cast<int>(pd.prot_len);
+    const int nstrips = static_cast<int>(pd.n_strips);
+    const uint8_t *P = a.prot + pd.prot_off;
+    uint64_t *rows = static_cast<uint64_t *>(a.bnd) + pd.bnd_off + kBndPad;          // see RowsIn
+    const bool anchored = a.sp.mode != MP_MODE_LOCAL;
+    const int32_t *c0 = anchored ? a.col0 + pd.col0_off : nullptr;      // c0[i] = H[i][0]
+    const ProfPos *pf = (pd.flags & PF_PROF) ? a.prof + pd.prof_off : nullptr;
+    const int32_t *ep = (pd.flags & PF_PROF) ? a.epre + pd.prof_off : nullptr;
+    const int j0 = kStripW * s + lane;                                  // 0-based column of the low cell
+    auto row0 = [&](int j) {
+        if (!anchored || j == 0) return 0;
+        if (pf) return -(pf[1].q + __ldg(ep + (j < m ? j : m)) + (j > m ? a.sp.e * (j - m) : 0));
+        return -(a.sp.q + a.sp.e * j);
+    };
+    Ops::Consts c;
+    {
+        auto gq = [&](int j) { return pf && j < m ? pf[j + 1].q : a.sp.q; };    // of 0-based column j
+        auto ge = [&](int j) { return pf && j < m ? pf[j + 1].e : a.sp.e; };
+        auto pair = [](int lo, int hi) { return static_cast<uint32_t>(lo) | (static_cast<uint32_t>(hi) << 16); };
+        c.NQE = neg2(gq(j0) + ge(j0), gq(j0 + kUp) + ge(j0 + kUp));
+        c.E = pair(ge(j0), ge(j0 + kUp));
+        c.EN = pair(ge(j0 + 1), ge(j0 + 1 + kUp));
+        c.NF = neg2(static_cast<uint32_t>(a.sp.f), static_cast<uint32_t>(a.sp.f));
+        c.FLOOR = anchored ? 0u : Ops::Z;
+        c.ROW0 = Ops16::pack2(row0(j0 + 1), row0(j0 + 1 + kUp));
+        asm volatile("mov.u32 %0, %1;" : "=r"(c.mult) : "r"(lane == 0 ? 65536u : 1u));
+    }
+    const uint4 *recs = a.recs + pd.rec_off;            // recs[ii + kRecPre] is position ii
+    const uint32_t limit = a.spin_limit ? a.spin_limit : kSpinLimit;
+    const uint32_t item = static_cast<uint32_t>(s);
+    bool timed_out = false;
+    if (lane == 0) {
+        const int schunks = (n + kLast + kChunk - 1) / kChunk;
+        const size_t strip_bytes = static_cast<size_t>(schunks) * kChunk * kStepBytes;
+        uint8_t *codes = a.codes + pd.code_off;
+        sm.it.recs = recs;
+        sm.it.rows = rows;
+        sm.it.lo = codes + static_cast<size_t>(s) * strip_bytes;
+        // per-chunk column maxima follow the strips' streams: [strip][chunk][lane]
+        sm.it.cmax = reinterpret_cast<uint32_t *>(codes + static_cast<size_t>(nstrips) * strip_bytes) +
+                     static_cast<size_t>(s) * schunks * 32;
+        sm.it.c0 = c0;
+        sm.it.n = n;
+        sm.it.nsteps = n + kLast;
+        sm.it.schunks = schunks;
+        sm.it.tag = item;
+        sm.it.limit = limit;
+        sm.it.publish = s + 1 < nstrips && !a.no_publish;
+        sm.it.anchored = anchored;
+    }
+    // records for ii in [-kChunk, kChunk)
+    fetch_records_s(sm, recs, -kChunk, lane);
+    fetch_records_s(sm, recs, 0, lane);
+    {
+        // profile: the scores of the lane's two columns
+        const int pc0 = j0 < m ? P[j0] : 21, pc1 = j0 + kUp < m ? P[j0 + kUp] : 21;
+        auto score = [&](int aa, int j, int pc) -> int {
+            if (pf && aa != 21 && j < m) return pf[j + 1].s[aa];
+            return subst_score(a.sp, aa, pf ? 21 : pc);
+        };
+#pragma unroll 2
+        for (int aa = 0; aa < kProfRows; ++aa) {
+            sm.prof[0][aa * 32 + lane] = Ops16::prof_entry(score(aa, j0, pc0), 0);
+            sm.prof[1][aa * 32 + lane] = Ops16::prof_entry(0, score(aa, j0 + kUp, pc1));
+        }
+        for (int k = lane; k < kChunk + kBody; k += 32) sm.zero[k] = 0;
+    }
+    cp_async_wait_all();
+    __syncwarp();
+    Ops::State st;
+    RowsIn in;
+    {
+        uint32_t w0 = anchored ? Ops16::col0_entry(__ldg(c0 + 1)) : Ops16::kBnd0;
+        if (s > 0) {
+            // row 0 (every lane's words are the same), then the first chunk's rows
+            RowsIn first;
+            first.fetch(rows, -lane, 1, item, lane);
+            if (!first.settle(rows, -lane, item, lane, limit)) timed_out = true;
+            w0 = static_cast<uint32_t>(first.v[0]);
+            in.fetch(rows, 1, n, item, lane);
+        }
+        Ops::init(st, sm, lane, w0, row0(j0 + 1), row0(j0));
+    }
+    uint32_t rmax = 0;
+    Best best{0, 0x7fffffff, 0x7fffffff};
+
+#pragma unroll 1
+    for (int t0 = 0; t0 < sm.it.nsteps; t0 += kChunk) {
+        const WarpSmemD::Item &it = sm.it;
+        if (t0 > 0) cp_async_wait_all();                 // this chunk's records (queued last chunk)
+        if (it.tag > 0) {
+            if (!timed_out && !in.settle(it.rows, t0 + 1, it.tag, lane, it.limit)) timed_out = true;
+#pragma unroll
+            for (int q = 0; q < kChunk / 32; ++q) {
+                sm.in[0][lane + 32 * q] = static_cast<uint32_t>(in.v[q]) & 0xffffu;
+                sm.in[1][lane + 32 * q] = static_cast<uint32_t>(in.v[q]) >> 16;
+            }
+            // the next chunk's rows, on their way while this one computes
+            in.fetch(it.rows, t0 + kChunk + 1, it.n, it.tag, lane);
+        } else {
+            // column 0: H = 0, I = -inf; in the anchored modes entry k is row t0 + 2 + k
+            for (int k = lane; k < kChunk; k += 32) {
+                const uint32_t w = it.c0 ? Ops16::col0_entry(__ldg(it.c0 + t0 + 2 + k)) : Ops16::kBnd0;
+                sm.in[0][k] = w & 0xffffu;
+                sm.in[1][k] = w >> 16;
+            }
+        }
+        __syncwarp();
+        // next chunk's records land in ring slots this chunk does not read
+        if (t0 + kChunk < it.nsteps) fetch_records_s(sm, it.recs, t0 + kChunk, lane);
+        // the last chunk runs no further than the last valid row
+        Ops::chunk<STORE>(st, c, sm, lane, t0, it.n, it.anchored != 0,
+                          (min(kChunk, it.nsteps - t0) + kBody - 1) / kBody * kBody, it.lo);
+        __syncwarp();
+        if (it.publish) {
+            // publish the strip's last residue
+            for (int k = lane; k < kChunk; k += 32) {
+                const int r = t0 + k - kLast;
+                if (r >= 0 && r < it.n)
+                    st_relaxed64(it.rows + r,
+                                 static_cast<uint64_t>(it.tag + 1) << 32 | prmt<0x7632>(sm.out[0][k], sm.out[1][k]));
+            }
+        }
+        if (STORE) {
+            it.cmax[t0 / kChunk * 32 + lane] = st.cm;
+            rmax = vmax(rmax, st.cm);
+            st.cm = 0;
+        } else {
+            // fold this chunk's best cells into the warp's best
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const uint32_t key = k ? st.k1 : st.k0;
+                const int sc = static_cast<int>(key >> 16) - 32768;
+                const int jj = j0 + k * kUp, ii = t0 + static_cast<int>(0xffffu - (key & 0xffffu)) - lane - k * kUp;
+                if (sc > 0 && jj < m && better(sc, ii, jj, best)) best = Best{sc, ii, jj};
+            }
+            st.TC = 0xffffu;
+            st.k0 = st.k1 = 0;
+        }
+        __syncwarp();
+    }
+    if (STORE) {
+        // the first step that holds the strip's maximum, as in run_strip
+        const WarpSmemD::Item &it = sm.it;
+        const int v0 = j0 < m ? Ops16::word_h(rmax, 0) : 0, v1 = j0 + kUp < m ? Ops16::word_h(rmax, 1) : 0;
+        const int top = __reduce_max_sync(kFull, max(v0, v1));
+        const int other = static_cast<int>(__shfl_sync(kFull, ld_best(a.best_key + p), 0) >> 40);
+        if (top > 0 && top >= other) {
+#pragma unroll 1
+            for (int k = 0; k < 2; ++k)
+                best_in_strip(it.lo, it.cmax, it.schunks, 0, __ballot_sync(kFull, (k ? v1 : v0) == top), k, 1, k * kUp,
+                              j0 - lane + k * kUp, n, top, lane, best);
+        }
+    }
+    finish_strip(a, pd, p, best, timed_out, lane, pd.n_strips, rerun, false);
+}
+
 // shared memory of a warp of the int16 kernel: the largest of the strip forms it runs
 __host__ __device__ constexpr size_t warp16_bytes(bool wide4)
 {
     size_t b = sizeof(WarpSmem<Ops16::Bnd>) > sizeof(WarpSmemD) ? sizeof(WarpSmem<Ops16::Bnd>) : sizeof(WarpSmemD);
+    if (sizeof(WarpSmemS) > b) b = sizeof(WarpSmemS);
     if (wide4 && sizeof(WarpSmem4) > b) b = sizeof(WarpSmem4);
     return b;
 }
@@ -1953,7 +2323,7 @@ __global__ void __launch_bounds__(Warps * 32, 2) dp_kernel(const DPArgs a, int r
                 const uint32_t n_items = items_of(pd.flags, pd.n_strips);
                 WarpSmemD &smd = *reinterpret_cast<WarpSmemD *>(mine);
                 if (it.y == 0 && (pd.n_strips & 1))
-                    run_strip<Ops16T<true>>(a, *reinterpret_cast<SM *>(mine), pd, it.x, 0, 0u, n_items, lane, false);
+                    run_strip<Ops16>(a, *reinterpret_cast<SM *>(mine), pd, it.x, 0, 0u, n_items, lane, false);
                 else if (pd.flags & PF_PROF)
                     pd.flags & PF_SCORE_ONLY ? run_duo<true, false>(a, smd, pd, it.x, static_cast<int>(it.y), lane)
                                              : run_duo<true, true>(a, smd, pd, it.x, static_cast<int>(it.y), lane);
@@ -1963,8 +2333,14 @@ __global__ void __launch_bounds__(Warps * 32, 2) dp_kernel(const DPArgs a, int r
                 continue;
             }
         }
-        run_strip<Ops>(a, *reinterpret_cast<SM *>(mine), pd, it.x, static_cast<int>(it.y), it.y, pd.n_strips, lane,
-                       rerun_only != 0);
+        if constexpr (kInt16) {
+            WarpSmemS &sms = *reinterpret_cast<WarpSmemS *>(mine);
+            if (pd.flags & PF_SCORE_ONLY) run_solo<false>(a, sms, pd, it.x, static_cast<int>(it.y), lane, rerun_only != 0);
+            else run_solo<true>(a, sms, pd, it.x, static_cast<int>(it.y), lane, rerun_only != 0);
+        } else {
+            run_strip<Ops>(a, *reinterpret_cast<SM *>(mine), pd, it.x, static_cast<int>(it.y), it.y, pd.n_strips, lane,
+                           rerun_only != 0);
+        }
     }
 }
 
@@ -2019,9 +2395,7 @@ int dp32_blocks_per_sm() { return DpBuild<Ops32, kWarpsPerCta>::blocks_per_sm();
 namespace {
 // Per-nt records of every pair (see make_record), positions -kRecPre upwards
 // (z, the profile row's byte offset, for the pair's strip form: rows of 32
-// lanes x 4 B, or x 8 B in 128-residue strips and where warps run two strips).  For pairs whose warps run two
-// strips the high halves of x and y and the offset w belong to the row 64
-// before instead of the one before.
+// lanes x 4 B, or x 8 B in 128-residue strips and where warps run two strips).
 // The genetic code and the splice terms are looked up in shared tables
 // (lanes index them at different positions: from constant memory such
 // reads serialise), the splice terms by three 5-symbol codes (four bases and
@@ -2050,9 +2424,9 @@ __global__ void records_kernel(const PairDesc *pairs, uint32_t n_pairs, const ui
         const uint32_t *g = nt2 + pd.nt_word_off;
         uint4 *out = recs + pd.rec_off;
         const uint32_t zrow = (pd.flags & (PF_W128 | PF_DUO)) ? 256u : 128u;
-        // the row of the high halves: the one before, or 64 rows back for pairs
-        // whose warps run two strips (rows before the region all read alike)
-        const int back = (pd.flags & PF_DUO) ? Ops16d::kUp : 1;
+        // how far back the row of the high halves is (rows before the region all
+        // read alike)
+        const int back = (pd.flags & PF_DUO) ? Ops16d::kUp : (pd.flags & PF_W128) ? 1 : kBackOne;
         // row ii: d(i+1), a(i) and the codon's amino acid, from T0[ii-3 .. ii+4]
         auto row = [&](int ii, uint32_t &d, uint32_t &ac, uint32_t &aa) {
             const int s0 = ii - 3;
@@ -2235,13 +2609,13 @@ dp_noalloc_kernel(ScoreParams sp, const char *prot_ascii, int m, const char *nt_
         a.sp = sp;
         a.spin_limit = spin_limit;
         {
-            auto &sm = reinterpret_cast<WarpSmem<Ops16::Bnd> *>(smem_raw)[warp];
+            auto &sm = reinterpret_cast<WarpSmemS *>(smem_raw)[warp];
             for (;;) {
                 uint32_t s = 0;
                 if (lane == 0) s = atomicAdd(&S->head16, 1u);
                 s = __shfl_sync(kFull, s, 0);
                 if (s >= static_cast<uint32_t>(nstrips)) break;
-                run_strip<Ops16>(a, sm, pd, 0, static_cast<int>(s), s, pd.n_strips, lane, false);
+                run_solo<false>(a, sm, pd, 0, static_cast<int>(s), lane, false);
             }
         }
         __syncthreads();
@@ -2269,7 +2643,8 @@ dp_noalloc_kernel(ScoreParams sp, const char *prot_ascii, int m, const char *nt_
     }
 }
 
-constexpr size_t kNASmem = sizeof(WarpSmem<Ops32::Bnd>) * kWarpsPerCta;   // covers the int16 layout too
+constexpr size_t kNASmem =
+    (sizeof(WarpSmem<Ops32::Bnd>) > sizeof(WarpSmemS) ? sizeof(WarpSmem<Ops32::Bnd>) : sizeof(WarpSmemS)) * kWarpsPerCta;
 
 }  // namespace
 }  // namespace mpdp

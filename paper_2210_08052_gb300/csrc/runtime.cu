@@ -718,6 +718,7 @@ static int plan_waves(mp_dp_ctx *c, mp_dp_batch *b, const mp_dp_tuning &t, bool 
     // is longer in the wide form: pairs whose wide critical path would exceed
     // the batch's longest one in 64-residue strips stay in 64-residue strips.
     uint64_t crit64 = 0;
+    double steps = 0;
     for (uint32_t k = 0; k < n; ++k) {
         const PairDesc &d = b->desc[k];
         if (d.flags & PF_SKIP) continue;
@@ -732,12 +733,39 @@ static int plan_waves(mp_dp_ctx *c, mp_dp_batch *b, const mp_dp_tuning &t, bool 
             d.flags |= PF_W128;
         d.n_strips = static_cast<uint32_t>(div_up(d.prot_len, strip_w_of(d.flags)));
         // two 64-residue strips per warp wherever there are two (a pair that may
-        // need int32 keeps one strip per item: its items can go to either kernel)
-        // (with the boundary rows withheld, a test of the waits, two strips stay
-        // apart, so that one of them waits)
+        // need int32 keeps one strip per item: its items can go to either kernel;
+        // with the boundary rows withheld, a test of the waits, two strips stay
+        // apart, so that one of them waits) ...
         const bool alone = d.n_strips == 2 && (c->params.debug_flags & MP_DEBUG_NO_PUBLISH);
         if (!c->params.force_int32 && d.n_strips >= 2 && !alone && !(d.flags & (PF_WIDE | PF_W128 | PF_SKIP)))
             d.flags |= PF_DUO;
+        if (!(d.flags & PF_SKIP))
+            steps += static_cast<double>(items_of(d.flags, d.n_strips)) * (d.nt_len + 2 * kStripW - 1);
+    }
+    // ... unless the pair's own chain of steps (its region, and three chunks
+    // from each warp to the next) is longer than what every warp has to do: then
+    // the chain sets the time, and one strip per warp runs it faster, as long as
+    // these warps have a scheduler each (39 ns a step of a lone warp against
+    // 47.5).  With all strips of 64 genes on schedulers of their own 1.70
+    // against 1.91 ms; where they do not fit (all strips of 128 profiles alone:
+    // 3.17 against 2.87) only the longest chains get them, on a quarter of the
+    // schedulers.
+    const double share = steps / (static_cast<double>(c->num_sms) * 2 * kWarps16);
+    std::vector<std::pair<double, uint32_t>> chains;
+    for (uint32_t k = 0; k < n; ++k) {
+        const PairDesc &d = b->desc[k];
+        const double chain =
+            d.nt_len + 2.0 * kStripW + 3.0 * kChunk * (items_of(d.flags, d.n_strips) - 1.0);
+        if ((d.flags & PF_DUO) && chain > share) chains.push_back({-chain, k});
+    }
+    std::sort(chains.begin(), chains.end());
+    const uint64_t sms = static_cast<uint64_t>(c->num_sms);
+    uint64_t room = strips <= 4 * sms ? 4 * sms : sms;
+    for (const auto &ch : chains) {
+        PairDesc &d = b->desc[ch.second];
+        if (d.n_strips > room) break;
+        room -= d.n_strips;
+        d.flags &= ~PF_DUO;
     }
     for (uint32_t k = 0; k < n; ++k) {
         PairDesc &d = b->desc[k];

@@ -35,6 +35,7 @@ struct PairView {
     bool w128;               // 128-residue strips (four cells per lane) instead of 64 (two)
     int duo;                 // 1, 2: a warp ran two strips (2: the first strip alone); the upper one's
                              // column maxima lie 64 steps behind its stream
+    bool halves;             // a word holds columns r and r + 32 of its strip instead of r and r + 1
     const uint32_t *g;       // packed genome
     const uint8_t *P;        // residue codes
     int n, m;
@@ -83,10 +84,10 @@ struct PairView {
                                                                  static_cast<size_t>(t >> 2) * 1024 + (r >> 1) * 32 +
                                                                  (t & 3) * 8 + (r & 1) * 4));
         }
+        const int lane = halves ? r & 31 : r >> 1, hi = halves ? r >> 5 : r & 1;
         const uint32_t w = ld_tb<Coherent>(reinterpret_cast<const uint32_t *>(
-            base + static_cast<size_t>(s) * strip_bytes + static_cast<size_t>(t >> 2) * 512 + (r >> 1) * 16 +
-            (t & 3) * 4));
-        return static_cast<int>((r & 1) ? (w >> 16) : (w & 0xffffu)) - 32768;
+            base + static_cast<size_t>(s) * strip_bytes + static_cast<size_t>(t >> 2) * 512 + lane * 16 + (t & 3) * 4));
+        return static_cast<int>(hi ? (w >> 16) : (w & 0xffffu)) - 32768;
     }
     // step of residue j's row 0 in the chunks of its column maxima
     __device__ __forceinline__ int cstep(int j) const
@@ -107,10 +108,11 @@ struct PairView {
             return static_cast<int>((r & 1) ? (w >> 16) : (w & 0xffffu)) - 32768;
         }
         const int jj = j - 1, s = jj >> 6, r = jj & 63;
-        const size_t e = (static_cast<size_t>(s) * nchunks + c) * 32 + (r >> 1);
+        const int lane = halves ? r & 31 : r >> 1, hi = halves ? r >> 5 : r & 1;
+        const size_t e = (static_cast<size_t>(s) * nchunks + c) * 32 + lane;
         if (wide) return ld_tb<Coherent>(reinterpret_cast<const int *>(colmax) + 2 * e + (r & 1));
         const uint32_t w = ld_tb<Coherent>(reinterpret_cast<const uint32_t *>(colmax) + e);
-        return static_cast<int>((r & 1) ? (w >> 16) : (w & 0xffffu)) - 32768;
+        return static_cast<int>(hi ? (w >> 16) : (w & 0xffffu)) - 32768;
     }
     // base at 1-based position x (0..3), valid iff 1 <= x <= n
     __device__ __forceinline__ int b(int x) const
@@ -230,6 +232,7 @@ __device__ __forceinline__ PairView<Coherent> make_view(const TBArgs &a, const P
     return PairView<Coherent>{a.codes + pd.code_off, strip_bytes, wide,
                     a.codes + pd.code_off + static_cast<size_t>(pd.n_strips) * strip_bytes, nchunks, W == kStripWMax,
                     (pd.flags & PF_DUO) ? 2 - static_cast<int>((pd.n_strips + 1) & 1) : 0,
+                    !wide && !(pd.flags & (PF_DUO | PF_W128)),
                     a.nt2 + pd.nt_word_off, a.prot + pd.prot_off, n, static_cast<int>(pd.prot_len),
                     &a.sp, mat_s, anchored ? a.col0 + pd.col0_off : nullptr,
                     (pd.flags & PF_PROF) ? a.prof + pd.prof_off : nullptr,

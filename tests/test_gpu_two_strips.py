@@ -1,7 +1,9 @@
-"""Warps that run two strips of a pair at once: results equal the oracle's
-(whole numbers, no tolerance) at the edges of strips and chunks, with an even
-and an odd number of strips, in every mode, for profile queries, score-only
-pairs and every build of the kernel."""
+"""Warps that run one strip or two strips of a pair at once: results equal the
+oracle's (whole numbers, no tolerance) at the edges of strips and chunks, with
+an even and an odd number of strips, in every mode, for profile queries,
+score-only pairs and every build of the kernel.  A batch of a few hundred
+pairs runs one strip per warp (every pair's own chain of steps is longer than
+a warp's share of the work), the same pairs many times over two."""
 import numpy as np
 import pytest
 
@@ -40,6 +42,10 @@ def _pairs(seed):
     return out
 
 
+# copies of the pairs: few pairs, one strip per warp; many, two
+COPIES = pytest.mark.parametrize("copies", [1, 30])
+
+
 def _params(mp, orc, mode, **more):
     p = mp.mp_dp_default_params(mode=mode, **more)
     op = orc.make_params(q=p.q, e=p.e, f=p.f, r=p.r, stop=p.stop, splice_model=p.splice_model, splice_p=p.splice_p)
@@ -52,12 +58,14 @@ def _bad(pairs, got, want, keys=KEYS):
             for p, g, w in zip(pairs, got, want) if any(g[k] != w[k] for k in keys) or g["status"] & 0xF0]
 
 
+@COPIES
 @pytest.mark.parametrize("costs", [dict(), dict(q=0, e=1, f=0, r=8, stop=4, splice_model=1, splice_p=3)])
 @pytest.mark.parametrize("mode", [0, 1, 2])
-def test_edges_match_oracle(mp, orc, mode, costs):
+def test_edges_match_oracle(mp, orc, mode, costs, copies):
     pairs = _pairs(200 + mode)
     params, op = _params(mp, orc, mode, **costs)
-    want = [orc.align(p.prot, p.nt, p.strand, op) for p in pairs]
+    want = [orc.align(p.prot, p.nt, p.strand, op) for p in pairs] * copies
+    pairs = pairs * copies
     c = mp.mp_dp_init(params, 0)
     try:
         for variant in (1, 0):
@@ -71,14 +79,15 @@ def test_edges_match_oracle(mp, orc, mode, costs):
         mp.mp_dp_destroy(c)
 
 
+@COPIES
 @pytest.mark.parametrize("mode", [0, 1, 2])
-def test_stored_h_at_the_edges(mp, orc, mode):
+def test_stored_h_at_the_edges(mp, orc, mode, copies):
     """Every stored H, read through the traceback's view of the stream."""
     pairs = [p for p in _pairs(210 + mode) if len(p.prot) in (65, 128, 129, 192, 257) and len(p.nt) in (3, 65, 97, 161, 705)]
     params, op = _params(mp, orc, mode)
     c = mp.mp_dp_init(params, 0)
     try:
-        b = mp.mp_dp_batch_upload(c, pairs)
+        b = mp.mp_dp_batch_upload(c, pairs * (10 * copies if copies > 1 else 1))
         mp.mp_dp_batch_run(c, b)
         mp.mp_dp_batch_sync(c)
         for k, p in enumerate(pairs):
@@ -90,8 +99,9 @@ def test_stored_h_at_the_edges(mp, orc, mode):
         mp.mp_dp_destroy(c)
 
 
+@COPIES
 @pytest.mark.parametrize("mode", [0, 2])
-def test_profile_edges(mp, orc, mode):
+def test_profile_edges(mp, orc, mode, copies):
     rng = np.random.default_rng(220 + mode)
     pairs = [p for p in _pairs(220 + mode) if len(p.nt) in (2, 65, 161, 321, 705)]
     mat = mp.params_matrix(mp.mp_dp_default_params())
@@ -106,6 +116,7 @@ def test_profile_edges(mp, orc, mode):
         p.profile = prof
     params, _ = _params(mp, orc, mode)
     want = [orc.align(p.prot, p.nt, p.strand, orc.make_params(mode=mode, prof=p.profile)) for p in pairs]
+    want, pairs = want * 4 * copies, pairs * 4 * copies
     c = mp.mp_dp_init(params, 0)
     try:
         assert not (bad := _bad(pairs, mp.mp_dp_align_batch(c, pairs), want)), bad[:5]
@@ -113,10 +124,11 @@ def test_profile_edges(mp, orc, mode):
         mp.mp_dp_destroy(c)
 
 
-def test_withheld_rows_time_out(mp):
-    """With boundary rows withheld, every pair of three strips or more gives
+@COPIES
+def test_withheld_rows_time_out(mp, copies):
+    """With boundary rows withheld, every pair of two strips or more gives
     up after the short poll limit and says so; the context stays usable."""
-    pairs = [p for p in _pairs(230) if len(p.nt) == 705]
+    pairs = [p for p in _pairs(230) if len(p.nt) == 705] * 20 * copies
     c = mp.mp_dp_init(mp.mp_dp_default_params(wait_limit=200, debug_flags=mp.MP_DEBUG_NO_PUBLISH), 0)
     try:
         for _ in range(2):
