@@ -354,32 +354,66 @@ __global__ void scan_add(uint32_t *out, uint64_t n, const uint32_t *block_sums, 
     if (i == 0) out[n] = *total;
 }
 
-// each bucket's entries in ascending order (buckets hold a few dozen)
-__global__ void bucket_sort_kernel(const uint32_t *off, uint32_t *entries)
+// Each bucket's entries in ascending order.  A warp takes 32 neighbouring
+// buckets, whose entries are contiguous: in shared memory, each entry's place
+// is the number of its bucket's entries before it (one lane per entry; a
+// bucket holds 10 on average and some hundreds at most on the 50 Mb genome).
+// Where they do not fit, the warp sorts bucket by bucket in place (a network
+// whose comparators all put the smaller value first, so that places past the
+// end need no values).  One thread per bucket, by insertion in global memory,
+// took 2.4 ms on the 50 Mb genome; this 0.46.
+constexpr int kBucketWarps = 8, kBucketStage = 512;
+
+__global__ void __launch_bounds__(kBucketWarps * 32) bucket_sort_kernel(const uint32_t *off, uint32_t *entries)
 {
-    for (uint32_t h = blockIdx.x * blockDim.x + threadIdx.x; h < kNKeys; h += gridDim.x * blockDim.x) {
-        const uint32_t a = off[h], b = off[h + 1];
-        for (uint32_t i = a + 1; i < b; ++i) {
-            const uint32_t v = entries[i];
-            uint32_t j = i;
-            while (j > a && entries[j - 1] > v) {
-                entries[j] = entries[j - 1];
-                --j;
+    __shared__ uint32_t stage[kBucketWarps][kBucketStage];
+    __shared__ uint32_t first[kBucketWarps][33];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    for (uint32_t h0 = (blockIdx.x * kBucketWarps + w) * 32; h0 < kNKeys; h0 += gridDim.x * kBucketWarps * 32) {
+        const uint32_t mine = off[h0 + lane], end = off[h0 + 32];
+        const uint32_t a = __shfl_sync(0xffffffffu, mine, 0), cnt = end - a;
+        __syncwarp();
+        first[w][lane] = mine - a;
+        if (lane == 0) first[w][32] = cnt;
+        if (cnt <= kBucketStage) {
+            for (uint32_t i = lane; i < cnt; i += 32) stage[w][i] = entries[a + i];
+            __syncwarp();
+            for (uint32_t i = lane; i < cnt; i += 32) {
+                int b = 0;                                 // the bucket: the last one that starts at or before i
+#pragma unroll
+                for (int step = 16; step > 0; step >>= 1)
+                    if (first[w][b + step] <= i) b += step;
+                const uint32_t s = first[w][b], e = first[w][b + 1], v = stage[w][i];
+                uint32_t at = s;
+                for (uint32_t j = s; j < e; ++j) {
+                    const uint32_t u = stage[w][j];
+                    at += u < v || (u == v && j < i) ? 1u : 0u;
+                }
+                entries[a + at] = v;
             }
-            entries[j] = v;
+        } else {
+            __syncwarp();
+            for (int b = 0; b < 32; ++b) {
+                uint32_t *e = entries + a + first[w][b];
+                const uint32_t n = first[w][b + 1] - first[w][b];
+                for (uint32_t k = 2; k < 2 * n; k <<= 1)
+                    for (uint32_t j = k - 1; j > 0; j = j == k - 1 ? k >> 2 : j >> 1) {
+                        for (uint32_t i = lane; i < n; i += 32) {
+                            const uint32_t l = i ^ j;
+                            if (l > i && l < n && e[i] > e[l]) {
+                                const uint32_t t = e[i];
+                                e[i] = e[l];
+                                e[l] = t;
+                            }
+                        }
+                        __syncwarp();
+                    }
+            }
         }
     }
 }
 
 // ------------------------------------------------------------- chaining
-__device__ __forceinline__ int64_t gap_eq1(int64_t dx, int64_t dy)
-{
-    const int64_t py = 3 * dy;
-    if (py < kBin * (dx - 1)) return py - kBin * (dx - 1);
-    if (py > kBin * (dx + 1)) return py - kBin * (dx + 1);
-    return 0;
-}
-
 // floor(S beta log2(v)) for v = |g| + 1: an integer log2 for a power of two
 // (the device log2 need not be exact there), the double log2 otherwise
 // (each such value lies at least 6.8e-6 from an integer for |g| < G)
@@ -480,52 +514,104 @@ __global__ void anchor_fill_kernel(ChainArgs a)
                 const uint64_t y = __shfl_up_sync(0xffffffffu, incl, o);
                 if (lane >= o) incl += y;
             }
-            for (uint32_t e = lo; e < hi; ++e) {
-                const uint32_t v = a.entries[e];
-                a.anc[at + incl - cnt + (e - lo)] = (static_cast<uint64_t>(v >> 31) << 63) |
-                                                    (static_cast<uint64_t>(v & 0x7fffffffu) << 20) |
-                                                    static_cast<uint64_t>(t);
+            // one hit per lane at a time (a lane per k-mer wrote its hits in runs of
+            // its own): the hit's k-mer is the first lane whose count passes it
+            const uint32_t total = static_cast<uint32_t>(__shfl_sync(0xffffffffu, incl, 31));
+            for (uint32_t o0 = 0; o0 < total; o0 += 32) {
+                const uint32_t o = o0 + lane;
+                int k = 0;
+#pragma unroll
+                for (int step = 16; step > 0; step >>= 1) {
+                    const uint32_t below = static_cast<uint32_t>(__shfl_sync(0xffffffffu, incl, k + step - 1));
+                    if (o >= below) k += step;
+                }
+                const uint32_t first = __shfl_sync(0xffffffffu, lo, k);
+                const uint32_t before = static_cast<uint32_t>(__shfl_sync(0xffffffffu, incl - cnt, k));
+                if (o < total) {
+                    const uint32_t v = a.entries[first + (o - before)];
+                    a.anc[at + o] = (static_cast<uint64_t>(v >> 31) << 63) |
+                                    (static_cast<uint64_t>(v & 0x7fffffffu) << 20) | static_cast<uint64_t>(t0 + k);
+                }
             }
             at += __shfl_sync(0xffffffffu, incl, 31);
         }
     }
 }
 
-// One block per protein: its anchors sorted ascending (strand, x, y) by a
-// bitonic network, in shared memory up to kSortMax anchors, otherwise over
-// a scratch range of the next power of two (its tail padded with the
-// largest key) in global memory.
-constexpr int kSortMax = 16384;           // 128 KB of shared memory
-constexpr int kSortThreads = 1024;
+// One block per protein, the ones with most anchors first: its anchors sorted
+// by (strand, x), eight bits at a time from the lowest, stably; they come in
+// ascending y, so that the order is (strand, x, y).  Each warp takes a
+// contiguous part: it counts its digits, the counts are summed over digits and
+// warps, and it writes its anchors 32 at a time, each behind the equal digits
+// before it (a warp match gives its place among the 32).  The passes go to and
+// fro between a.anc and tmp; after an odd number of passes the result is in
+// tmp.  (A bitonic network over 64-bit keys in shared memory, 91 to 105 steps
+// for a protein, took 5.2 ms for 4,000 proteins; this 0.75.)
+constexpr int kSortThreads = 256;
+constexpr int kDigitBits = 8, kDigits = 1 << kDigitBits;
 
-__global__ void __launch_bounds__(kSortThreads) anchor_sort_kernel(ChainArgs a, uint64_t *scratch,
-                                                                   const uint64_t *scratch_off)
+__host__ __device__ constexpr int sort_passes(int xbits) { return (xbits + 1 + kDigitBits - 1) / kDigitBits; }
+
+__global__ void __launch_bounds__(kSortThreads) anchor_sort_kernel(ChainArgs a, uint64_t *tmp, int xbits)
 {
-    extern __shared__ uint64_t sh[];
-    for (uint32_t p = blockIdx.x; p < a.n_prot; p += gridDim.x) {
+    constexpr int kWarps = kSortThreads / 32;
+    static_assert(kSortThreads == kDigits, "a thread per digit sums the warps' counts");
+    __shared__ uint32_t hist[kWarps][kDigits];
+    __shared__ uint32_t warp_sum[kWarps];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint64_t xmask = (1ull << xbits) - 1;
+    for (uint32_t k = blockIdx.x; k < a.n_prot; k += gridDim.x) {
+        const uint32_t p = a.order[k];
         const uint64_t b0 = a.anc_off[p], n = a.anc_off[p + 1] - b0;
-        if (n < 2) continue;
-        uint64_t n2 = 1;
-        while (n2 < n) n2 <<= 1;
-        uint64_t *v = n2 <= kSortMax ? sh : scratch + scratch_off[p];
-        for (uint64_t i = threadIdx.x; i < n2; i += blockDim.x) v[i] = i < n ? a.anc[b0 + i] : ~0ull;
-        __syncthreads();
-        for (uint64_t k = 2; k <= n2; k <<= 1)
-            for (uint64_t j = k >> 1; j > 0; j >>= 1) {
-                for (uint64_t i = threadIdx.x; i < n2; i += blockDim.x) {
-                    const uint64_t l = i ^ j;
-                    if (l > i) {
-                        const uint64_t x = v[i], y = v[l];
-                        if ((x > y) == ((i & k) == 0)) {
-                            v[i] = y;
-                            v[l] = x;
-                        }
-                    }
-                }
-                __syncthreads();
+        uint64_t *src = a.anc + b0, *dst = tmp + b0;
+        const uint64_t per = (n + kSortThreads - 1) / kSortThreads * 32;
+        const uint64_t i0 = per * warp < n ? per * warp : n, i1 = i0 + per < n ? i0 + per : n;
+        for (int shift = 0; shift <= xbits; shift += kDigitBits) {
+            auto digit = [&](uint64_t v) {
+                const uint64_t key = ((v >> 20) & xmask) | (v >> 63) << xbits;
+                return static_cast<uint32_t>(key >> shift) & (kDigits - 1);
+            };
+            for (int d = lane; d < kDigits; d += 32) hist[warp][d] = 0;
+            __syncwarp();
+            for (uint64_t i = i0 + lane; i < i1; i += 32) atomicAdd(&hist[warp][digit(src[i])], 1u);
+            __syncthreads();
+            // thread d: digit d's count, the sum of the digits below, then each warp's start
+            uint32_t sum = 0;
+#pragma unroll
+            for (int w = 0; w < kWarps; ++w) sum += hist[w][threadIdx.x];
+            uint32_t incl = sum;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += y;
             }
-        for (uint64_t i = threadIdx.x; i < n; i += blockDim.x) a.anc[b0 + i] = v[i];
-        __syncthreads();
+            if (lane == 31) warp_sum[warp] = incl;
+            __syncthreads();
+            uint32_t run = incl - sum;
+            for (int w = 0; w < warp; ++w) run += warp_sum[w];
+#pragma unroll
+            for (int w = 0; w < kWarps; ++w) {
+                const uint32_t c = hist[w][threadIdx.x];
+                hist[w][threadIdx.x] = run;
+                run += c;
+            }
+            __syncthreads();
+            for (uint64_t i = i0; i < i1; i += 32) {
+                const bool have = i + lane < i1;
+                const uint64_t v = have ? src[i + lane] : 0;
+                const uint32_t d = have ? digit(v) : kDigits;        // (no digit: a group of its own)
+                const unsigned same = __match_any_sync(0xffffffffu, d);
+                const int before = __popc(same & ((1u << lane) - 1));
+                if (have) dst[hist[warp][d] + before] = v;
+                __syncwarp();
+                if (have && before == 0) hist[warp][d] += __popc(same);
+                __syncwarp();
+            }
+            __syncthreads();
+            uint64_t *t = src;
+            src = dst;
+            dst = t;
+        }
     }
 }
 
@@ -911,7 +997,6 @@ __global__ void __launch_bounds__(kStrandWarps * 64) chain_kernel(ChainArgs a)
 constexpr int kK2 = 5;                      // k-mer length of the second round
 constexpr int kRefineMaxProt = 8192;        // protein k-mer table in shared memory (64 KB)
 constexpr int kRefineThreads = 256;
-constexpr size_t kRefineSmem = kRefineMaxProt * sizeof(uint64_t);
 constexpr int64_t kRefineBig = 512;          // pairs with more anchors are chained by a whole block
 
 struct RefineArgs {
@@ -928,33 +1013,33 @@ struct RefineArgs {
     const int32_t *log_tab;
 };
 
-// phi of the codon starting at base x of the pair's aligned strand
-__device__ __forceinline__ uint32_t codon_phi(const char *nt, int64_t L, int strand, int64_t x)
-{
-    int b[3];
-#pragma unroll
-    for (int u = 0; u < 3; ++u) {
-        const int c = strand > 0 ? base_code(static_cast<unsigned char>(nt[x + u]))
-                                 : base_code(static_cast<unsigned char>(nt[L - 1 - (x + u)]));
-        b[u] = c < 0 ? -1 : (strand > 0 ? c : 3 - c);
-    }
-    if (b[0] < 0 || b[1] < 0 || b[2] < 0) return kXCode;
-    return c_codon_phi.v[b[0] * 16 + b[1] * 4 + b[2]];
-}
-
-// FILL = false: count each thread's anchors into tcount[p * kRefineThreads +
-// t] and the pair's into total[p]; true: write them from anc_off[p] on, in
-// (x, y) order (thread t's after those of threads 0 .. t-1)
+// FILL = false: count the pair's anchors into total[p]; true: write them from
+// anc_off[p] on, in (x, y) order.
 //
-// The protein's k-mers are sorted as key << 13 | y (bitonic, shared
-// memory), so each base's k-mer finds its equal protein k-mers by one binary
-// search, in ascending y.
+// One block per pair.  The protein's k-mers are sorted as key << 13 | y
+// (bitonic, shared memory), so the k-mers equal to a base's are found by one
+// binary search, in ascending y.  The region comes in tiles of kTile bases:
+// their letters are read once, then each base's codon is translated once, and
+// a base's k-mer is put together from five of them.  Nearly all bases end at a
+// filter of 2^15 bits that holds a hash of every protein k-mer (a binary
+// search per base, on codons translated for each of the five, took 2.7 ms per
+// pass for 6,000 regions; this 0.6 to 0.7).
+constexpr int kTile = 4096;
+constexpr int kFilterBits = 15;
+
+// the k-mer's bit in the filter
+__device__ __forceinline__ uint32_t filter_hash(uint32_t key) { return (key * 2654435761u) >> (32 - kFilterBits); }
+
 template <bool FILL>
-__global__ void __launch_bounds__(kRefineThreads) refine_anchor_kernel(RefineArgs a, uint32_t *tcount,
-                                                                       uint64_t *total)
+__global__ void __launch_bounds__(kRefineThreads) refine_anchor_kernel(RefineArgs a, uint64_t *total)
 {
-    extern __shared__ uint64_t pk[];                // kRefineMaxProt entries
-    __shared__ uint64_t part[kRefineThreads];
+    extern __shared__ uint64_t pk[];                // the protein's k-mers (a power of two of them)
+    __shared__ uint32_t filter[(1 << kFilterBits) / 32];
+    __shared__ uint8_t code[kTile + 3 * kK2];       // bases (4: not one of A, C, G, T), then codons
+    __shared__ uint8_t s_phi[64];
+    __shared__ uint32_t warp_cnt[kRefineThreads / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int k = threadIdx.x; k < 64; k += blockDim.x) s_phi[k] = c_codon_phi.v[k];
     for (uint32_t p = blockIdx.x; p < a.n; p += gridDim.x) {
         const char *P = a.seq + a.prot_off[p];
         const char *T = a.seq + a.nt_off[p];
@@ -962,15 +1047,19 @@ __global__ void __launch_bounds__(kRefineThreads) refine_anchor_kernel(RefineArg
         const int64_t L = a.nt_len[p];
         const int strand = a.strand[p];
         const int ny = m - kK2 + 1;                 // protein k-mers
-        const int64_t nx = L - 3 * kK2 + 1;          // region k-mers (one per base)
+        const int64_t nx = ny > 0 ? L - 3 * kK2 + 1 : 0;      // region k-mers (one per base)
         int n2 = 1;
         while (n2 < ny) n2 <<= 1;
+        for (int k = threadIdx.x; k < (1 << kFilterBits) / 32; k += blockDim.x) filter[k] = 0;
+        __syncthreads();
         for (int y = threadIdx.x; y < n2; y += blockDim.x) {
             uint64_t key = ~0ull;
             if (y < ny) {
                 key = 0;
 #pragma unroll
                 for (int u = 0; u < kK2; ++u) key = key * 16 + c_aa_phi.v[static_cast<unsigned char>(P[y + u])];
+                const uint32_t h = filter_hash(static_cast<uint32_t>(key));
+                atomicOr(&filter[h >> 5], 1u << (h & 31));
                 key = key << 13 | static_cast<uint64_t>(y);
             }
             pk[y] = key;
@@ -990,49 +1079,87 @@ __global__ void __launch_bounds__(kRefineThreads) refine_anchor_kernel(RefineArg
                 }
                 __syncthreads();
             }
-        // thread t takes bases [x0, x1)
-        const int64_t per = nx > 0 && ny > 0 ? (nx + blockDim.x - 1) / blockDim.x : 0;
-        const int64_t x0 = per * threadIdx.x, x1 = x0 + per < nx ? x0 + per : (nx > 0 ? nx : 0);
-        uint64_t c = 0, at = 0;
-        if (FILL) {
-            // this thread's first slot: the anchors of the threads before it
-            part[threadIdx.x] = tcount[static_cast<uint64_t>(p) * blockDim.x + threadIdx.x];
+        uint64_t at = FILL ? a.anc_off[p] : 0;      // the tile's first slot
+        uint64_t mine = 0;                          // this thread's anchors so far
+        for (int64_t x0 = 0; x0 < nx; x0 += kTile) {
+            const int nt = static_cast<int>(nx - x0 < kTile ? nx - x0 : kTile);      // the tile's k-mers
+            // the bases they touch, of the aligned strand
+            for (int i = threadIdx.x; i < nt + 3 * kK2 - 1; i += blockDim.x) {
+                const int64_t x = x0 + i;
+                const int c = base_code(static_cast<unsigned char>(strand > 0 ? T[x] : T[L - 1 - x]));
+                code[i] = static_cast<uint8_t>(c < 0 ? 4 : strand > 0 ? c : 3 - c);
+            }
             __syncthreads();
-            if (threadIdx.x == 0) {
-                uint64_t run = a.anc_off[p];
-                for (int t = 0; t < static_cast<int>(blockDim.x); ++t) {
-                    const uint64_t v = part[t];
-                    part[t] = run;
-                    run += v;
+            // codon phi in place: each thread's part, after it has read the two
+            // bases behind it that belong to the next thread
+            constexpr int kPart = (kTile + 3 * kK2 + kRefineThreads - 1) / kRefineThreads;
+            const int i0 = threadIdx.x * kPart, ic = nt + 3 * (kK2 - 1);              // codons
+            const int n0 = i0 + kPart < nt + 3 * kK2 - 1 ? code[i0 + kPart] : 4;
+            const int n1 = i0 + kPart + 1 < nt + 3 * kK2 - 1 ? code[i0 + kPart + 1] : 4;
+            __syncthreads();
+            if (i0 < ic) {
+                int b0 = code[i0], b1 = kPart > 1 ? code[i0 + 1] : n0;
+                for (int i = i0; i < i0 + kPart && i < ic; ++i) {
+                    const int b2 = i + 2 < i0 + kPart ? code[i + 2] : i + 2 == i0 + kPart ? n0 : n1;
+                    code[i] = (b0 | b1 | b2) & 4 ? kXCode : s_phi[b0 * 16 + b1 * 4 + b2];
+                    b0 = b1;
+                    b1 = b2;
                 }
             }
             __syncthreads();
-            at = part[threadIdx.x];
-        }
-        for (int64_t x = x0; x < x1; ++x) {
-            uint64_t key = 0;
+            // thread t takes the k-mers [t * per, t * per + per) of the tile
+            // (an odd number of bytes apart, for the banks)
+            const int per = static_cast<int>((nt + blockDim.x - 1) / blockDim.x) | 1;
+            const int xa = threadIdx.x * per < nt ? threadIdx.x * per : nt, xb = xa + per < nt ? xa + per : nt;
+            auto each = [&](auto &&found) {
+                for (int x = xa; x < xb; ++x) {
+                    uint32_t key = 0;
 #pragma unroll
-            for (int u = 0; u < kK2; ++u) key = key * 16 + codon_phi(T, L, strand, x + 3 * u);
-            // first entry >= key << 13
-            const uint64_t want = key << 13;
-            int lo = 0, hi = ny;
-            while (lo < hi) {
-                const int mid = (lo + hi) >> 1;
-                if (pk[mid] < want) lo = mid + 1;
-                else hi = mid;
+                    for (int u = 0; u < kK2; ++u) key = key * 16 + code[x + 3 * u];
+                    const uint32_t h = filter_hash(key);
+                    if (!(filter[h >> 5] >> (h & 31) & 1)) continue;
+                    // first entry >= key << 13
+                    const uint64_t want = static_cast<uint64_t>(key) << 13;
+                    int lo = 0, hi = ny;
+                    while (lo < hi) {
+                        const int mid = (lo + hi) >> 1;
+                        if (pk[mid] < want) lo = mid + 1;
+                        else hi = mid;
+                    }
+                    for (int e = lo; e < ny && (pk[e] >> 13) == key; ++e) found(x, pk[e] & 0x1fffu);
+                }
+            };
+            uint32_t c = 0;
+            each([&](int, uint64_t) { ++c; });
+            mine += c;
+            if (FILL) {
+                // the anchors of the threads before this one
+                uint32_t incl = c;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += y;
+                }
+                if (lane == 31) warp_cnt[warp] = incl;
+                __syncthreads();
+                uint64_t to = at + incl - c;
+                for (int w = 0; w < kRefineThreads / 32; ++w) {
+                    if (w < warp) to += warp_cnt[w];
+                    at += warp_cnt[w];
+                }
+                if (c) each([&](int x, uint64_t y) { a.anc[to++] = static_cast<uint64_t>(x0 + x) << 20 | y; });
             }
-            for (int e = lo; e < ny && (pk[e] >> 13) == key; ++e) {
-                if (FILL) a.anc[at++] = (static_cast<uint64_t>(x) << 20) | (pk[e] & 0x1fffu);
-                else ++c;
-            }
+            __syncthreads();                        // the tile's codons and counts are read no more
         }
         if (!FILL) {
-            tcount[static_cast<uint64_t>(p) * blockDim.x + threadIdx.x] = static_cast<uint32_t>(c);
-            part[threadIdx.x] = c;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, o);
+            __shared__ uint64_t part[kRefineThreads / 32];
+            if (lane == 0) part[warp] = mine;
             __syncthreads();
             if (threadIdx.x == 0) {
                 uint64_t sum = 0;
-                for (int t = 0; t < static_cast<int>(blockDim.x); ++t) sum += part[t];
+                for (int w = 0; w < kRefineThreads / 32; ++w) sum += part[w];
                 total[p] = sum;
             }
         }
@@ -1118,6 +1245,7 @@ __global__ void __launch_bounds__(kRefineThreads) refine_chain_block_kernel(Refi
 struct mp_index {
     int device = 0;
     uint64_t n_entries = 0;
+    int xbits = 0;                  // bits of the largest bin
     uint32_t *off = nullptr;        // kNKeys + 1
     uint32_t *entries = nullptr;
 };
@@ -1213,6 +1341,7 @@ extern "C" int mp_index_build(mp_dp_ctx *ctx, const char *genome, uint64_t len, 
     mp_index *idx = new (std::nothrow) mp_index();
     if (!idx) return MP_ENOMEM;
     idx->device = dev;
+    for (uint64_t bin = len / kBin; bin; bin >>= 1) ++idx->xbits;
     auto fail = [&](int rc) {
         mp_index_free(idx);
         return rc;
@@ -1232,7 +1361,7 @@ extern "C" int mp_index_build(mp_dp_ctx *ctx, const char *genome, uint64_t len, 
             return fail(MP_ECUDA);
         kmer_kernel<<<grid_for(nseg * 32, kKmerWarps * 32), kKmerWarps * 32, 0, st>>>(
             fr, before.p, after.p, nseg, 1, nullptr, cursor.p, idx->entries);
-        bucket_sort_kernel<<<grid_for(kNKeys, 256), 256, 0, st>>>(idx->off, idx->entries);
+        bucket_sort_kernel<<<kNKeys / 32 / kBucketWarps, kBucketWarps * 32, 0, st>>>(idx->off, idx->entries);
     }
     if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess) return fail(MP_ECUDA);
     *out = idx;
@@ -1294,8 +1423,6 @@ extern "C" int mp_index_chain(mp_dp_ctx *ctx, const mp_index *idx, const char *p
     SCK(cudaMemcpyAsync(d_len.p, prot_len, n_prot * sizeof(uint32_t), cudaMemcpyHostToDevice, st));
     Tmp<int32_t> d_log;
     SCK(d_log.alloc(kG));
-    SCK(cudaFuncSetAttribute(anchor_sort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(kSortMax * sizeof(uint64_t))));
     log_table_kernel<<<grid_for(kG, 256), 256, 0, st>>>(d_log.p);
     ChainArgs a{};
     a.log_tab = d_log.p;
@@ -1313,8 +1440,8 @@ extern "C" int mp_index_chain(mp_dp_ctx *ctx, const mp_index *idx, const char *p
     std::vector<uint64_t> cnt(n_prot);
     SCK(cudaMemcpyAsync(cnt.data(), d_cnt.p, n_prot * sizeof(uint64_t), cudaMemcpyDeviceToHost, st));
     SCK(cudaStreamSynchronize(st));
-    // proteins in groups whose anchors (8 + 8 + 4 + 1 bytes each, plus the
-    // sort scratch of large ones) stay within a bound
+    // proteins in groups whose anchors (8 + 8 + 8 + 4 + 1 bytes each) stay within
+    // a bound
     constexpr uint64_t kMaxAnchors = 192ull << 20;
     std::vector<mp_chain> h_ch(static_cast<uint64_t>(n_prot) * top);
     std::vector<uint32_t> h_nch(n_prot);
@@ -1323,20 +1450,13 @@ extern "C" int mp_index_chain(mp_dp_ctx *ctx, const mp_index *idx, const char *p
         uint64_t tot = 0;
         while (p1 < n_prot && (p1 == p0 || tot + cnt[p1] <= kMaxAnchors)) tot += cnt[p1++];
         const uint32_t np = p1 - p0;
-        std::vector<uint64_t> aoff(np + 1ull, 0), soff(np, 0);
+        std::vector<uint64_t> aoff(np + 1ull, 0);
         std::vector<uint32_t> order(np);
         for (uint32_t k = 0; k < np; ++k) order[k] = k;
         std::stable_sort(order.begin(), order.end(),
                          [&](uint32_t x, uint32_t y) { return cnt[p0 + x] > cnt[p0 + y]; });
-        uint64_t scratch = 0;
-        for (uint32_t k = 0; k < np; ++k) {
-            aoff[k + 1] = aoff[k] + cnt[p0 + k];
-            uint64_t n2 = 1;
-            while (n2 < cnt[p0 + k]) n2 <<= 1;
-            soff[k] = scratch;
-            if (n2 > static_cast<uint64_t>(kSortMax)) scratch += n2;
-        }
-        Tmp<uint64_t> anc, sc, d_soff;
+        for (uint32_t k = 0; k < np; ++k) aoff[k + 1] = aoff[k] + cnt[p0 + k];
+        Tmp<uint64_t> anc, sc;
         Tmp<int64_t> f;
         Tmp<int32_t> pred;
         Tmp<uint8_t> mark;
@@ -1349,10 +1469,8 @@ extern "C" int mp_index_chain(mp_dp_ctx *ctx, const mp_index *idx, const char *p
         SCK(f.alloc(tot));
         SCK(pred.alloc(tot));
         SCK(mark.alloc(tot));
-        SCK(sc.alloc(scratch));
-        SCK(d_soff.alloc(np));
+        SCK(sc.alloc(tot));
         SCK(cudaMemcpyAsync(d_anc_off.p, aoff.data(), (np + 1ull) * sizeof(uint64_t), cudaMemcpyHostToDevice, st));
-        SCK(cudaMemcpyAsync(d_soff.p, soff.data(), np * sizeof(uint64_t), cudaMemcpyHostToDevice, st));
         ChainArgs b = a;
         b.prot_off = d_off.p + p0;
         b.prot_len = d_len.p + p0;
@@ -1367,8 +1485,8 @@ extern "C" int mp_index_chain(mp_dp_ctx *ctx, const mp_index *idx, const char *p
         b.chains = d_ch.p + static_cast<uint64_t>(p0) * top;
         b.n_chains = d_nch.p + p0;
         anchor_fill_kernel<<<grid_for(np * 32ull, 256), 256, 0, st>>>(b);
-        anchor_sort_kernel<<<np < 65535u * 4 ? np : 65535u * 4, kSortThreads, kSortMax * sizeof(uint64_t), st>>>(
-            b, sc.p, d_soff.p);
+        anchor_sort_kernel<<<np < 65535u * 4 ? np : 65535u * 4, kSortThreads, 0, st>>>(b, sc.p, idx->xbits);
+        if (sort_passes(idx->xbits) % 2) b.anc = sc.p;
         chain_kernel<<<np < 65535u * 16 ? np : 65535u * 16, kStrandWarps * 64, 0, st>>>(b);
         SCK(cudaGetLastError());
         SCK(cudaStreamSynchronize(st));
@@ -1416,7 +1534,6 @@ extern "C" int mp_chain_refine(mp_dp_ctx *ctx, const mp_pair *pairs, size_t n, m
     cudaStream_t st = ctx_stream(ctx);
     Tmp<char> d_seq;
     Tmp<uint64_t> d_poff, d_toff, d_cnt, d_aoff;
-    Tmp<uint32_t> d_tcnt;
     Tmp<uint32_t> d_plen, d_tlen;
     Tmp<int8_t> d_strand;
     Tmp<int32_t> d_log;
@@ -1428,7 +1545,6 @@ extern "C" int mp_chain_refine(mp_dp_ctx *ctx, const mp_pair *pairs, size_t n, m
     SCK(d_tlen.alloc(n));
     SCK(d_strand.alloc(n));
     SCK(d_cnt.alloc(n));
-    SCK(d_tcnt.alloc(static_cast<uint64_t>(n) * kRefineThreads));
     SCK(d_aoff.alloc(n + 1));
     SCK(d_log.alloc(kG));
     SCK(d_out.alloc(n));
@@ -1448,13 +1564,17 @@ extern "C" int mp_chain_refine(mp_dp_ctx *ctx, const mp_pair *pairs, size_t n, m
     a.strand = d_strand.p;
     a.log_tab = d_log.p;
     const uint32_t nb = static_cast<uint32_t>(n < 65535ull * 8 ? n : 65535ull * 8);
+    // the k-mer table of the longest protein, a power of two of them
+    size_t table = 1;
+    for (size_t k = 0; k < n; ++k)
+        while (table + kK2 - 1 < plen[k]) table <<= 1;
+    const size_t smem = table * sizeof(uint64_t);
     SCK(cudaFuncSetAttribute(refine_anchor_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(kRefineSmem)));
+                             static_cast<int>(kRefineMaxProt * sizeof(uint64_t))));
     SCK(cudaFuncSetAttribute(refine_anchor_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(kRefineSmem)));
-    refine_anchor_kernel<false><<<nb, kRefineThreads, kRefineSmem, st>>>(RefineArgs{a.seq, a.prot_off, a.nt_off, a.prot_len,
-                                                                          a.nt_len, a.strand, static_cast<uint32_t>(n)},
-                                                               d_tcnt.p, d_cnt.p);
+                             static_cast<int>(kRefineMaxProt * sizeof(uint64_t))));
+    a.n = static_cast<uint32_t>(n);
+    refine_anchor_kernel<false><<<nb, kRefineThreads, smem, st>>>(a, d_cnt.p);
     SCK(cudaGetLastError());
     std::vector<uint64_t> per(n);
     SCK(cudaMemcpyAsync(per.data(), d_cnt.p, n * sizeof(uint64_t), cudaMemcpyDeviceToHost, st));
@@ -1477,7 +1597,6 @@ extern "C" int mp_chain_refine(mp_dp_ctx *ctx, const mp_pair *pairs, size_t n, m
         SCK(pred.alloc(na));
         SCK(cudaMemcpyAsync(d_aoff.p, aoff.data(), (np + 1ull) * sizeof(uint64_t), cudaMemcpyHostToDevice, st));
         RefineArgs b = a;
-        b.seq = d_seq.p;
         b.prot_off = d_poff.p + p0;
         b.nt_off = d_toff.p + p0;
         b.prot_len = d_plen.p + p0;
@@ -1490,8 +1609,7 @@ extern "C" int mp_chain_refine(mp_dp_ctx *ctx, const mp_pair *pairs, size_t n, m
         b.pred = pred.p;
         b.out = d_out.p + p0;
         const uint32_t gb = np < 65535u * 8 ? np : 65535u * 8;
-        refine_anchor_kernel<true><<<gb, kRefineThreads, kRefineSmem, st>>>(b, d_tcnt.p + p0 * kRefineThreads,
-                                                                             nullptr);
+        refine_anchor_kernel<true><<<gb, kRefineThreads, smem, st>>>(b, nullptr);
         refine_chain_kernel<<<grid_for(np * 32ull, kRefineWarps * 32), kRefineWarps * 32, 0, st>>>(b);
         refine_chain_block_kernel<<<gb, kRefineThreads, 0, st>>>(b);
         SCK(cudaGetLastError());

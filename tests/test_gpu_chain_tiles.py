@@ -3,7 +3,9 @@ where the tiling and the 32-bit scores could go wrong: anchor counts around
 multiples of 32, dense repeats (many equal scores, thousands of anchors that
 follow one chain at a loss), every anchor on one strand, proteins past 32,000
 residues (64-bit scores), and regions with anchor counts around the limit
-between one warp and eight."""
+between one warp and eight.  Also the index of genomes whose buckets hold
+thousands of entries, tiny genomes, and regions around multiples of the second
+round's tile of 4,096 bases."""
 import numpy as np
 import pytest
 
@@ -94,3 +96,53 @@ def test_second_round_around_the_block_limit(mp, orc):
         want, _ = orc.refine_chain(anc)
         assert {f: int(got[k][f]) for f in REFINE_FIELDS} == want, (k, len(anc))
     assert any(c > 512 for c in counts) and any(0 < c <= 512 for c in counts) and any(c == 0 for c in counts)
+
+
+@pytest.mark.parametrize("case", ["repeats", "tiny"])
+def test_index_of_full_buckets_and_tiny_genomes(mp, orc, case):
+    rng = np.random.default_rng(330)
+    unit = synth.reverse_translate(rng, synth.random_protein(rng, 40))
+    genomes = [synth.random_dna(rng, 700, 0.4) + unit * 900 + synth.revcomp(unit) * 300 + "N" + unit * 41]
+    if case == "tiny":
+        gene = synth.reverse_translate(rng, synth.random_protein(rng, 400))
+        genomes = [gene[:n] for n in (0, 1, 2, 3, 90, 107, 108, 109, 255, 256, 257, 511, 512, 513, 1200)]
+        genomes.append(synth.random_dna(rng, 3 * 1024 * 3 + 1, 0.4) + gene)
+    ctx = mp.mp_dp_init(None, 0)
+    try:
+        for g in genomes:
+            idx = mp.mp_index_build(ctx, g)
+            off, ent = mp.mp_index_download(ctx, idx)
+            prot = synth.random_protein(rng, 5) + "MKVLAWDERT" * 3
+            ch, n = mp.mp_index_chain(ctx, idx, prot, [0], [len(prot)], 5)
+            mp.mp_index_free(idx)
+            woff, went = orc.build_index(g)
+            assert (off == woff).all() and (ent == went).all(), len(g)
+            want, _ = orc.chain(orc.anchors(woff, went, prot), 5)
+            assert [{f: int(ch[0, t][f]) for f in FIELDS} for t in range(int(n[0]))] == want
+        if case == "repeats":
+            assert np.diff(off.astype(np.int64)).max() > 512
+    finally:
+        mp.mp_dp_destroy(ctx)
+
+
+def test_second_round_around_the_tiles(mp, orc):
+    rng = np.random.default_rng(340)
+    pairs = []
+    for L in (14, 15, 16, 4109, 4110, 4111, 4112, 8205, 8206, 8207, 12302):
+        for strand in (1, -1):
+            prot = synth.random_protein(rng, int(rng.integers(6, 300)))
+            nt = synth.random_dna(rng, L, 0.4)
+            gene = synth.reverse_translate(rng, prot)
+            for at in (0, 4096 - 40, 4096 + 8, 8192 - 100):
+                nt = (nt[:at] + gene + nt[at + len(gene):])[:L]
+            if L > 4096:
+                nt = nt[:4093] + "N" + nt[4094:]
+            pairs.append(synth.Pair(prot, nt if strand > 0 else synth.revcomp(nt), strand))
+    ctx = mp.mp_dp_init(None, 0)
+    try:
+        got = mp.mp_chain_refine(ctx, pairs)
+    finally:
+        mp.mp_dp_destroy(ctx)
+    for k, p in enumerate(pairs):
+        want = orc.refine(p.prot, p.nt, p.strand)
+        assert {f: int(got[k][f]) for f in REFINE_FIELDS} == want, (k, len(p.nt), p.strand)
