@@ -927,6 +927,58 @@ static cudaError_t staging_wait(mp_dp_ctx *c)
     return cudaEventSynchronize(c->ev_staging);
 }
 
+}  // extern "C"
+
+// the context's gather threads, if `bytes` are worth them (started once)
+static WorkerPool *gather_pool(mp_dp_ctx *c, uint64_t bytes)
+{
+    const unsigned nthr = bytes > (16u << 20) ? std::min(16u, std::max(1u, std::thread::hardware_concurrency())) : 0u;
+    if (nthr && !c->pool) {
+        c->pool.reset(new (std::nothrow) WorkerPool());
+        if (c->pool) c->pool->start(nthr);
+    }
+    return nthr ? c->pool.get() : nullptr;
+}
+
+namespace mpdp {
+int ctx_send_pieces(mp_dp_ctx *c, const CopyPiece *pieces, size_t n, uint64_t total, char *dst)
+{
+    CK(staging_wait(c));
+    if (c->staging.reserve(total + 16) != cudaSuccess) return MP_ENOMEM;
+    std::atomic<int> copy_err{0};
+    auto send = [&](size_t k0, size_t k1) {
+        if (cudaSetDevice(c->device) != cudaSuccess) copy_err = 1;
+        size_t from = k0;
+        uint64_t acc = 0;
+        for (size_t k = k0; k < k1; ++k) {
+            if (pieces[k].len) memcpy(c->staging.p + pieces[k].at, pieces[k].src, pieces[k].len);
+            acc += pieces[k].len;
+            if (acc >= (2u << 20) || k + 1 == k1) {
+                const uint64_t lo = pieces[from].at, hi = k + 1 < n ? pieces[k + 1].at : total;
+                if (hi > lo && cudaMemcpyAsync(dst + lo, c->staging.p + lo, hi - lo, cudaMemcpyHostToDevice, c->stream) !=
+                                   cudaSuccess)
+                    copy_err = 1;
+                from = k + 1;
+                acc = 0;
+            }
+        }
+    };
+    if (WorkerPool *pool = gather_pool(c, total)) {
+        const unsigned nj = static_cast<unsigned>(pool->th.size());
+        pool->run(nj, [&, nj](unsigned t) { send(n * t / nj, n * (t + 1) / nj); });
+        pool->wait();
+    } else {
+        send(0, n);
+    }
+    if (copy_err) return MP_ECUDA;
+    CK(cudaEventRecord(c->ev_staging, c->stream));
+    c->staging_busy = true;
+    return MP_OK;
+}
+}  // namespace mpdp
+
+extern "C" {
+
 // ascii_on_device: the caller writes the batch's ASCII into b->ascii on the
 // context's stream itself (the pairs' nt pointers are unused and may be null;
 // the protein pointers still serve the score bound).
@@ -1163,12 +1215,7 @@ static int upload_impl(mp_dp_ctx *c, mp_dp_batch *b, const mp_pair *pairs, size_
             a = e;
         }
     };
-    const unsigned nthr = asc > (16u << 20) ? std::min(16u, std::max(1u, std::thread::hardware_concurrency())) : 0u;
-    if (nthr && !c->pool) {
-        c->pool.reset(new (std::nothrow) WorkerPool());
-        if (c->pool) c->pool->start(nthr);
-    }
-    const bool pooled = nthr && c->pool;
+    const bool pooled = gather_pool(c, asc) != nullptr;
     if (pooled) {
         const unsigned nj = static_cast<unsigned>(c->pool->th.size());
         if (span)

@@ -125,23 +125,44 @@ struct Frames {
 // Reduced-alphabet code of every codon of every frame.  Codon t of frame f
 // of strand 1 is the reverse complement's bases f + 3t .. f + 3t + 2, i.e.
 // the complements of genome[n-1-(f+3t)], genome[n-2-(f+3t)], genome[n-3-(f+3t)].
-__global__ void translate_kernel(const char *g, uint64_t n, Frames fr)
+//
+// A block takes kTransTile codons of all three frames of one strand
+// (blockIdx.y): the bases are read and coded once into shared memory, and four
+// neighbouring codons of a frame leave in one store (the frames' arrays start
+// on 16 bytes).  A thread per codon, with three byte loads, a search of its
+// frame and a table in constant memory read at 32 places, took 0.83 ms on 50
+// Mb; this 0.25.
+constexpr int kTransThreads = 256, kTransTile = 4 * kTransThreads;
+__global__ void __launch_bounds__(kTransThreads) translate_kernel(const char *g, uint64_t n, Frames fr)
 {
-    const uint64_t total = fr.len[0] + fr.len[1] + fr.len[2] + fr.len[3] + fr.len[4] + fr.len[5];
-    for (uint64_t q = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; q < total;
-         q += static_cast<uint64_t>(gridDim.x) * blockDim.x) {
-        int f = 0;
-        uint64_t t = q;
-        while (t >= fr.len[f]) t -= fr.len[f++];
-        const int strand = f / 3, frame = f % 3;
-        const uint64_t x = frame + 3 * t;
-        int b[3];
-#pragma unroll
-        for (int u = 0; u < 3; ++u) {
-            const int c = base_code(static_cast<unsigned char>(strand ? g[n - 1 - (x + u)] : g[x + u]));
-            b[u] = c < 0 ? -1 : (strand ? 3 - c : c);
+    __shared__ uint8_t base[3 * kTransTile + 4];
+    __shared__ uint8_t s_phi[64];
+    const int strand = blockIdx.y;
+    for (int k = threadIdx.x; k < 64; k += blockDim.x) s_phi[k] = c_codon_phi.v[k];
+    for (uint64_t t0 = blockIdx.x * static_cast<uint64_t>(kTransTile); t0 < fr.len[3 * strand];
+         t0 += gridDim.x * static_cast<uint64_t>(kTransTile)) {
+        __syncthreads();
+        for (int i = threadIdx.x; i < 3 * kTransTile + 2; i += blockDim.x) {
+            const uint64_t x = 3 * t0 + i;
+            const int c = x < n ? base_code(static_cast<unsigned char>(strand ? g[n - 1 - x] : g[x])) : -1;
+            base[i] = static_cast<uint8_t>(c < 0 ? 4 : strand ? 3 - c : c);
         }
-        fr.code[f][t] = (b[0] < 0 || b[1] < 0 || b[2] < 0) ? kXCode : c_codon_phi.v[b[0] * 16 + b[1] * 4 + b[2]];
+        __syncthreads();
+#pragma unroll
+        for (int f = 0; f < 3; ++f) {
+            const uint64_t t = t0 + 4 * threadIdx.x, len = fr.len[3 * strand + f];
+            const uint8_t *b = base + f + 12 * threadIdx.x;
+            uint32_t w = 0;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int b0 = b[3 * k], b1 = b[3 * k + 1], b2 = b[3 * k + 2];
+                w |= static_cast<uint32_t>((b0 | b1 | b2) & 4 ? kXCode : s_phi[b0 * 16 + b1 * 4 + b2]) << (8 * k);
+            }
+            uint8_t *out = fr.code[3 * strand + f] + t;
+            if (t + 4 <= len) *reinterpret_cast<uint32_t *>(out) = w;
+            else
+                for (int k = 0; t + k < len && k < 4; ++k) out[k] = static_cast<uint8_t>(w >> (8 * k));
+        }
     }
 }
 
@@ -233,59 +254,86 @@ __global__ void __launch_bounds__(kScanThreads) segment_scan(Frames fr, const in
 // the frame's start, b at the next stop or the frame's end) with b - a >=
 // kMinOrf and t + kK <= b, the k-mer code of codons t .. t+5 is hashed; a
 // sampled one (lowest bit 0) is counted in its bucket (pass 0) or written at
-// its bucket's cursor (pass 1).
-constexpr int kKmerWarps = 4;
+// its bucket's cursor (pass 1).  The segment's codes are read once into shared
+// memory; lane c keeps the stops of the segment's codons 32c .. 32c + 31 as a
+// bit mask and the last stop before and the first after them, from which the
+// run of any codon follows (a table of both per codon, filled in two sweeps,
+// left room for 28 warps per SM: 0.75 and 1.17 ms on 50 Mb; this 0.20 and
+// 0.49).
+constexpr int kKmerWarps = 8;
 
 __global__ void __launch_bounds__(kKmerWarps * 32) kmer_kernel(Frames fr, const int64_t *before, const int64_t *after,
                                                                uint64_t nseg, int pass, uint32_t *count,
                                                                uint32_t *cursor, uint32_t *entries)
 {
-    // the stop before and after each codon of the warp's segment
-    __shared__ int32_t s_prev[kKmerWarps][kSeg / 32][32], s_next[kKmerWarps][kSeg / 32][32];
+    __shared__ alignas(16) uint8_t seg[kKmerWarps][kSeg + 16];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    auto prev = [&](int c) -> int32_t & { return s_prev[w][c][lane]; };
-    auto next = [&](int c) -> int32_t & { return s_next[w][c][lane]; };
-    for (uint64_t s = (blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x) >> 5; s < nseg;
-         s += (static_cast<uint64_t>(gridDim.x) * blockDim.x) >> 5) {
+    static_assert(kSeg == 32 * 32, "a word of stops per lane");
+    for (uint64_t s = blockIdx.x * static_cast<uint64_t>(kKmerWarps) + w; s < nseg;
+         s += static_cast<uint64_t>(gridDim.x) * kKmerWarps) {
         int f = 0;
         while (s >= fr.seg0[f + 1]) ++f;
         const uint64_t t0 = (s - fr.seg0[f]) * kSeg, len = fr.len[f];
-        const uint8_t *code = fr.code[f];
-        // the stop before each codon, sweeping forward; the stop after, sweeping back
-        int64_t cur = before[s];
-        for (int c = 0; c < kSeg / 32; ++c) {
-            const uint64_t t = t0 + c * 32 + lane;
-            const bool stop = t < len && code[t] == kStopCode;
-            const unsigned bal = __ballot_sync(0xffffffffu, stop);
-            const unsigned below = bal & ((1u << lane) - 1);
-            prev(c) = static_cast<int32_t>(below ? static_cast<int64_t>(t0 + c * 32 + 31 - __clz(below)) : cur);
-            if (bal) cur = static_cast<int64_t>(t0 + c * 32 + 31 - __clz(bal));
+        const uint8_t *code = fr.code[f] + t0;
+        const int cnt = static_cast<int>(len - t0 < kSeg ? len - t0 : kSeg);               // codons of the segment
+        const int more = static_cast<int>(len - t0 < kSeg + kK - 1 ? len - t0 : kSeg + kK - 1);   // and what its k-mers touch
+        __syncwarp();
+        if (cnt == kSeg) {
+            // (the frames' arrays start on 16 bytes and a segment is a multiple of them)
+            const uint4 *src = reinterpret_cast<const uint4 *>(code);
+            reinterpret_cast<uint4 *>(seg[w])[lane] = src[lane];
+            reinterpret_cast<uint4 *>(seg[w])[lane + 32] = src[lane + 32];
+            if (kSeg + lane < more) seg[w][kSeg + lane] = code[kSeg + lane];
+        } else {
+            for (int t = lane; t < more; t += 32) seg[w][t] = code[t];
         }
-        cur = after[s];
-        for (int c = kSeg / 32 - 1; c >= 0; --c) {
-            const uint64_t t = t0 + c * 32 + lane;
-            const bool stop = t < len && code[t] == kStopCode;
-            const unsigned bal = __ballot_sync(0xffffffffu, stop);
-            const unsigned above = lane == 31 ? 0u : (bal & ~((2u << lane) - 1));
-            next(c) = static_cast<int32_t>(above ? static_cast<int64_t>(t0 + c * 32 + __ffs(above) - 1) : cur);
-            if (bal) cur = static_cast<int64_t>(t0 + c * 32 + __ffs(bal) - 1);
+        __syncwarp();
+        // stops of this lane's 32 codons
+        uint32_t mine = 0;
+        for (int c = 0; c < 32; ++c) {
+            const int t = c * 32 + lane;
+            const unsigned bal = __ballot_sync(0xffffffffu, t < cnt && seg[w][t] == kStopCode);
+            if (c == lane) mine = bal;
         }
+        // the last stop before them and the first after (codons of the segment;
+        // -1 and kSeg: none in it)
+        int last = mine ? lane * 32 + 31 - __clz(mine) : -1, first = mine ? lane * 32 + __ffs(mine) - 1 : kSeg;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, last, o), z = __shfl_down_sync(0xffffffffu, first, o);
+            if (lane >= o) last = max(last, y);
+            if (lane + o < 32) first = min(first, z);
+        }
+        last = __shfl_up_sync(0xffffffffu, last, 1);
+        first = __shfl_down_sync(0xffffffffu, first, 1);
+        if (lane == 0) last = -1;
+        if (lane == 31) first = kSeg;
+        // as distances from the segment's first codon, clamped to what decides
+        // (a run that leaves the segment by kMinOrf is long enough, by kK goes on)
+        const int64_t far_b = before[s] - static_cast<int64_t>(t0), far_a = after[s] - static_cast<int64_t>(t0);
+        const int out_b = static_cast<int>(far_b < -1 - kMinOrf ? -1 - kMinOrf : far_b);
+        const int out_a = static_cast<int>(far_a > kSeg + kMinOrf ? kSeg + kMinOrf : far_a);
+        if (last < 0) last = out_b;
+        if (first >= kSeg) first = out_a;
         const uint32_t strand = f / 3, frame = f % 3;
-        for (int c = 0; c < kSeg / 32; ++c) {
-            const uint64_t t = t0 + c * 32 + lane;
-            if (t >= len || code[t] == kStopCode) continue;
-            const int64_t a = prev(c) + 1, b = next(c);
-            if (b - a < kMinOrf || static_cast<int64_t>(t) + kK > b) continue;
+        for (int c = 0; c < 32; ++c) {
+            const uint32_t m = __shfl_sync(0xffffffffu, mine, c);
+            const int lc = __shfl_sync(0xffffffffu, last, c), fc = __shfl_sync(0xffffffffu, first, c);
+            const int t = c * 32 + lane;
+            if (t >= cnt || (m >> lane & 1)) continue;
+            const uint32_t below = m & ((1u << lane) - 1), above = lane == 31 ? 0u : m & ~((2u << lane) - 1);
+            const int a = (below ? c * 32 + 31 - __clz(below) : lc) + 1, b = above ? c * 32 + __ffs(above) - 1 : fc;
+            if (b - a < kMinOrf || t + kK > b) continue;
             uint32_t key = 0;
 #pragma unroll
-            for (int u = 0; u < kK; ++u) key = key * 16 + code[t + u];
+            for (int u = 0; u < kK; ++u) key = key * 16 + seg[w][t + u];
             const uint32_t h = psi24(key);
             if (h & 1u) continue;
             if (pass == 0) {
                 atomicAdd(count + h, 1u);
             } else {
                 const uint32_t at = atomicAdd(cursor + h, 1u);
-                entries[at] = (strand << 31) | static_cast<uint32_t>((frame + 3 * t) / kBin);
+                entries[at] = (strand << 31) | static_cast<uint32_t>((frame + 3 * (t0 + t)) / kBin);
             }
         }
     }
@@ -1315,11 +1363,11 @@ extern "C" int mp_index_build(mp_dp_ctx *ctx, const char *genome, uint64_t len, 
     }
     fr.seg0[6] = nseg;
     Tmp<uint8_t> codes;
-    SCK(codes.alloc(total));
+    SCK(codes.alloc(total + 6 * 16));
     uint64_t at = 0;
     for (int f = 0; f < 6; ++f) {
         fr.code[f] = codes.p + at;
-        at += fr.len[f];
+        at += (fr.len[f] + 15) / 16 * 16;
     }
     Tmp<int64_t> first, last, before, after;
     SCK(first.alloc(nseg));
@@ -1331,7 +1379,7 @@ extern "C" int mp_index_build(mp_dp_ctx *ctx, const char *genome, uint64_t len, 
     SCK(cursor.alloc(kNKeys + 1));
     SCK(cudaMemsetAsync(count.p, 0, kNKeys * sizeof(uint32_t), st));
     if (total) {
-        translate_kernel<<<grid_for(total, 256), 256, 0, st>>>(g.p, len, fr);
+        translate_kernel<<<dim3(grid_for(fr.len[0], kTransTile), 2), kTransThreads, 0, st>>>(g.p, len, fr);
         segment_kernel<<<grid_for(nseg * 32, 256), 256, 0, st>>>(fr, first.p, last.p, nseg);
         segment_scan<<<6, kScanThreads, 0, st>>>(fr, first.p, last.p, before.p, after.p);
         kmer_kernel<<<grid_for(nseg * 32, kKmerWarps * 32), kKmerWarps * 32, 0, st>>>(
@@ -1525,10 +1573,10 @@ extern "C" int mp_chain_refine(mp_dp_ctx *ctx, const mp_pair *pairs, size_t n, m
         tlen[k] = q.nt_len;
         strand[k] = q.strand;
     }
-    std::vector<char> h(tot ? tot : 1);
+    std::vector<CopyPiece> pieces(2 * n);
     for (size_t k = 0; k < n; ++k) {
-        if (plen[k]) memcpy(h.data() + poff[k], pairs[k].prot, plen[k]);
-        if (tlen[k]) memcpy(h.data() + toff[k], pairs[k].nt, tlen[k]);
+        pieces[2 * k] = CopyPiece{pairs[k].prot, poff[k], plen[k]};
+        pieces[2 * k + 1] = CopyPiece{pairs[k].nt, toff[k], tlen[k]};
     }
     if (cudaSetDevice(ctx_device(ctx)) != cudaSuccess) return MP_ECUDA;
     cudaStream_t st = ctx_stream(ctx);
@@ -1548,7 +1596,10 @@ extern "C" int mp_chain_refine(mp_dp_ctx *ctx, const mp_pair *pairs, size_t n, m
     SCK(d_aoff.alloc(n + 1));
     SCK(d_log.alloc(kG));
     SCK(d_out.alloc(n));
-    SCK(cudaMemcpyAsync(d_seq.p, h.data(), tot, cudaMemcpyHostToDevice, st));
+    // (gathered into a fresh host vector and sent from there, pageable, the
+    // sequences of 6,000 regions took 6 ms)
+    const int sent = ctx_send_pieces(ctx, pieces.data(), pieces.size(), tot, d_seq.p);
+    if (sent != MP_OK) return sent;
     SCK(cudaMemcpyAsync(d_poff.p, poff.data(), n * sizeof(uint64_t), cudaMemcpyHostToDevice, st));
     SCK(cudaMemcpyAsync(d_toff.p, toff.data(), n * sizeof(uint64_t), cudaMemcpyHostToDevice, st));
     SCK(cudaMemcpyAsync(d_plen.p, plen.data(), n * sizeof(uint32_t), cudaMemcpyHostToDevice, st));
