@@ -429,7 +429,8 @@ typedef struct {
                                   taken about two chunks after strip s; 0: pairs' strips back to
                                   back (a strip's warp first waits for its predecessor) */
     float ms;                  /* set by mp_dp_autotune: device time of one run of the batch */
-    int32_t strip_width;       /* 0: every pair in strips of 64 residues (two per lane of a warp);
+    int32_t strip_width;       /* 0: every pair in strips of 64 residues (two strips to a warp, or
+                                  one where strips are fewer than the GPU's schedulers);
                                   1: int16 pairs in strips of 128 residues (four per lane: one
                                   shuffle, record load and profile load serve four cells) where that
                                   adds little padding (an even number of 64-residue strips, or 9 or
