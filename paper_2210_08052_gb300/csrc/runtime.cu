@@ -941,38 +941,50 @@ static WorkerPool *gather_pool(mp_dp_ctx *c, uint64_t bytes)
 }
 
 namespace mpdp {
+static constexpr uint64_t kSendWindow = 256ull << 20;
+
 int ctx_send_pieces(mp_dp_ctx *c, const CopyPiece *pieces, size_t n, uint64_t total, char *dst)
 {
-    CK(staging_wait(c));
-    if (c->staging.reserve(total + 16) != cudaSuccess) return MP_ENOMEM;
-    std::atomic<int> copy_err{0};
-    auto send = [&](size_t k0, size_t k1) {
-        if (cudaSetDevice(c->device) != cudaSuccess) copy_err = 1;
-        size_t from = k0;
-        uint64_t acc = 0;
-        for (size_t k = k0; k < k1; ++k) {
-            if (pieces[k].len) memcpy(c->staging.p + pieces[k].at, pieces[k].src, pieces[k].len);
-            acc += pieces[k].len;
-            if (acc >= (2u << 20) || k + 1 == k1) {
-                const uint64_t lo = pieces[from].at, hi = k + 1 < n ? pieces[k + 1].at : total;
-                if (hi > lo && cudaMemcpyAsync(dst + lo, c->staging.p + lo, hi - lo, cudaMemcpyHostToDevice, c->stream) !=
-                                   cudaSuccess)
-                    copy_err = 1;
-                from = k + 1;
-                acc = 0;
+    // in windows of at most kSendWindow bytes (or one longer piece), so that the
+    // pinned buffer stays bounded however many pieces there are
+    for (size_t w0 = 0; w0 < n;) {
+        const uint64_t base = pieces[w0].at;
+        auto end_of = [&](size_t k) { return k + 1 < n ? pieces[k + 1].at : total; };
+        size_t w1 = w0 + 1;
+        while (w1 < n && end_of(w1) - base <= kSendWindow) ++w1;
+        const uint64_t bytes = end_of(w1 - 1) - base;
+        CK(staging_wait(c));
+        if (c->staging.reserve(bytes + 16) != cudaSuccess) return MP_ENOMEM;
+        std::atomic<int> copy_err{0};
+        auto send = [&](size_t k0, size_t k1) {
+            if (cudaSetDevice(c->device) != cudaSuccess) copy_err = 1;
+            size_t from = k0;
+            uint64_t acc = 0;
+            for (size_t k = k0; k < k1; ++k) {
+                if (pieces[k].len) memcpy(c->staging.p + (pieces[k].at - base), pieces[k].src, pieces[k].len);
+                acc += pieces[k].len;
+                if (acc >= (2u << 20) || k + 1 == k1) {
+                    const uint64_t lo = pieces[from].at, hi = end_of(k);
+                    if (hi > lo && cudaMemcpyAsync(dst + lo, c->staging.p + (lo - base), hi - lo,
+                                                   cudaMemcpyHostToDevice, c->stream) != cudaSuccess)
+                        copy_err = 1;
+                    from = k + 1;
+                    acc = 0;
+                }
             }
+        };
+        if (WorkerPool *pool = gather_pool(c, bytes)) {
+            const unsigned nj = static_cast<unsigned>(pool->th.size());
+            pool->run(nj, [&, nj](unsigned t) { send(w0 + (w1 - w0) * t / nj, w0 + (w1 - w0) * (t + 1) / nj); });
+            pool->wait();
+        } else {
+            send(w0, w1);
         }
-    };
-    if (WorkerPool *pool = gather_pool(c, total)) {
-        const unsigned nj = static_cast<unsigned>(pool->th.size());
-        pool->run(nj, [&, nj](unsigned t) { send(n * t / nj, n * (t + 1) / nj); });
-        pool->wait();
-    } else {
-        send(0, n);
+        CK(cudaEventRecord(c->ev_staging, c->stream));
+        c->staging_busy = true;
+        if (copy_err) return MP_ECUDA;
+        w0 = w1;
     }
-    if (copy_err) return MP_ECUDA;
-    CK(cudaEventRecord(c->ev_staging, c->stream));
-    c->staging_busy = true;
     return MP_OK;
 }
 }  // namespace mpdp

@@ -1491,8 +1491,6 @@ extern "C" int mp_index_chain(mp_dp_ctx *ctx, const mp_index *idx, const char *p
     // proteins in groups whose anchors (8 + 8 + 8 + 4 + 1 bytes each) stay within
     // a bound
     constexpr uint64_t kMaxAnchors = 192ull << 20;
-    std::vector<mp_chain> h_ch(static_cast<uint64_t>(n_prot) * top);
-    std::vector<uint32_t> h_nch(n_prot);
     for (uint32_t p0 = 0; p0 < n_prot;) {
         uint32_t p1 = p0;
         uint64_t tot = 0;
@@ -1632,7 +1630,6 @@ extern "C" int mp_chain_refine(mp_dp_ctx *ctx, const mp_pair *pairs, size_t n, m
     SCK(cudaStreamSynchronize(st));
     // pairs in groups whose anchors (8 + 8 + 4 bytes each) stay within a bound
     constexpr uint64_t kMaxAnchors = 192ull << 20;
-    std::vector<mp_chain2> h_out(n);
     for (size_t p0 = 0; p0 < n;) {
         size_t p1 = p0;
         uint64_t na = 0;

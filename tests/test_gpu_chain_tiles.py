@@ -146,3 +146,27 @@ def test_second_round_around_the_tiles(mp, orc):
     for k, p in enumerate(pairs):
         want = orc.refine(p.prot, p.nt, p.strand)
         assert {f: int(got[k][f]) for f in REFINE_FIELDS} == want, (k, len(p.nt), p.strand)
+
+
+def test_second_round_of_more_bytes_than_are_sent_at_once(mp):
+    """Sequences go to the device in windows of 256 MB: the pairs of every
+    window, the ones at its edges included, have the chains they have alone."""
+    rng = np.random.default_rng(350)
+    kinds = []
+    for L in (7_000_000, 6_999_999, 5_000_003):
+        prot = synth.random_protein(rng, 90)
+        nt = synth.random_dna(rng, L - 270, 0.4)
+        kinds.append(synth.Pair(prot, nt[:L // 2] + synth.reverse_translate(rng, prot) + nt[L // 2:], 1))
+    pairs = [kinds[k % 3] for k in range(90)]
+    assert sum(len(p.nt) + len(p.prot) for p in pairs) > 2 * (256 << 20)
+    ctx = mp.mp_dp_init(None, 0)
+    try:
+        alone = [mp.mp_chain_refine(ctx, [p])[0] for p in kinds]
+        got = mp.mp_chain_refine(ctx, pairs)
+    finally:
+        mp.mp_dp_destroy(ctx)
+    for k in range(len(pairs)):
+        assert all(int(got[k][f]) == int(alone[k % 3][f]) for f in REFINE_FIELDS), k
+    # (the planted gene scores its length; of the links of equal worth along its
+    # diagonal the one from the earliest anchor is taken, so its anchors are fewer)
+    assert all(int(a["score"]) >= 90 << 16 for a in alone)
