@@ -439,8 +439,9 @@ def roofline(m, cells, torch, device, peaks):
                 "stream_per_cell": m["code_bytes"] / cells if cells else None,
                 "basis": "counted by the library's planner for this run, per pipeline run: the H stream "
                          "(padding of the last strip and chunk and the column maxima included), the per-nt "
-                         "records (written once, read by every strip of the pair, mostly from L2), the "
-                         "boundary rows between strips (written and read once, mostly in L2); "
+                         "records (written once, read by every warp of the pair, mostly from L2), the "
+                         "boundary rows between warps (written and read once, mostly in L2; 4 bytes per "
+                         "entry, the int16 words' 4-byte tags not counted); "
                          "'traffic' is the DRAM count of the committed ncu capture, scaled by cells"},
             "issue_frac": (cells / 64 * ips / (dp_avg_ms / 1000) / (nsm * 4 * f_mhz * 1e6))
             if (dp_avg_ms and ips) else None,

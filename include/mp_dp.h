@@ -401,11 +401,13 @@ typedef struct {
                                   (padding of the last strip and chunk included) and the
                                   per-chunk column maxima */
     uint64_t record_bytes;     /* per-nt records written by the precompute kernel */
-    uint64_t record_read_bytes;  /* records the strips read (every strip its pair's; two strips run by
-                                    one warp share one read; mostly L2 hits after the first) */
-    uint64_t boundary_bytes;   /* boundary rows handed from strip to strip, 4 bytes each (8 in the
-                                  int32 kernel); between the strips of one warp in registers,
-                                  otherwise through memory with a 4-byte tag */
+    uint64_t record_read_bytes;  /* records the warps read: once per strip, or once for the two
+                                    strips that one warp runs (mostly L2 hits after the first) */
+    uint64_t boundary_bytes;   /* boundary rows handed from warp to warp through memory, whole
+                                  chunks, 4 bytes per entry (8 for pairs that may need int32);
+                                  the packed int16 kernel writes each entry with a 4-byte tag,
+                                  not counted here.  Two strips of one warp pass theirs in
+                                  registers */
 } mp_dp_stats;
 
 /* Launch configuration of the DP.  The paper's DP is a SIMD loop on CPU

@@ -853,16 +853,21 @@ static int plan_waves(mp_dp_ctx *c, mp_dp_batch *b, const mp_dp_tuning &t, bool 
         cur += cbytes[p];
         if (cbytes[p])
             b->code_bytes_total += code_bytes(d.prot_len, d.nt_len, (d.flags & PF_WIDE) != 0, (d.flags & PF_W128) != 0);
+        const uint32_t items = items_of(d.flags, d.n_strips);
         {
             const uint64_t W = (d.flags & PF_W128) ? kStripWMax : kStripW;
             const uint64_t nch = div_up(static_cast<uint64_t>(d.nt_len) + W - 1, kChunk);
             b->record_bytes_total += records_of(d.nt_len) * sizeof(uint4);
-            // each strip queues one chunk of records ahead of its first
-            b->record_read_total += static_cast<uint64_t>(d.n_strips) * (nch + 1) * kChunk * sizeof(uint4);
-            b->bnd_bytes_total += static_cast<uint64_t>(d.n_strips > 0 ? d.n_strips - 1 : 0) * nch * kChunk *
+            // each work item queues one chunk of records ahead of its first; one of
+            // two strips has 64 more steps than one of a strip
+            const uint64_t duos = (d.flags & PF_DUO) ? d.n_strips / 2 : 0;
+            const uint64_t nch2 = div_up(static_cast<uint64_t>(d.nt_len) + 2 * kStripW - 1, kChunk);
+            b->record_read_total += ((items - duos) * (nch + 1) + duos * (nch2 + 1)) * kChunk * sizeof(uint4);
+            // entries from one item to the next (the strips of one item keep theirs
+            // in registers), without the int16 forms' tags
+            b->bnd_bytes_total += static_cast<uint64_t>(items > 0 ? items - 1 : 0) * nch * kChunk *
                                   ((d.flags & PF_WIDE) ? 8 : 4);
         }
-        const uint32_t items = items_of(d.flags, d.n_strips);
         for (uint32_t s = 0; s < items; ++s) b->h_items.push_back(make_uint2(p, s));
         if (wide(p) == 0) nwide += items;
     }
