@@ -744,12 +744,18 @@ static int plan_waves(mp_dp_ctx *c, mp_dp_batch *b, const mp_dp_tuning &t, bool 
     }
     // ... unless the pair's own chain of steps (its region, and three chunks
     // from each warp to the next) is longer than what every warp has to do: then
-    // the chain sets the time, and one strip per warp runs it faster, as long as
-    // these warps have a scheduler each (39 ns a step of a lone warp against
-    // 47.5).  With all strips of 64 genes on schedulers of their own 1.70
-    // against 1.91 ms; where they do not fit (all strips of 128 profiles alone:
-    // 3.17 against 2.87) only the longest chains get them, on a quarter of the
-    // schedulers.
+    // the chain sets the time, and one strip per warp runs it faster (39 ns a
+    // step of a warp alone on its scheduler against 47.5).  Where every strip of
+    // the batch finds a scheduler of its own, all such pairs run so: 64 genes
+    // 1.70 against 1.91 ms.  Otherwise only the longest chains do, as many
+    // strips of them as there are SMs.  Their warps share schedulers with the
+    // others (nothing keeps one for them), but a step of one strip still ends
+    // sooner than one of two: 90 genes 2.00 ms against 2.17 with all pairs two
+    // strips per warp, 320 genes 2.43 against 2.58, 60 uneven pairs 5.43
+    // against 5.96, 128 profiles 1.53 against 1.74; it no longer gains at 512
+    // global pairs (3.05, 3.11) and costs at 1,000 genes (4.20, 4.01).  With all
+    // such pairs one strip per warp 128 profiles took 3.17 against 2.87 ms from
+    // the host.
     const double share = steps / (static_cast<double>(c->num_sms) * 2 * kWarps16);
     std::vector<std::pair<double, uint32_t>> chains;
     for (uint32_t k = 0; k < n; ++k) {
