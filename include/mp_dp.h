@@ -113,7 +113,7 @@ typedef struct {
                                   at 60% of the device memory free at init) */
     int32_t force_int32;       /* 1: skip the packed int16 pass and run every pair in int32 */
     int32_t max_pairs_per_launch; /* 0: no limit; 1: one pair per kernel launch (plain form) */
-    int32_t wait_limit;        /* polls (~0.25 us each) before a warp waiting on the previous
+    int32_t wait_limit;        /* polls (about 0.5 us each) before a warp waiting on the previous
                                   strip of its pair gives up and marks the pair MP_ST_TIMEOUT;
                                   0: default (4e7) */
     int32_t debug_flags;       /* test hook: MP_DEBUG_NO_PUBLISH makes every strip withhold its

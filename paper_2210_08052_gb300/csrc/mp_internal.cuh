@@ -144,7 +144,7 @@ struct DPArgs {
     const int32_t *epre;    // per profile position j: the sum of gap_ext over positions 1..j
 };
 
-// bounded wait of a consumer strip for its producer (iterations of ~0.25 us)
+// bounded wait of a consumer strip for its producer (iterations of about 0.5 us)
 constexpr uint32_t kSpinLimit = 40u * 1000u * 1000u;
 
 struct TBArgs {

@@ -125,3 +125,24 @@ def test_each_form_of_profile_queries(mp, orc, mode, duo):
         assert not (bad := _bad(pairs * n, got, want * n)), bad[:5]
     finally:
         mp.mp_dp_destroy(c)
+
+
+def test_poll_limit_bounds_both_kernels_waits_alike(mp):
+    """With boundary rows withheld, a pair of three strips waits out its poll
+    limit, at most a fifth of a second, and is marked.  The int16 wait lasts as
+    long as the int32 kernel's under the same limit: its first 64 polls of 40,000
+    sleep less, and a poll's load may take a little less (5 per cent)."""
+    rng = np.random.default_rng(270)
+    pair = synth.Pair(synth.random_protein(rng, 192), synth.random_dna(rng, 300), 1)
+    ms = []
+    for force_int32 in (0, 1):
+        c = mp.mp_dp_init(mp.mp_dp_default_params(wait_limit=40_000, debug_flags=mp.MP_DEBUG_NO_PUBLISH,
+                                                  force_int32=force_int32), 0)
+        try:
+            mp.mp_dp_set_timing(c, True)
+            for _ in range(3):
+                assert mp.mp_dp_align_batch(c, [pair])[0]["status"] & mp.MP_ST_TIMEOUT
+            ms.append(mp.mp_dp_get_stats(c)["dp_ms"])
+        finally:
+            mp.mp_dp_destroy(c)
+    assert ms[0] > 0.95 * ms[1], ms
