@@ -416,8 +416,8 @@ typedef struct {
  * Every configuration computes bit-identical results: only the speed
  * differs. */
 typedef struct {
-    int32_t dp16_variant;      /* 0: int16 DP kernel built with 8-warp CTAs (<= 128 registers per
-                                  thread); 1: with 6-warp CTAs (<= 168 registers) */
+    int32_t dp16_variant;      /* 0: int16 DP kernel built with 8-warp CTAs, one per SM (<= 255
+                                  registers per thread); 1: with 6-warp CTAs, two per SM (<= 168) */
     int32_t dp16_ctas_per_sm;  /* resident CTAs per SM in the int16 launch; 0 = all that fit */
     int32_t dp32_ctas_per_sm;  /* the same for the int32 kernel */
     int32_t wide_direct;       /* 1: pairs whose score bound reaches the int16 limit skip the int16

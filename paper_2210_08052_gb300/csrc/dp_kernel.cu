@@ -945,13 +945,13 @@ struct Ops16x4 {
 // takes 32.1 instructions (19.3 of them on the ALU) and 9.4 shared-memory rows
 // per 64 cells, here the same cells take 26.5, 14.7 and 8: 51.6 clocks of a
 // scheduler against 44.  A warp alone takes 98 clocks per step of 128 cells
-// (one strip per warp without the loads ahead of their step: 87 for 64).  Every form tried ran at 0.6 instructions per clock when
-// several warps shared a scheduler, so what counted was instructions: two
-// maxima of a pair of steps in one, frameshift maxima shared by a and b, no
-// permute in the hand-over, profile halves added instead of permuted, and
-// registers enough for no spill (a reload in the loop cost more than the
-// warps it made room for: 16 warps per SM at 128 registers 12.6 ms on the
-// 4,096-pair workload, 12 at 168 registers 10.55; start of this form, one
+// (one strip per warp without the loads ahead of their step: 87 for 64).
+// Every form tried ran at 0.6 instructions per clock when several warps shared
+// a scheduler, so what counted was instructions: two maxima of a pair of steps
+// in one, frameshift maxima shared by a and b, no permute in the hand-over,
+// profile halves added instead of permuted, and registers enough for no spill
+// (4,096-pair workload: 8 warps per SM held to 128 registers, with reloads in
+// the loop, 11.35 ms, at 255 registers 10.45; 12 at 168 10.4; start, one
 // strip per warp, 12.8).  Bodies of 24 unrolled steps instead of 12 gain 3%
 // while all warps run in step and lose 10% when they do not (instruction
 // fetch).
@@ -2289,11 +2289,22 @@ __host__ __device__ constexpr size_t warp16_bytes(bool wide4)
     return b;
 }
 
-// Warps: warps per CTA, two CTAs per SM (8: at most 128 registers per thread,
-// 6: 168).  Wide4: the int16 build that also runs pairs in 128-residue strips
-// (PF_W128), each warp's shared memory sized for either strip form.
+// Dynamic shared memory of a CTA, and the CTAs that one SM then has room for
+// (228 KB, of which each takes 1 KB besides), two at most: what the compiler
+// may count on when it shares out the registers.
+template <typename Ops, int Warps, bool Wide4>
+constexpr size_t kCtaBytes = Warps * (sizeof(typename Ops::Bnd) == 4 ? warp16_bytes(Wide4) : sizeof(typename Ops::Smem));
+template <typename Ops, int Warps, bool Wide4>
+constexpr int kCtasPerSm = 2 * (kCtaBytes<Ops, Warps, Wide4> + 1024) <= 228 * 1024 ? 2 : 1;
+
+// Warps: warps per CTA.  int16: 6, two CTAs per SM (168 registers per thread),
+// or 8, of which the two-strip form's shared memory leaves one (255; as if for
+// two, at 128 registers with spills, that build took 11.35 ms on the 4,096-pair
+// workload against 10.45).  int32: 8, two CTAs per SM.  Wide4: the int16 build
+// that also runs pairs in 128-residue strips (PF_W128), each warp's shared
+// memory sized for either strip form.
 template <typename Ops, int Warps, bool Wide4 = false>
-__global__ void __launch_bounds__(Warps * 32, 2) dp_kernel(const DPArgs a, int rerun_only)
+__global__ void __launch_bounds__(Warps * 32, (kCtasPerSm<Ops, Warps, Wide4>)) dp_kernel(const DPArgs a, int rerun_only)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     using SM = typename Ops::Smem;
@@ -2361,8 +2372,7 @@ static int blocks_per_sm(const void *fn, int warps, size_t smem)
 // read the occupancy, once per device and build.
 template <typename Ops, int Warps, bool Wide4 = false>
 struct DpBuild {
-    static constexpr size_t kSmem =
-        Warps * (sizeof(typename Ops::Bnd) == 4 ? warp16_bytes(Wide4) : sizeof(typename Ops::Smem));
+    static constexpr size_t kSmem = kCtaBytes<Ops, Warps, Wide4>;
     static int blocks_per_sm()
     {
         constexpr int kMaxDev = 64;

@@ -18,7 +18,7 @@ constexpr int kProfRows = 22;   // translated amino acid 0..19, stop 20, no codo
 constexpr int kBndPad = kStripWMax;   // boundary entries before genome position 0
 constexpr int kRecPre = 2 * kChunk;   // per-nt records before genome position 0
 constexpr int kWarpsPerCta = 8; // warps per CTA of the persistent DP kernels
-constexpr int kWarps16 = 6;     // of the int16 build with more registers per thread (168 instead of 128)
+constexpr int kWarps16 = 6;     // of the int16 build of which an SM holds two CTAs
 constexpr int kNtPadWords = 16; // zero words around each packed genome
 
 // bytes of the traceback stream per strip step in the int16 path: 64 cells * 2 B
@@ -167,9 +167,10 @@ cudaError_t launch_pack(const PairDesc *pairs, uint32_t n, const char *ascii, ui
                         uint32_t *nt2, PairOut *out, cudaStream_t st);
 cudaError_t launch_records(const PairDesc *pairs, uint32_t n, const uint32_t *nt2, const ScoreParams &sp, uint4 *recs,
                            uint64_t *bnd, cudaStream_t st);
-// variant 0: the int16 DP kernel built with kWarpsPerCta warps per CTA (up to
-// 128 registers per thread); 1: with kWarps16 (up to 168).  wide4: the latter
-// that also runs PF_W128 pairs in 128-residue strips.  Same results.
+// variant 0: the int16 DP kernel built with kWarpsPerCta warps per CTA, one per
+// SM (up to 255 registers per thread); 1: with kWarps16, two per SM (up to 168).
+// wide4: the latter that also runs PF_W128 pairs in 128-residue strips.  Same
+// results.
 constexpr int kDp16Variants = 2;
 cudaError_t launch_dp16(const DPArgs &a, int grid, int variant, bool wide4, cudaStream_t st);
 cudaError_t launch_dp32(const DPArgs &a, int grid, bool rerun_only, cudaStream_t st);
