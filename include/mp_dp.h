@@ -357,7 +357,9 @@ void mp_index_free(mp_index *idx);
  * anchor.  MP_EINVAL: a null argument, a protein longer than 8,192
  * residues, a region longer than about 134 Mb (with such a protein) or a
  * strand other than +1 / -1.  Device memory: the sequences,
- * plus 20 bytes per anchor in groups of at most about 200 M anchors. */
+ * plus 20 bytes per anchor in groups of at most about 200 M anchors.  The
+ * sequences go to the device through at most 256 MB of page-locked memory,
+ * which the context keeps, or without it where that cannot be had. */
 typedef struct {
     int32_t n_anchors;
     int32_t reserved;

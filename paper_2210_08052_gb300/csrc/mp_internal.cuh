@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include "mp_dp.h"
+#include "send_pieces.h"
 
 namespace mpdp {
 
@@ -203,14 +204,11 @@ cudaError_t launch_compact(const PairDesc *pairs, PairOut *out, uint32_t n, cons
 int dp16_blocks_per_sm(int variant, bool wide4 = false);
 int dp16_warps_per_cta(int variant, bool wide4);
 
-// Copy host pieces, one after the other on the device from dst on (piece k at
-// dst + pieces[k].at, `total` bytes in all), on the context's stream: gathered
-// in its pinned staging buffer and sent in runs of about 2 MB as they are
-// gathered.  Returns an MP_* code.
-struct CopyPiece {
-    const char *src;
-    uint64_t at, len;
-};
+// Copy host pieces (see send_pieces.h; `total` bytes in all) to the device from
+// dst on, on the context's stream: gathered in its pinned staging buffer, of
+// which this takes 256 MB at most, and sent in runs of 2 MB as they are
+// gathered; without that much pinned memory, straight from where they are.
+// Returns an MP_* code.
 int ctx_send_pieces(mp_dp_ctx *c, const CopyPiece *pieces, size_t n, uint64_t total, char *dst);
 
 // the device and stream of a context (for the seeding and chaining calls)

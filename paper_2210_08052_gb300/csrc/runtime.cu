@@ -952,51 +952,45 @@ static WorkerPool *gather_pool(mp_dp_ctx *c, uint64_t bytes)
 }
 
 namespace mpdp {
-static constexpr uint64_t kSendWindow = 256ull << 20;
-
 int ctx_send_pieces(mp_dp_ctx *c, const CopyPiece *pieces, size_t n, uint64_t total, char *dst)
 {
-    // in windows of at most kSendWindow bytes (or one longer piece), so that the
-    // pinned buffer stays bounded however many pieces there are
-    for (size_t w0 = 0; w0 < n;) {
-        const uint64_t base = pieces[w0].at;
-        auto end_of = [&](size_t k) { return k + 1 < n ? pieces[k + 1].at : total; };
-        size_t w1 = w0 + 1;
-        while (w1 < n && end_of(w1) - base <= kSendWindow) ++w1;
-        const uint64_t bytes = end_of(w1 - 1) - base;
+    return for_windows(total, kSendWindow, [&](uint64_t w0, uint64_t w1) -> int {
+        const uint64_t bytes = w1 - w0;
         CK(staging_wait(c));
-        if (c->staging.reserve(bytes + 16) != cudaSuccess) return MP_ENOMEM;
+        if (c->staging.reserve(bytes + 16) != cudaSuccess) {
+            // no pinned memory to be had: pageable copies, each piece's part of the
+            // window (the last error is read, so that no launch check meets it)
+            cudaGetLastError();
+            for (size_t k = 0; k < n; ++k) {
+                const uint64_t a = std::max(pieces[k].at, w0), e = std::min(pieces[k].at + pieces[k].len, w1);
+                if (a < e)
+                    CK(cudaMemcpyAsync(dst + a, pieces[k].src + (a - pieces[k].at), e - a, cudaMemcpyHostToDevice,
+                                       c->stream));
+            }
+            return MP_OK;
+        }
         std::atomic<int> copy_err{0};
-        auto send = [&](size_t k0, size_t k1) {
+        auto send = [&](uint64_t lo, uint64_t hi) {
             if (cudaSetDevice(c->device) != cudaSuccess) copy_err = 1;
-            size_t from = k0;
-            uint64_t acc = 0;
-            for (size_t k = k0; k < k1; ++k) {
-                if (pieces[k].len) memcpy(c->staging.p + (pieces[k].at - base), pieces[k].src, pieces[k].len);
-                acc += pieces[k].len;
-                if (acc >= (2u << 20) || k + 1 == k1) {
-                    const uint64_t lo = pieces[from].at, hi = end_of(k);
-                    if (hi > lo && cudaMemcpyAsync(dst + lo, c->staging.p + (lo - base), hi - lo,
-                                                   cudaMemcpyHostToDevice, c->stream) != cudaSuccess)
-                        copy_err = 1;
-                    from = k + 1;
-                    acc = 0;
-                }
+            for (uint64_t a = lo; a < hi;) {
+                const uint64_t e = std::min<uint64_t>(hi, a + (2u << 20));
+                char *h = c->staging.p + (a - w0);
+                gather_range(pieces, n, a, e, h);
+                if (cudaMemcpyAsync(dst + a, h, e - a, cudaMemcpyHostToDevice, c->stream) != cudaSuccess) copy_err = 1;
+                a = e;
             }
         };
         if (WorkerPool *pool = gather_pool(c, bytes)) {
             const unsigned nj = static_cast<unsigned>(pool->th.size());
-            pool->run(nj, [&, nj](unsigned t) { send(w0 + (w1 - w0) * t / nj, w0 + (w1 - w0) * (t + 1) / nj); });
+            pool->run(nj, [&, nj](unsigned t) { send(w0 + bytes * t / nj, w0 + bytes * (t + 1) / nj); });
             pool->wait();
         } else {
             send(w0, w1);
         }
         CK(cudaEventRecord(c->ev_staging, c->stream));
         c->staging_busy = true;
-        if (copy_err) return MP_ECUDA;
-        w0 = w1;
-    }
-    return MP_OK;
+        return copy_err ? MP_ECUDA : MP_OK;
+    });
 }
 }  // namespace mpdp
 
