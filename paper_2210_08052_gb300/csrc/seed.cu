@@ -405,11 +405,13 @@ __global__ void scan_add(uint32_t *out, uint64_t n, const uint32_t *block_sums, 
 
 // Each bucket's entries in ascending order.  A warp takes 32 neighbouring
 // buckets, whose entries are contiguous: in shared memory, each entry's place
-// is the number of its bucket's entries before it (one lane per entry; a
-// bucket holds 10 on average and some hundreds at most on the 50 Mb genome).
+// is the number of its bucket's entries before it (one lane per entry; 32
+// buckets hold 34 on average on the 50 Mb genome, 340 on 500 Mb, where a fifth
+// of them, with 57% of the entries, have more than fit).
 // Where they do not fit, the warp sorts bucket by bucket in place (the network
 // of merge_network.h).  One thread per bucket, by insertion in global memory,
-// took 2.4 ms on the 50 Mb genome; this 0.46.
+// took 2.4 ms on the 50 Mb genome; this 0.46 (the whole index of 50 Mb 6.5 ->
+// 2.8 ms, of 120 Mb 21.5 -> 6.3, of 500 Mb 230 -> 26).
 constexpr int kBucketWarps = 8, kBucketStage = 512;
 
 __global__ void __launch_bounds__(kBucketWarps * 32) bucket_sort_kernel(const uint32_t *off, uint32_t *entries)
@@ -1556,11 +1558,11 @@ extern "C" int mp_chain_refine(mp_dp_ctx *ctx, const mp_pair *pairs, size_t n, m
     uint64_t tot = 0;
     for (size_t k = 0; k < n; ++k) {
         const mp_pair &q = pairs[k];
-        // (a thread's anchor count, at most its bases times the protein's
-        // k-mers, is 32-bit)
+        // (the longest regions that the call takes, as its header says: the anchors
+        // of one pair are chained by one block, each against those within G)
         if ((q.prot_len && !q.prot) || (q.nt_len && !q.nt) || q.prot_len > static_cast<uint32_t>(kRefineMaxProt) ||
             (q.strand != 1 && q.strand != -1) ||
-            (static_cast<uint64_t>(q.nt_len) / kRefineThreads + 1) * q.prot_len >= (1ull << 32))
+            (static_cast<uint64_t>(q.nt_len) / 256 + 1) * q.prot_len >= (1ull << 32))
             return MP_EINVAL;
         poff[k] = tot;
         tot += q.prot_len;
