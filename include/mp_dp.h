@@ -50,7 +50,8 @@ extern "C" {
 #define MP_EAGAIN (-7)    /* mp_dp_submit: request ring full, retry later */
 #define MP_ETICKET (-8)   /* unknown or already-consumed ticket */
 #define MP_ESTATE (-9)    /* call not valid in the context's current state */
-#define MP_ETOOLARGE (-10) /* mp_dp_score_pair_noalloc: input beyond its fixed scratch limits */
+#define MP_ETOOLARGE (-10) /* mp_dp_score_pair_noalloc: input beyond its fixed scratch limits;
+                              mp_index_chain, mp_chain_refine: 2^31 anchors or more */
 
 /* -------------------------------------------------- per-pair status bits */
 #define MP_ST_OK 0x0
@@ -325,7 +326,8 @@ int mp_index_build(mp_dp_ctx *ctx, const char *genome, uint64_t len, mp_index **
 /* Chain n_prot proteins (host ASCII; protein k at prot + prot_off[k],
  * prot_len[k] residues) against the index: chains (caller-owned, n_prot x
  * top) receives up to `top` chains per protein in extraction order,
- * n_chains[k] how many.  Blocking. */
+ * n_chains[k] how many.  Blocking.  MP_ETOOLARGE: a protein with 2^31
+ * anchors or more. */
 int mp_index_chain(mp_dp_ctx *ctx, const mp_index *idx, const char *prot, const uint64_t *prot_off,
                    const uint32_t *prot_len, uint32_t n_prot, int32_t top, mp_chain *chains, uint32_t *n_chains);
 
@@ -356,7 +358,8 @@ void mp_index_free(mp_index *idx);
  * order on ties) and its predecessors; n_anchors 0 if that is a single
  * anchor.  MP_EINVAL: a null argument, a protein longer than 8,192
  * residues, a region longer than about 134 Mb (with such a protein) or a
- * strand other than +1 / -1.  Device memory: the sequences,
+ * strand other than +1 / -1.  MP_ETOOLARGE: a pair with 2^31 anchors or
+ * more.  Device memory: the sequences,
  * plus 20 bytes per anchor in groups of at most about 200 M anchors.  The
  * sequences go to the device through at most 256 MB of page-locked memory,
  * which the context keeps, or without it where that cannot be had. */

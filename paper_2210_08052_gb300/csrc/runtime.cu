@@ -422,7 +422,7 @@ const char *mp_dp_strerror(int code)
     case MP_EAGAIN: return "request ring full";
     case MP_ETICKET: return "unknown ticket";
     case MP_ESTATE: return "invalid state";
-    case MP_ETOOLARGE: return "input exceeds the fixed scratch of the allocation-free entry point";
+    case MP_ETOOLARGE: return "input exceeds a fixed limit (the allocation-free entry point's scratch, or 2^31 anchors)";
     default: return "unknown error";
     }
 }

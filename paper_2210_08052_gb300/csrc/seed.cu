@@ -1325,6 +1325,13 @@ int grid_for(uint64_t threads, int block)
     return static_cast<int>(g < 65535ull * 16 ? (g ? g : 1) : 65535ull * 16);
 }
 
+// whether anchors are numbered in 31 bits throughout (predecessors are 32-bit
+// and signed, and a warp numbers the hits of 32 k-mers in 32 bits)
+bool few_enough(const std::vector<uint64_t> &anchors)
+{
+    return std::all_of(anchors.begin(), anchors.end(), [](uint64_t c) { return c <= INT_MAX; });
+}
+
 // exclusive prefix sums of n counts: out[0..n] (out[n] the total)
 int scan_counts(const uint32_t *in, uint64_t n, uint32_t *out, cudaStream_t st)
 {
@@ -1489,6 +1496,7 @@ extern "C" int mp_index_chain(mp_dp_ctx *ctx, const mp_index *idx, const char *p
     std::vector<uint64_t> cnt(n_prot);
     SCK(cudaMemcpyAsync(cnt.data(), d_cnt.p, n_prot * sizeof(uint64_t), cudaMemcpyDeviceToHost, st));
     SCK(cudaStreamSynchronize(st));
+    if (!few_enough(cnt)) return MP_ETOOLARGE;
     // proteins in groups whose anchors (8 + 8 + 8 + 4 + 1 bytes each) stay within
     // a bound
     constexpr uint64_t kMaxAnchors = 192ull << 20;
@@ -1629,6 +1637,7 @@ extern "C" int mp_chain_refine(mp_dp_ctx *ctx, const mp_pair *pairs, size_t n, m
     std::vector<uint64_t> per(n);
     SCK(cudaMemcpyAsync(per.data(), d_cnt.p, n * sizeof(uint64_t), cudaMemcpyDeviceToHost, st));
     SCK(cudaStreamSynchronize(st));
+    if (!few_enough(per)) return MP_ETOOLARGE;
     // pairs in groups whose anchors (8 + 8 + 4 bytes each) stay within a bound
     constexpr uint64_t kMaxAnchors = 192ull << 20;
     for (size_t p0 = 0; p0 < n;) {
