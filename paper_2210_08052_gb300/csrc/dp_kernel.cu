@@ -4,18 +4,18 @@
 //
 // Layout of the computation
 // -------------------------
-// The protein is cut into strips of 64 residues, one or two of them to a warp
-// (a pair of two strips or more runs two per warp, see Ops16d).  With one,
-// lane l holds residues 2l ("lo") and 2l+1 ("hi") of the strip.  The warp sweeps anti-diagonals: at step t the lo cell of lane l is
-// genome position ii = t - 2l and the hi cell is ii - 1, so every cell
-// depends only on cells of earlier steps:
-//   - the residue to the left (j-1) comes from lane l-1's hi cell of the
-//     previous step (one __shfl_up_sync of a packed [H, I] word), or, for
-//     the hi cell, from the lane's own lo cell of the previous step;
+// The protein is cut into strips of 64 residues, of which a warp runs one or,
+// in the packed int16 form, two (Ops16d; Ops16s and Ops16 run one, see there
+// for where a lane's two residues lie; plan_waves chooses).  The warp sweeps
+// anti-diagonals, each lane some rows behind the lane before it, so that every
+// cell depends only on cells of earlier steps:
+//   - the residue to the left (j-1) comes from the lane before or from the
+//     lane's own cell, both of the previous step;
 //   - genome-direction terms (i-1, i-2, i-3) come from the lane's own
 //     register history.
-// Strip s+1 reads the last residue of strip s from a per-pair boundary
-// buffer ([H, I] per genome position).
+// A warp reads the last residue of the strip before its own from a per-pair
+// boundary buffer ([H, I] per genome position), which the warp of that strip
+// fills as it goes (see RowsIn).
 //
 // Arithmetic
 // ----------
@@ -89,7 +89,8 @@ __host__ __device__ __forceinline__ uint32_t neg2(uint32_t lo, uint32_t hi)
 // function), 64 where it runs two, and the one before in 128-residue strips
 // (records_kernel).
 constexpr int kBackOne = kStripW / 2;
-__device__ __forceinline__ void row_terms(const uint32_t *g, int n, int ii, const ScoreParams &sp, int &d, int &ac, int &aa)
+__device__ __forceinline__ void row_terms(const uint32_t *g, int n, int ii, const ScoreParams &sp, int &d, int &ac,
+                                          int &aa)
 {
     const int s = ii - 3;                  // window T0[ii-3 .. ii+4]
     const int w = s >> 4;                  // floor division (s may be negative)
@@ -237,7 +238,8 @@ struct WarpSmemS {
 };
 
 // 16-byte store to shared memory that leaves the compiler free to move loads of
-// other shared data across it (what is stored here is read after a warp barrier)
+// other shared data across it: it names no memory.  What is stored here is read
+// after a __syncwarp, past which the compiler moves no volatile statement.
 __device__ __forceinline__ void st_shared16(void *smem, uint32_t x, uint32_t y, uint32_t z, uint32_t w)
 {
     const uint32_t sa = static_cast<uint32_t>(__cvta_generic_to_shared(smem));
@@ -246,7 +248,8 @@ __device__ __forceinline__ void st_shared16(void *smem, uint32_t x, uint32_t y, 
 
 // the same to the stream in global memory (a pointer kept in shared memory is
 // not known to be global: as a generic store it would order every shared load
-// behind it)
+// behind it).  Read again, by this warp's search for its best cell and by
+// tracebacks, after the __syncwarp at the chunk's end or later.
 __device__ __forceinline__ void st_stream16(uint8_t *p, uint32_t x, uint32_t y, uint32_t z, uint32_t w)
 {
     asm volatile("st.global.v4.u32 [%0], {%1, %2, %3, %4};" ::"l"(p), "r"(x), "r"(y), "r"(z), "r"(w));
@@ -546,7 +549,6 @@ struct Ops32 {
         return Consts{V2{sp.q + sp.e, sp.q + sp.e}, V2{sp.e, sp.e}, sp.f, sp.mode == MP_MODE_LOCAL ? 0 : NEG, 0, 0};
     }
 
-    static __device__ __forceinline__ V2 pack2(int lo, int hi) { return V2{lo, hi}; }
     static __device__ __forceinline__ void set_row0(Consts &c, int lo, int hi) { c.row0lo = lo; c.row0hi = hi; }
     // profile queries: the gap costs of the lane's two columns
     static __device__ __forceinline__ void set_gaps(Consts &c, int qlo, int elo, int qhi, int ehi, int)
@@ -1066,8 +1068,8 @@ struct Ops16d {
     // pair, which takes both steps' cells into the chunk maximum.
     template <int MASK, bool KEYS, bool SECOND>
     static __device__ __forceinline__ void step(State &s, const Consts &c, const uint2 rec, const uint2 Xl,
-                                                const uint2 Xh, uint32_t inH, uint32_t inI, int lane, int ii, int n, uint32_t &Ha,
-                                                uint32_t &Hb, uint32_t &Ib)
+                                                const uint2 Xh, uint32_t inH, uint32_t inI, int lane, int ii, int n,
+                                                uint32_t &Ha, uint32_t &Hb, uint32_t &Ib)
     {
         const uint32_t Sa = Xl.x + Xh.x;
         uint32_t Da, Db, Ia, Ib0;
@@ -1200,7 +1202,8 @@ struct Ops16d {
         // stream has begun
         constexpr int kFirst = 2 * kStripW, kUpFirst = kUp;
         uint8_t *pl = lo + static_cast<size_t>(t0) * kStepBytes + lane * 16;
-        Cursor q{lane == 0 ? sm.in[0] : sm.zero, sm.out[0], pl, pl + (static_cast<ptrdiff_t>(strip_bytes) - kUp * kStepBytes), (t0 >> 1) - lane, t0};
+        uint8_t *pu = pl + (static_cast<ptrdiff_t>(strip_bytes) - kUp * kStepBytes);
+        Cursor q{lane == 0 ? sm.in[0] : sm.zero, sm.out[0], pl, pu, (t0 >> 1) - lane, t0};
         const int t1 = t0 + steps;
         if (anchored) {
 #pragma unroll 1
@@ -1508,10 +1511,11 @@ struct RowsIn {
 
 // The pair's best cell among a strip's cells that hold `top`, the strip's
 // maximum: the lanes of `who` hold it in half k of their words, whose column
-// is j0 + mul * lane and which are at row 0 in step r + mul * lane.  cmax: the strip's column maxima per chunk of kChunk
-// steps, which start `shift` steps of the strip before multiples of kChunk
-// (the last one's covers every later step).  The whole warp searches: the
-// chunks 32 at a time, then the first such chunk's steps.
+// is j0 + mul * lane and which are at row 0 in step r + mul * lane.  cmax: the
+// strip's column maxima per chunk of kChunk steps, which start `shift` steps of
+// the strip before multiples of kChunk (the last one's covers every later
+// step).  The whole warp searches: the chunks 32 at a time, then the first such
+// chunk's steps.
 __device__ __forceinline__ void best_in_strip(const uint8_t *strip, const uint32_t *cmax, int schunks, int shift,
                                               unsigned who, int k, int mul, int r, int j0, int n, int top, int lane,
                                               Best &best)
@@ -1823,19 +1827,19 @@ __device__ void run_strip(const DPArgs &a, typename Ops::Smem &sm, const PairDes
         }
         __syncwarp();
         if (s + 1 < nstrips && !a.no_publish) {
-          // publish residue W(s+1)-1 for strip s+1
-          if constexpr (kTagged) {
-            for (int k = lane; k < kChunk; k += 32) {
-                const int r = t0 + k - (W - 1);
-                if (r >= 0 && r < n) st_relaxed64(rows + r, static_cast<uint64_t>(item + 1) << 32 | sm.bout[k]);
+            // publish residue W(s+1)-1 for strip s+1
+            if constexpr (kTagged) {
+                for (int k = lane; k < kChunk; k += 32) {
+                    const int r = t0 + k - (W - 1);
+                    if (r >= 0 && r < n) st_relaxed64(rows + r, static_cast<uint64_t>(item + 1) << 32 | sm.bout[k]);
+                }
+            } else {
+                for (int k = lane; k < kChunk; k += 32) bnd[t0 + k - (W - 1)] = sm.bout[k];
+                // __syncwarp orders every lane's stores before lane 0's release
+                // (release is cumulative), so one release store publishes the chunk
+                __syncwarp();
+                if (lane == 0) st_release(mine, static_cast<uint32_t>(ch + 1));
             }
-          } else {
-            for (int k = lane; k < kChunk; k += 32) bnd[t0 + k - (W - 1)] = sm.bout[k];
-            // __syncwarp orders every lane's stores before lane 0's release
-            // (release is cumulative), so one release store publishes the chunk
-            __syncwarp();
-            if (lane == 0) st_release(mine, static_cast<uint32_t>(ch + 1));
-          }
         }
         if (store) colmax[static_cast<size_t>(ch) * 32 + lane] = Ops::chunk_max(st);
         bool folded = false;
@@ -1998,8 +2002,10 @@ __device__ void run_duo(const DPArgs &a, WarpSmemD &sm, const PairDesc &pd, uint
         };
 #pragma unroll 2
         for (int aa = 0; aa < kProfRows; ++aa) {
-            sm.prof[0][aa * 32 + lane] = make_uint2(Ops16::prof_entry(score(aa, 0), 0), Ops16::prof_entry(score(aa, 1), 0));
-            sm.prof[1][aa * 32 + lane] = make_uint2(Ops16::prof_entry(0, score(aa, 2)), Ops16::prof_entry(0, score(aa, 3)));
+            sm.prof[0][aa * 32 + lane] =
+                make_uint2(Ops16::prof_entry(score(aa, 0), 0), Ops16::prof_entry(score(aa, 1), 0));
+            sm.prof[1][aa * 32 + lane] =
+                make_uint2(Ops16::prof_entry(0, score(aa, 2)), Ops16::prof_entry(0, score(aa, 3)));
         }
         for (int k = lane; k < kChunk + kBodyD; k += 32) sm.zero[k] = 0;
     }
@@ -2050,7 +2056,8 @@ __device__ void run_duo(const DPArgs &a, WarpSmemD &sm, const PairDesc &pd, uint
             // the last chunk runs no further than the last valid row
             const int steps = (min(kChunk, it.nsteps - t0) + kBody - 1) / kBody * kBody;
             const int ulimit = it.schunks * kChunk;
-            Ops::chunk<STORE>(st, c, sm, lane, t0, it.n, it.anchored != 0, steps, it.lo, static_cast<size_t>(ulimit) * kStepBytes, ulimit);
+            Ops::chunk<STORE>(st, c, sm, lane, t0, it.n, it.anchored != 0, steps, it.lo,
+                              static_cast<size_t>(ulimit) * kStepBytes, ulimit);
         }
         __syncwarp();
         if (it.publish) {
@@ -2106,9 +2113,8 @@ __device__ void run_duo(const DPArgs &a, WarpSmemD &sm, const PairDesc &pd, uint
 #pragma unroll 1
             for (int k = 0; k < 4; ++k) {
                 const int vk = k == 0 ? v[0] : k == 1 ? v[1] : k == 2 ? v[2] : v[3];
-                best_in_strip(k < 2 ? it.lo : it.lo + strip_bytes, k < 2 ? it.cmax : it.cmax + it.schunks * 32, it.schunks,
-                              (k >> 1) * kUp,
-                              __ballot_sync(kFull, vk == top), k & 1, 2, k & 1,
+                best_in_strip(k < 2 ? it.lo : it.lo + strip_bytes, k < 2 ? it.cmax : it.cmax + it.schunks * 32,
+                              it.schunks, (k >> 1) * kUp, __ballot_sync(kFull, vk == top), k & 1, 2, k & 1,
                               j0 - 2 * lane + (k & 1) + (k >> 1) * kUp, n, top, lane, best);
             }
         }
@@ -2293,7 +2299,8 @@ __host__ __device__ constexpr size_t warp16_bytes(bool wide4)
 // (228 KB, of which each takes 1 KB besides), two at most: what the compiler
 // may count on when it shares out the registers.
 template <typename Ops, int Warps, bool Wide4>
-constexpr size_t kCtaBytes = Warps * (sizeof(typename Ops::Bnd) == 4 ? warp16_bytes(Wide4) : sizeof(typename Ops::Smem));
+constexpr size_t kCtaBytes =
+    Warps * (sizeof(typename Ops::Bnd) == 4 ? warp16_bytes(Wide4) : sizeof(typename Ops::Smem));
 template <typename Ops, int Warps, bool Wide4>
 constexpr int kCtasPerSm = 2 * (kCtaBytes<Ops, Warps, Wide4> + 1024) <= 228 * 1024 ? 2 : 1;
 
@@ -2350,8 +2357,9 @@ __global__ void __launch_bounds__(Warps * 32, (kCtasPerSm<Ops, Warps, Wide4>)) d
         }
         if constexpr (kInt16) {
             WarpSmemS &sms = *reinterpret_cast<WarpSmemS *>(mine);
-            if (pd.flags & PF_SCORE_ONLY) run_solo<false>(a, sms, pd, it.x, static_cast<int>(it.y), lane, rerun_only != 0);
-            else run_solo<true>(a, sms, pd, it.x, static_cast<int>(it.y), lane, rerun_only != 0);
+            const int s = static_cast<int>(it.y);
+            if (pd.flags & PF_SCORE_ONLY) run_solo<false>(a, sms, pd, it.x, s, lane, rerun_only != 0);
+            else run_solo<true>(a, sms, pd, it.x, s, lane, rerun_only != 0);
         } else {
             run_strip<Ops>(a, *reinterpret_cast<SM *>(mine), pd, it.x, static_cast<int>(it.y), it.y, pd.n_strips, lane,
                            rerun_only != 0);

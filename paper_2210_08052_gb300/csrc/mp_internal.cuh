@@ -74,7 +74,8 @@ constexpr int32_t kStTraced = 0x200;
 // PF_DUO: a warp runs two neighbouring 64-residue strips of the pair at once
 // (int16 only, never with PF_WIDE or PF_W128)
 enum : uint32_t {
-    PF_SCORE_ONLY = 1u, PF_BADSEQ = 2u, PF_SKIP = 4u, PF_BUDGET = 8u, PF_WIDE = 16u, PF_W128 = 32u, PF_PROF = 64u, PF_DUO = 128u
+    PF_SCORE_ONLY = 1u, PF_BADSEQ = 2u, PF_SKIP = 4u, PF_BUDGET = 8u, PF_WIDE = 16u, PF_W128 = 32u, PF_PROF = 64u,
+    PF_DUO = 128u
 };
 
 // Device copy of mp_profile_pos: position-specific substitution scores

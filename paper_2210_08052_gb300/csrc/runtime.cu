@@ -422,7 +422,8 @@ const char *mp_dp_strerror(int code)
     case MP_EAGAIN: return "request ring full";
     case MP_ETICKET: return "unknown ticket";
     case MP_ESTATE: return "invalid state";
-    case MP_ETOOLARGE: return "input exceeds a fixed limit (the allocation-free entry point's scratch, or 2^31 anchors)";
+    case MP_ETOOLARGE:
+        return "input exceeds a fixed limit (the allocation-free entry point's scratch, or 2^31 anchors)";
     default: return "unknown error";
     }
 }
@@ -640,9 +641,10 @@ static uint64_t plan_code_bytes(const mp_dp_ctx *c, const mp_dp_batch *b)
 // predecessor has not yet published the boundary rows it starts with: pairs
 // in order (largest first), strip s+1 of a pair placed after strip s by
 // about as many items as the warps pop while the predecessor runs the chunks
-// it is ahead by (2, or 3 where a warp runs two strips; the strips of a pair still run close together, so its per-nt
-// records and boundary rows are read from L2).  PF_WIDE pairs' items stay a
-// prefix of the wave (the int32 queue may take them as a block).
+// it is ahead by (2, or 3 where a warp runs two strips; the strips of a pair
+// still run close together, so its per-nt records and boundary rows are read
+// from L2).  PF_WIDE pairs' items stay a prefix of the wave (the int32 queue may
+// take them as a block).
 static void interleave_items(const mp_dp_ctx *c, mp_dp_batch *b)
 {
     const double warps = static_cast<double>(c->num_sms) * 2 * kWarps16;
@@ -651,11 +653,11 @@ static void interleave_items(const mp_dp_ctx *c, mp_dp_batch *b)
     auto segment = [&](uint32_t lo, uint32_t hi) {
         if (hi - lo < 2) return;
         double chunks = 0, lag = 0;
-        for (uint32_t k = lo; k < hi; ++k)
-        {
+        for (uint32_t k = lo; k < hi; ++k) {
             const PairDesc &d = b->desc[b->h_items[k].x];
             const bool duo = (d.flags & PF_DUO) != 0;
-            chunks += static_cast<double>((d.nt_len + (duo ? 2 * kStripW : strip_w_of(d.flags)) - 1 + kChunk - 1) / kChunk);
+            const int width = duo ? 2 * kStripW : strip_w_of(d.flags);
+            chunks += static_cast<double>((d.nt_len + width - 1 + kChunk - 1) / kChunk);
             lag += duo ? 3.0 : 2.0;
         }
         const uint32_t D = static_cast<uint32_t>(std::max(1.0, std::round(warps * lag / chunks)));
@@ -928,8 +930,6 @@ static int plan_waves(mp_dp_ctx *c, mp_dp_batch *b, const mp_dp_tuning &t, bool 
     return MP_OK;
 }
 
-// (Re)fill batch b with n pairs: plan strips, waves and offsets on the host,
-// grow the device buffers when needed, and copy the inputs to the device.
 // Wait until the last copy out of the staging buffer has left it.
 static cudaError_t staging_wait(mp_dp_ctx *c)
 {
@@ -996,9 +996,6 @@ int ctx_send_pieces(mp_dp_ctx *c, const CopyPiece *pieces, size_t n, uint64_t to
 
 extern "C" {
 
-// ascii_on_device: the caller writes the batch's ASCII into b->ascii on the
-// context's stream itself (the pairs' nt pointers are unused and may be null;
-// the protein pointers still serve the score bound).
 // A profile query's positions are within range and keep the degenerate
 // intron paths losing (r above every negated score, as mp_dp_init requires
 // of the matrix).
@@ -1027,6 +1024,11 @@ static int64_t profile_score_bound(const mp_profile_pos *pf, uint32_t m)
     return s;
 }
 
+// (Re)fill batch b with n pairs: plan strips, waves and offsets on the host,
+// grow the device buffers when needed, and copy the inputs to the device.
+// ascii_on_device: the caller writes the batch's ASCII into b->ascii on the
+// context's stream itself (the pairs' nt pointers are unused and may be null;
+// the protein pointers still serve the score bound).
 static int upload_impl(mp_dp_ctx *c, mp_dp_batch *b, const mp_pair *pairs, size_t n, bool ascii_on_device = false)
 {
     for (size_t k = 0; k < n; ++k) {

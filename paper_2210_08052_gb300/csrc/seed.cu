@@ -17,8 +17,8 @@
 //   scan kernels       exclusive prefix sums (bucket counts -> CSR offsets)
 //   bucket_sort_kernel each bucket's entries in ascending order
 //
-// Chaining, per protein (one warp each): its k-mers' hits as anchors
-// (strand, x = bin, y = residue), sorted; the recurrence of Eq. 2 with the
+// Chaining, per protein (a block each, four warps to a strand): its k-mers'
+// hits as anchors (strand, x = bin, y = residue), sorted; the recurrence of Eq. 2 with the
 // gap of Eq. 1 and the penalty of Eq. 3 (G = 200,000, beta = 0.75) in fixed
 // point with 16 fractional bits (the log term from a table of every |g| < G),
 // 32 anchors at a time, one per lane (see chain_dp); then the chains in order
@@ -26,10 +26,10 @@
 //
 // Second round, per (protein, region) pair: every 5-mer of the protein
 // (reduced alphabet, sorted in shared memory) against the 5-mer starting at
-// every base of the region's aligned strand by binary search (one block per
-// pair, contiguous base ranges per thread, so the anchors come out in (x, y)
-// order), counted then written; chained by one warp per pair with
-// g' = 3 dy - dx and Eq. 3.
+// every base of the region's aligned strand, by a filter and a binary search
+// (one block per pair, the region in tiles, contiguous bases per thread, so the
+// anchors come out in (x, y) order), counted then written; chained by one warp
+// per pair, or eight, with g' = 3 dy - dx and Eq. 3.
 #include <algorithm>
 #include <climits>
 #include <cstdint>
@@ -277,7 +277,8 @@ __global__ void __launch_bounds__(kKmerWarps * 32) kmer_kernel(Frames fr, const 
         const uint64_t t0 = (s - fr.seg0[f]) * kSeg, len = fr.len[f];
         const uint8_t *code = fr.code[f] + t0;
         const int cnt = static_cast<int>(len - t0 < kSeg ? len - t0 : kSeg);               // codons of the segment
-        const int more = static_cast<int>(len - t0 < kSeg + kK - 1 ? len - t0 : kSeg + kK - 1);   // and what its k-mers touch
+        // and what its k-mers touch
+        const int more = static_cast<int>(len - t0 < kSeg + kK - 1 ? len - t0 : kSeg + kK - 1);
         __syncwarp();
         if (cnt == kSeg) {
             // (the frames' arrays start on 16 bytes and a segment is a multiple of them)
@@ -793,13 +794,15 @@ struct Seeker {
         const T lin = static_cast<T>(sizeof(T) == 4 ? min(a, kClamp32) : a) * 21845;        // 65536 = 3 * 21845 + 1
         const T low = g < 0 ? (lin < static_cast<T>(l2) ? lin : static_cast<T>(l2)) : lin + static_cast<T>(l2);
         // (32 bits: f is positive and the rest above -2^31)
-        return a < static_cast<int32_t>(kG) && f + (static_cast<T>(min(dy, Geo::K)) * static_cast<T>(kScale) - low) > best;
+        return a < static_cast<int32_t>(kG) &&
+               f + (static_cast<T>(min(dy, Geo::K)) * static_cast<T>(kScale) - low) > best;
     }
     __device__ __forceinline__ void try_link(uint32_t x, int32_t y, T f, int32_t i, const int32_t *lt)
     {
         int32_t g, dy;
         if (may(x, y, f, g, dy) && may_win(f, g, dy)) {
-            const int64_t c = static_cast<int64_t>(f) + static_cast<int64_t>(min(dy, Geo::K)) * kScale - penalty_eq3(g, lt);
+            const int64_t c =
+                static_cast<int64_t>(f) + static_cast<int64_t>(min(dy, Geo::K)) * kScale - penalty_eq3(g, lt);
             if (c > static_cast<int64_t>(best)) {
                 best = static_cast<T>(c);
                 arg = i;
@@ -927,6 +930,9 @@ __device__ void chain_dp(const uint64_t *A, int64_t n, const Geo &geo, const int
     }
 }
 
+// where a protein's tiles start in ChainArgs::tmax
+__device__ __forceinline__ uint64_t tile_base(uint64_t b0, uint32_t p) { return b0 / 32 + 2ull * p; }
+
 // One block per protein, the ones with most anchors first: Eq. 2 over its
 // sorted anchors, kStrandWarps warps per strand (chains stay on one; the
 // longest protein's tiles are a chain of their own), then its chains.
@@ -941,8 +947,6 @@ __device__ void chain_dp(const uint64_t *A, int64_t n, const Geo &geo, const int
 // follow it at a loss, and with a look at every anchor before each of them one
 // protein of 4,000 took 20 ms.  The best is found from the largest f of each
 // tile; a tile whose largest is out of date is seen when it is looked at.
-__device__ __forceinline__ uint64_t tile_base(uint64_t b0, uint32_t p) { return b0 / 32 + 2ull * p; }    // in ChainArgs::tmax
-
 constexpr int kStrandWarps = 4;
 __global__ void __launch_bounds__(kStrandWarps * 64) chain_kernel(ChainArgs a)
 {
@@ -1270,7 +1274,8 @@ __global__ void __launch_bounds__(kRefineWarps * 32) refine_chain_kernel(RefineA
     __shared__ ChainSmem<1> sm[kRefineWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (uint32_t p = blockIdx.x * kRefineWarps + warp; p < a.n; p += gridDim.x * kRefineWarps)
-        if (static_cast<int64_t>(a.anc_off[p + 1] - a.anc_off[p]) <= kRefineBig) refine_pair<1>(a, p, sm[warp], 0, lane);
+        if (static_cast<int64_t>(a.anc_off[p + 1] - a.anc_off[p]) <= kRefineBig)
+            refine_pair<1>(a, p, sm[warp], 0, lane);
 }
 
 // One block per pair with more than kRefineBig anchors: every earlier anchor

@@ -58,6 +58,7 @@ int main()
 def test_windows_and_ranges(tmp_path):
     src, exe = tmp_path / "pieces.cpp", tmp_path / "pieces"
     src.write_text(SOURCE)
-    subprocess.run(["g++", "-std=c++17", "-O1", "-fsanitize=address", "-I" + CSRC, str(src), "-o", str(exe)], check=True)
+    subprocess.run(["g++", "-std=c++17", "-O1", "-fsanitize=address", "-I" + CSRC, str(src), "-o", str(exe)],
+                   check=True)
     r = subprocess.run([str(exe)], capture_output=True, text=True, timeout=120)
     assert r.returncode == 0, r.stdout + r.stderr
