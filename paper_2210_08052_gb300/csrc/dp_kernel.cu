@@ -1488,10 +1488,10 @@ struct RowsIn {
             v[q] = r < n ? ld_relaxed64(rows + r) : static_cast<uint64_t>(tag) << 32 | kPast;
         }
     }
-    // polls that sleep less: rows come in every few microseconds while the warp
-    // before computes.  Later ones sleep as long as the int32 kernel's, so that a
-    // poll limit bounds both kernels' waits alike (0.26 and 0.51 us a poll)
-    static constexpr uint32_t kQuick = 64;
+    // polls that last as long as `limit` of the int32 kernel's: they sleep for 100
+    // ns instead of 256 and take half as long in all (0.257 and 0.513 us), so that
+    // a poll limit bounds both kernels' waits alike
+    static __device__ __forceinline__ uint32_t polls(uint32_t limit) { return 2 * min(limit, 0x7fffffffu); }
     // wait (bounded) until every row queued has arrived; false: it ran out
     __device__ __forceinline__ bool settle(const uint64_t *rows, int row, uint32_t tag, int lane, uint32_t limit)
     {
@@ -1501,7 +1501,7 @@ struct RowsIn {
             for (int q = 0; q < kChunk / 32; ++q) ok = ok && static_cast<uint32_t>(v[q] >> 32) == tag;
             if (__all_sync(kFull, ok)) return true;
             if (it >= limit) return false;
-            __nanosleep(it < kQuick ? 100 : 256);
+            __nanosleep(100);
 #pragma unroll
             for (int q = 0; q < kChunk / 32; ++q)
                 if (static_cast<uint32_t>(v[q] >> 32) != tag) v[q] = ld_relaxed64(rows + row + lane + 32 * q);
@@ -1687,7 +1687,8 @@ __device__ void run_strip(const DPArgs &a, typename Ops::Smem &sm, const PairDes
     bool timed_out = false;
 
     // wait until strip s-1 has published `need` chunks (bounded)
-    const uint32_t spin_limit = a.spin_limit ? a.spin_limit : kSpinLimit;
+    const uint32_t spin_limit0 = a.spin_limit ? a.spin_limit : kSpinLimit;
+    const uint32_t spin_limit = kTagged ? RowsIn::polls(spin_limit0) : spin_limit0;
     auto wait_for = [&](uint32_t need) {
         if (kTagged || s == 0 || timed_out) return;
         uint32_t ok = 1;
@@ -1960,7 +1961,7 @@ __device__ void run_duo(const DPArgs &a, WarpSmemD &sm, const PairDesc &pd, uint
     // row of a cell at step t: t - 2l - k (lower strip), t - 2l - k - 64 (upper)
     constexpr int kLast = 2 * kStripW - 1;
     const uint4 *recs = a.recs + pd.rec_off;            // recs[ii + kRecPre] is position ii
-    const uint32_t limit = a.spin_limit ? a.spin_limit : kSpinLimit;
+    const uint32_t limit = RowsIn::polls(a.spin_limit ? a.spin_limit : kSpinLimit);
     bool timed_out = false;
     if (lane == 0) {
         const int schunks = (n + kStripW - 1 + kChunk - 1) / kChunk;    // chunks of a strip's stream
@@ -2157,7 +2158,7 @@ __device__ void run_solo(const DPArgs &a, WarpSmemS &sm, const PairDesc &pd, uin
         asm volatile("mov.u32 %0, %1;" : "=r"(c.mult) : "r"(lane == 0 ? 65536u : 1u));
     }
     const uint4 *recs = a.recs + pd.rec_off;            // recs[ii + kRecPre] is position ii
-    const uint32_t limit = a.spin_limit ? a.spin_limit : kSpinLimit;
+    const uint32_t limit = RowsIn::polls(a.spin_limit ? a.spin_limit : kSpinLimit);
     const uint32_t item = static_cast<uint32_t>(s);
     bool timed_out = false;
     if (lane == 0) {

@@ -130,8 +130,8 @@ def test_each_form_of_profile_queries(mp, orc, mode, duo):
 def test_poll_limit_bounds_both_kernels_waits_alike(mp):
     """With boundary rows withheld, a pair of three strips waits out its poll
     limit, at most a fifth of a second, and is marked.  The int16 wait lasts as
-    long as the int32 kernel's under the same limit: its first 64 polls of 40,000
-    sleep less, and a poll's load may take a little less (5 per cent)."""
+    long as the int32 kernel's under the same limit (less 5 per cent: a poll's load
+    may take a little less)."""
     rng = np.random.default_rng(270)
     pair = synth.Pair(synth.random_protein(rng, 192), synth.random_dna(rng, 300), 1)
     ms = []
