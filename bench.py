@@ -468,8 +468,9 @@ def with_ceilings(roof, mp, m, cells, torch, device):
         "unit": "warp instructions per clock per SM (each operation alone); cells per clock per SM (step)",
         "step_ceiling_gcups": step_cells_s / 1e9,
         "frac_of_step_ceiling": (cells / (dp_ms / 1000) / step_cells_s) if dp_ms else None,
-        "basis": "SM clocks counted in the kernels; the step ceiling is the int16 step's arithmetic on "
-                 "register state at full occupancy, without records, profile loads, stream stores or waits",
+        "basis": "SM clocks counted in the kernels; the step ceiling is the arithmetic of an int16 step of "
+                 "one strip in neighbouring columns on register state at full occupancy, without records, "
+                 "profile loads, stream stores or waits (two strips per warp take fewer instructions per cell)",
     }
     return roof
 

@@ -490,10 +490,12 @@ int mp_dp_num_sms(mp_dp_ctx *ctx);
  *     16-bit operation alone (max, fused add-max, three-way max, byte
  *     permute, three-input logic, integer multiply-add), eight independent
  *     chains per thread, one plain add per eight operations;
- *   - step_cells_per_clk_sm: cells per clock per SM of the int16 step's
- *     arithmetic alone (the eleven fused add-max terms of Eq. 7, the
- *     three-way maxima, the [H, I] hand-over by shuffle and byte permute,
- *     the chunk maximum) on register state, warps_per_sm_step warps per SM.
+ *   - step_cells_per_clk_sm: cells per clock per SM of the arithmetic alone
+ *     of an int16 step of one strip, two neighbouring residues per lane (the
+ *     eleven fused add-max terms of Eq. 7, the three-way maxima, the [H, I]
+ *     hand-over by shuffle and byte permute, the chunk maximum) on register
+ *     state, warps_per_sm_step warps per SM.  The DP kernel's own form of two
+ *     strips per warp takes fewer instructions per cell than this step.
  * The call allocates a few MB on `device` and runs for well under a second;
  * it needs no context.  MP_EINVAL: null out or no such device; MP_ENOMEM,
  * MP_ECUDA as usual. */

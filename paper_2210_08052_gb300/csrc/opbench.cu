@@ -9,11 +9,14 @@
 //   - the throughput of each packed 16-bit operation alone (warp
 //     instructions per clock per SM, eight independent chains per thread,
 //     every warp slot of every SM occupied);
-//   - the throughput of the step's arithmetic itself: Eq. 7's eleven
-//     penalised terms as fused add-max, the three-way maxima, the [H, I]
-//     hand-over to the next lane by shuffle and byte permute, the chunk
-//     maximum, on register state only (no shared-memory records, no stream
-//     stores), at full occupancy.  Reported as cells per clock per SM.
+//   - the throughput of a step's arithmetic itself, of one strip with two
+//     neighbouring residues per lane: Eq. 7's eleven penalised terms as fused
+//     add-max, the three-way maxima, the [H, I] hand-over to the next lane by
+//     shuffle and byte permute, the chunk maximum, on register state only (no
+//     shared-memory records, no stream stores), at full occupancy.  Reported
+//     as cells per clock per SM; a fixed yardstick: the kernel's form of two
+//     strips per warp (Ops16d) has no byte permute in its hand-over and takes
+//     fewer instructions per cell.
 //
 // Clocks are counted on the SM (clock64) over each block's run, so the
 // rates do not depend on the clock the GPU chose.
